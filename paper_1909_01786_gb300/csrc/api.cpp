@@ -19,6 +19,10 @@ cudaError_t solve_attributes(cudaFuncAttributes *a);
 cudaError_t launch_sweep(const Dev &D, Acc *acc, int grid, int block, size_t smem, cudaStream_t st,
                          uint32_t passes);
 int batch_threads(int config);
+cudaError_t launch_reset(const Dev &D, bool codes, cudaStream_t st);
+uint32_t input_blocks(const Dev &D);
+cudaError_t launch_input(const Dev &D, const int8_t *partial, uint32_t *counts, cudaStream_t st);
+cudaError_t launch_closure(const Dev &D, int8_t *closure, cudaStream_t st);
 int mlp_prior(const uint16_t *d_w, const std::vector<float> &features, int64_t n, float *d_out, cudaStream_t st);
 cudaError_t batch_configure(int config, bool units, size_t smem, int *blocks_per_sm);
 cudaError_t launch_batch(int config, bool units, const Dev *devs, const uint32_t *order, uint32_t n, unsigned int *queue, int grid,
@@ -74,6 +78,9 @@ struct asp_prog {
     unsigned long long *d_models = nullptr;
     int64_t d_models_rows = 0;
     Acc *d_sweep_acc = nullptr;
+    // asp_debug_propagate, allocated by its first call: the input's and the
+    // closure's bytes (8 x asg_words), then the counts of launch_input
+    int8_t *d_io = nullptr;
 };
 
 namespace aspgpu {
@@ -761,38 +768,12 @@ void asp_free(asp_prog *p)
 
 }  // extern "C"
 
-// Reset the search state on the stream and set the first control block.
-static int reset_state(asp_prog *p, uint32_t mode, int64_t max_models, int64_t models_cap,
-                       unsigned long long *d_models, long long *d_result,
-                       uint32_t n_input)
+// The launch arguments that a call chooses (the state itself is reset on the
+// device: launch_reset, launch_input).
+static void set_launch(asp_prog *p, uint32_t mode, int64_t max_models, int64_t models_cap,
+                       unsigned long long *d_models, long long *d_result)
 {
     Dev &D = p->D;
-    cudaStream_t st = p->stream;
-    cudaError_t e = cudaSuccess;
-    if (mode == MODE_SOLVE) {
-        e = cudaMemsetAsync(D.asg, 0, (size_t)D.asg_words * 4 + 4, st);
-        if (e == cudaSuccess) e = cudaMemsetAsync(D.dl, 0, (size_t)D.nv * 4 + 4, st);
-    }
-    if (e == cudaSuccess) e = cudaMemsetAsync(D.act, 0, (size_t)D.J * 4 + 8, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(D.stats, 0, sizeof(DevStats), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(D.bar, 0, sizeof(Barrier), st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(D.level_start, 0, ((size_t)D.J + 4) * 4, st);
-    if (e == cudaSuccess && D.dirty) e = cudaMemsetAsync(D.dirty, 0, (size_t)D.dirty_words * 2 * 4, st);
-    static thread_local Ctl ctl[2];
-    static thread_local Acc acc[4];
-    std::memset(ctl, 0, sizeof(ctl));
-    ctl[0].op = OP_INIT;
-    ctl[0].cdl = 1;
-    ctl[0].tc = n_input;
-    ctl[0].tb = n_input;
-    ctl[0].lfill = D.lits_static;
-    for (int i = 0; i < 4; i++) {
-        acc[i].ckey = NO_KEY; acc[i].cslot[0] = acc[i].cslot[1] = acc[i].cslot[2] = NO_KEY; acc[i].dkey = 0; acc[i].nclaim = 0; acc[i].flag = 0;
-        acc[i].minU = 0xFFFFFFFFu; acc[i].nlits = 0; acc[i].checks = 0; acc[i].visits = 0; acc[i].tbusy = 0; acc[i].tsweep = 0; acc[i].tlong = 0; acc[i].tbuck = 0;
-    }
-    if (e == cudaSuccess) e = cudaMemcpyAsync(D.ctl, ctl, sizeof(ctl), cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(D.acc, acc, sizeof(acc), cudaMemcpyHostToDevice, st);
-    if (e != cudaSuccess) return cuda_fail(e, "reset");
     D.mode = mode;
     D.max_models = max_models;
     D.models_cap = models_cap;
@@ -800,7 +781,6 @@ static int reset_state(asp_prog *p, uint32_t mode, int64_t max_models, int64_t m
     D.result = d_result;
     D.conflict_budget = p->opt.conflict_budget;
     D.time_budget_ns = p->opt.time_budget_ms > 0 ? p->opt.time_budget_ms * 1000000ll : 0;
-    return ASP_OK;
 }
 
 static void fill_stats(const asp_prog *p, const DevStats &s, asp_stats_t &o)
@@ -837,20 +817,21 @@ int asp_solve_async(asp_prog *p, int64_t max_models, uint64_t *d_models, int64_t
         cudaError_t e = cudaMemcpyAsync(d_result, r, sizeof(r), cudaMemcpyHostToDevice, p->stream);
         return e == cudaSuccess ? ASP_OK : cuda_fail(e, "result");
     }
-    int rc = reset_state(p, MODE_SOLVE, max_models, models_cap, (unsigned long long *)d_models,
-                         (long long *)d_result, 0);
-    if (rc != ASP_OK) return rc;
-    cudaError_t e = launch_solve(p->D, p->grid, p->block, p->smem, p->stream);
+    set_launch(p, MODE_SOLVE, max_models, models_cap, (unsigned long long *)d_models, (long long *)d_result);
+    cudaError_t e = launch_reset(p->D, true, p->stream);
+    if (e != cudaSuccess) return cuda_fail(e, "reset");
+    e = launch_solve(p->D, p->grid, p->block, p->smem, p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "launch");
     return ASP_OK;
 }
 
 static int finish(asp_prog *p, long long *res)
 {
-    cudaError_t e = p->stream ? cudaStreamSynchronize(p->stream) : cudaDeviceSynchronize();
-    if (e != cudaSuccess) return cuda_fail(e, "solve");
-    e = cudaMemcpy(res, p->d_result, sizeof(long long) * 4, cudaMemcpyDeviceToHost);
+    // one wait for the solve and the copy of its result (two cost 8 us more)
+    cudaError_t e = cudaMemcpyAsync(res, p->d_result, sizeof(long long) * 4, cudaMemcpyDeviceToHost, p->stream);
     if (e != cudaSuccess) return cuda_fail(e, "result");
+    e = p->stream ? cudaStreamSynchronize(p->stream) : cudaDeviceSynchronize();
+    if (e != cudaSuccess) return cuda_fail(e, "solve");
     return ASP_OK;
 }
 
@@ -910,39 +891,35 @@ int asp_debug_propagate(asp_prog *p, const int8_t *partial, int8_t *closure, int
     g_err.clear();
     if (!p || !partial || !closure) return fail(ASP_E_ARG, "bad argument");
     const Dev &D = p->D;
-    std::vector<uint32_t> asg(D.asg_words + 1, 0u), trail;
-    std::vector<int32_t> dl(D.nv + 1, 0);
-    std::vector<uint32_t> reason(D.nv + 1, R_INPUT);
-    for (uint32_t v = 0; v < D.nv; v++) {
-        if (partial[v] == 0) continue;
-        uint32_t code = partial[v] > 0 ? V_T : V_F;
-        asg[v >> 3] |= code << ((v & 7u) * 4u);
-        trail.push_back(v | (code == V_F ? TRAIL_F : 0u));
-        dl[v] = 1;
+    const size_t io = (size_t)D.asg_words * 8;
+    if (!p->d_io) {
+        p->d_io = (int8_t *)dalloc(p, io + 4 * (size_t)input_blocks(D));
+        if (!p->d_io) return fail(ASP_E_OOM, "device allocation failed (partial assignment)");
     }
+    // codes, levels, reasons and trail are made on the device from one byte a
+    // variable (for 5.2M variables, 16 ms of host loops and 47 MB of copies
+    // were two thirds of the call)
     cudaStream_t st = p->stream;
-    cudaError_t e = cudaMemcpyAsync(p->D.asg, asg.data(), asg.size() * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(p->D.dl, dl.data(), (size_t)D.nv * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(p->D.reason, reason.data(), (size_t)D.nv * 4, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess && !trail.empty())
-        e = cudaMemcpyAsync(p->D.trail, trail.data(), trail.size() * 4, cudaMemcpyHostToDevice, st);
+    set_launch(p, MODE_PROPAGATE, 0, 0, nullptr, p->d_result);
+    cudaError_t e = cudaMemcpyAsync(p->d_io, partial, D.nv, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_input(D, p->d_io, reinterpret_cast<uint32_t *>(p->d_io + io), st);
     if (e != cudaSuccess) return cuda_fail(e, "upload partial");
-    int rc = reset_state(p, MODE_PROPAGATE, 0, 0, nullptr, p->d_result, (uint32_t)trail.size());
-    if (rc != ASP_OK) return rc;
     long long res[4] = {0, 0, 0, 0};
     if (p->empty_nogood) {
         res[3] = 1;
     } else {
         e = launch_solve(p->D, p->grid, p->block, p->smem, st);
         if (e != cudaSuccess) return cuda_fail(e, "launch");
-        rc = finish(p, res);
-        if (rc != ASP_OK) return rc;
     }
-    e = cudaMemcpy(asg.data(), p->D.asg, (size_t)D.asg_words * 4, cudaMemcpyDeviceToHost);
+    e = launch_closure(D, p->d_io, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(closure, p->d_io, D.nv, cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_fail(e, "download closure");
-    for (uint32_t v = 0; v < D.nv; v++) {
-        uint32_t c = (asg[v >> 3] >> ((v & 7u) * 4u)) & 3u;
-        closure[v] = c == V_T ? 1 : c == V_F ? -1 : c == 3u ? 2 : 0;
+    if (!p->empty_nogood) {
+        const int rc = finish(p, res);
+        if (rc != ASP_OK) return rc;
+    } else {
+        e = st ? cudaStreamSynchronize(st) : cudaDeviceSynchronize();
+        if (e != cudaSuccess) return cuda_fail(e, "download closure");
     }
     if (conflict) *conflict = (int32_t)res[3];
     if (res[2] != 0) return fail(ASP_E_DEVICE, "device-side error");

@@ -1,0 +1,157 @@
+// Search state around a launch: the reset before a solve, and the exchange of
+// a partial assignment and its closure for asp_debug_propagate.
+#include <cuda_runtime.h>
+
+#include <algorithm>
+#include <cstdint>
+
+#include "device.cuh"
+
+namespace aspgpu {
+
+namespace {
+
+__device__ __forceinline__ void first_control(const Dev &D, uint32_t n_input)
+{
+    Ctl c{};
+    D.ctl[1] = c;
+    c.op = OP_INIT;
+    c.cdl = 1u;
+    c.tc = c.tb = n_input;
+    c.lfill = D.lits_static;
+    D.ctl[0] = c;
+    Acc a{};
+    a.ckey = a.cslot[0] = a.cslot[1] = a.cslot[2] = NO_KEY;
+    a.minU = 0xFFFFFFFFu;
+    for (int i = 0; i < 4; i++) D.acc[i] = a;
+    *D.stats = DevStats{};
+    *D.bar = Barrier{};
+}
+
+// Clears what a search starts from and writes the first control block: one
+// launch where nine memsets and copies stood (about 1 us each on the stream).
+// codes: the assignment and levels too (a propagation sets them from its
+// input).
+__global__ void __launch_bounds__(256) reset_kernel(Dev D, bool codes, uint32_t n_input)
+{
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x, nt = gridDim.x * blockDim.x;
+    if (codes) {
+        for (uint32_t w = t; w <= D.asg_words; w += nt) D.asg[w] = 0u;
+        for (uint32_t v = t; v <= D.nv; v += nt) D.dl[v] = 0;
+    }
+    for (uint32_t j = t; j < D.J + 2u; j += nt) D.act[j] = 0u;
+    for (uint32_t j = t; j < D.J + 4u; j += nt) D.level_start[j] = 0u;
+    if (D.dirty)
+        for (uint32_t w = t; w < 2u * D.dirty_words; w += nt) D.dirty[w] = 0u;
+    if (t == 0) first_control(D, n_input);
+}
+
+// variables of one block of the input kernels: 256 threads x 32
+constexpr uint32_t IN_VARS = 8192;
+
+// The codes (8 per word), levels and reasons of the input, and the number of
+// assigned variables of each block of IN_VARS.
+__global__ void __launch_bounds__(256) input_codes_kernel(Dev D, const int8_t *partial, uint32_t *counts)
+{
+    __shared__ uint32_t s_n;
+    if (threadIdx.x == 0) s_n = 0u;
+    __syncthreads();
+    uint32_t n = 0;
+    const uint32_t w0 = blockIdx.x * (IN_VARS / 8u);
+    for (uint32_t w = w0 + threadIdx.x; w < min(w0 + IN_VARS / 8u, D.asg_words); w += blockDim.x) {
+        uint32_t m = 0;
+        for (uint32_t q = 0; q < 8u; q++) {
+            const uint32_t v = 8u * w + q;
+            const int8_t x = v < D.nv ? partial[v] : (int8_t)0;
+            if (x) { m |= (x > 0 ? V_T : V_F) << (4u * q); n++; }
+        }
+        D.asg[w] = m;
+    }
+    const uint32_t v0 = blockIdx.x * IN_VARS;
+    for (uint32_t v = v0 + threadIdx.x; v < min(v0 + IN_VARS, D.nv); v += blockDim.x) {
+        D.dl[v] = partial[v] ? 1 : 0;
+        D.reason[v] = R_INPUT;
+    }
+    if (blockIdx.x == 0 && threadIdx.x == 0) D.asg[D.asg_words] = 0u;
+    if (n) atomicAdd(&s_n, n);
+    __syncthreads();
+    if (threadIdx.x == 0) counts[blockIdx.x] = s_n;
+}
+
+// The input's variables on the trail in ascending order: a block starts after
+// the counts of the blocks before it, and a warp after those of its block.
+// The last block writes the first control block.
+__global__ void __launch_bounds__(256) input_trail_kernel(Dev D, const int8_t *partial, const uint32_t *counts)
+{
+    __shared__ uint32_t s_base, s_warp[8];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    if (threadIdx.x == 0) s_base = 0u;
+    __syncthreads();
+    uint32_t before = 0;
+    for (uint32_t b = threadIdx.x; b < blockIdx.x; b += blockDim.x) before += counts[b];
+    if (before) atomicAdd(&s_base, before);
+    // the warp's variables: 1024, a row of 32 at a time
+    const uint32_t v0 = blockIdx.x * IN_VARS + warp * 1024u;
+    uint32_t n = 0;
+    for (uint32_t r = 0; r < 32u; r++) {
+        const uint32_t v = v0 + 32u * r + lane;
+        n += __popc(__ballot_sync(0xFFFFFFFFu, v < D.nv && partial[v] != 0));
+    }
+    if (lane == 0) s_warp[warp] = n;
+    __syncthreads();
+    uint32_t pos = s_base;
+    for (uint32_t i = 0; i < warp; i++) pos += s_warp[i];
+    for (uint32_t r = 0; r < 32u; r++) {
+        const uint32_t v = v0 + 32u * r + lane;
+        const int8_t x = v < D.nv ? partial[v] : (int8_t)0;
+        const uint32_t m = __ballot_sync(0xFFFFFFFFu, x != 0);
+        if (x) D.trail[pos + __popc(m & ((1u << lane) - 1u))] = v | (x < 0 ? TRAIL_F : 0u);
+        pos += (uint32_t)__popc(m);
+    }
+    if (blockIdx.x == gridDim.x - 1u && threadIdx.x == blockDim.x - 1u) first_control(D, pos);
+}
+
+// The closure, one byte per variable: 1 true, -1 false, 2 both, 0 unassigned.
+__global__ void __launch_bounds__(256) closure_kernel(Dev D, int8_t *closure)
+{
+    const uint32_t nt = gridDim.x * blockDim.x;
+    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < D.asg_words; w += nt) {
+        const uint32_t m = D.asg[w];
+        unsigned long long out = 0;
+        for (uint32_t q = 0; q < 8u; q++) {
+            const uint32_t c = (m >> (4u * q)) & 3u;
+            out |= (unsigned long long)(uint8_t)(c == V_F ? -1 : c == 3u ? 2 : (int)c) << (8u * q);
+        }
+        reinterpret_cast<unsigned long long *>(closure)[w] = out;   // the buffer holds 8 x asg_words bytes
+    }
+}
+
+}  // namespace
+
+cudaError_t launch_reset(const Dev &D, bool codes, cudaStream_t st)
+{
+    const uint32_t n = std::max(std::max(codes ? D.nv : 0u, D.J + 4u), 2u * (D.dirty ? D.dirty_words : 0u));
+    reset_kernel<<<(int)std::min<uint32_t>((n + 255u) / 256u, 1216u), 256, 0, st>>>(D, codes, 0u);
+    return cudaGetLastError();
+}
+
+// Blocks of the input kernels (one count word each).
+uint32_t input_blocks(const Dev &D) { return std::max<uint32_t>(1u, (D.nv + IN_VARS - 1u) / IN_VARS); }
+
+// The state of a propagation from the partial assignment on the device.
+cudaError_t launch_input(const Dev &D, const int8_t *partial, uint32_t *counts, cudaStream_t st)
+{
+    cudaError_t e = launch_reset(D, false, st);
+    if (e != cudaSuccess) return e;
+    input_codes_kernel<<<input_blocks(D), 256, 0, st>>>(D, partial, counts);
+    input_trail_kernel<<<input_blocks(D), 256, 0, st>>>(D, partial, counts);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_closure(const Dev &D, int8_t *closure, cudaStream_t st)
+{
+    closure_kernel<<<(int)std::max<uint32_t>(1u, std::min<uint32_t>((D.asg_words + 255u) / 256u, 1216u)), 256, 0, st>>>(D, closure);
+    return cudaGetLastError();
+}
+
+}  // namespace aspgpu
