@@ -22,6 +22,8 @@ int batch_threads(int config);
 cudaError_t launch_reset(const Dev &D, bool codes, cudaStream_t st);
 uint32_t input_blocks(const Dev &D);
 cudaError_t launch_input(const Dev &D, const int8_t *partial, uint32_t *counts, cudaStream_t st);
+cudaError_t launch_occurrences(const Dev &D, uint32_t n_lits, uint32_t *off, uint32_t *occ, uint32_t *count,
+                               uint32_t *sums, cudaStream_t st);
 cudaError_t launch_closure(const Dev &D, int8_t *closure, cudaStream_t st);
 int mlp_prior(const uint16_t *d_w, const std::vector<float> &features, int64_t n, float *d_out, cudaStream_t st);
 cudaError_t batch_configure(int config, bool units, size_t smem, int *blocks_per_sm);
@@ -297,7 +299,7 @@ static void use_unit_lists(Dev &D, const UnitLists &U)
 static int plan_grid(asp_prog *p, const HostStore &H)
 {
     Dev &D = p->D;
-    const size_t max_smem = 220 * 1024;
+    const size_t max_smem = SOLVE_SMEM_BUDGET;
     const size_t base_smem = 8ull * D.WW + 8ull * 32 + 4ull * 16 + MLP_SMEM_BYTES;
     int per_sm = 0;
     cudaError_t e = solve_configure(p->block, max_smem, &per_sm);
@@ -312,6 +314,10 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     if (p->opt.grid_ctas > 0) g = std::min(p->opt.grid_ctas, max_grid);
     p->grid = g;
     D.G = (uint32_t)g;
+    // one CTA follows up to this many claims in the time a sweep round takes:
+    // about 8 us and 0.2 ns a literal of the CTA's part, against about 0.03 us
+    // a claim
+    if (D.occ) D.narrow_max = (uint32_t)std::min<uint64_t>(256u + total / (uint64_t)g / 128u, 1u << 20);
     // groups [glo[i], glo[i+1]) for CTA i, balanced by literal count
     const uint32_t ng = (uint32_t)H.n_groups;
     std::vector<uint32_t> glo(g + 1, ng);
@@ -368,7 +374,7 @@ static int plan_grid(asp_prog *p, const HostStore &H)
 // they fit in the per-CTA shared-memory budget of the batch kernel
 // configuration (3 or 6 CTAs in an SM's 228 KB, less reserved and static
 // shared memory).
-constexpr size_t BATCH_SMEM_BUDGET[2] = {72 * 1024 - 1024, 34 * 1024};
+constexpr size_t BATCH_SMEM_BUDGET[2] = {68 * 1024, 30 * 1024};
 // frontier by units in batches: the unit lists of a program's single-CTA
 // partition are built for programs of at most this many sweep units (about
 // 20k atoms at 4 rules per atom), whatever the program's own frontier option,
@@ -385,6 +391,7 @@ static int plan_batch(asp_prog *p, const HostStore &H, int config)
     an[0] = 3 * D1.J;
     const size_t base = 8ull * D1.WW + 8ull * 32 + 4ull * 16 + MLP_SMEM_BYTES;
     D1.G = 1;
+    if (D1.occ) D1.narrow_max = (uint32_t)std::min<uint64_t>(64u + p->D.static_checks / 1024u, 1u << 20);
     int rc = choose_view(p, H, D1, boff, alo, an, base, BATCH_SMEM_BUDGET[config]);
     if (rc != ASP_OK) return rc;
     D1.cta_boff = upload(p, boff, rc);
@@ -702,7 +709,7 @@ int asp_load_ground(int32_t n_atoms, int32_t n_rules, const int32_t *head,
     D.asg = (uint32_t *)alloc((size_t)D.asg_words * 4 + 4);
     D.dl = (int32_t *)alloc((size_t)D.nv * 4 + 4);
     D.reason = (uint32_t *)alloc((size_t)D.nv * 4 + 4);
-    D.deps = (unsigned long long *)alloc((size_t)D.nv * WW * 8 + 8);
+    D.deps = (unsigned long long *)alloc((size_t)D.nv * WW * 8 + 16);
     D.trail = (uint32_t *)alloc((size_t)D.nv * 4 + 4);
     D.level_start = (uint32_t *)alloc(((size_t)D.J + 4) * 4);
     D.dec_var = (uint32_t *)alloc(((size_t)D.J + 4) * 4);
@@ -724,24 +731,16 @@ int asp_load_ground(int32_t n_atoms, int32_t n_rules, const int32_t *head,
             if (e != cudaSuccess) rc = cuda_fail(e, "clear stamps");
         }
     }
-    if (rc == ASP_OK && p->opt.frontier == 1) {
-        // per variable, the ids of the bucket nogoods it occurs in
-        std::vector<uint32_t> off((size_t)D.nv + 1, 0), occ;
-        for (int L = 2; L <= BUCKET_MAX; L++) {
-            const std::vector<uint32_t> &rows = H.bucket_rows[L];
-            for (size_t t = 0; t < rows.size(); t++) off[(rows[t] >> 1) + 1]++;
+    if (rc == ASP_OK && D.nv > 0) {
+        // occurrence lists by literal, built on the device; the bitmaps and
+        // the trail, not in use yet, hold its counters
+        uint32_t *off = (uint32_t *)alloc(((size_t)2 * D.nv + 1) * 4), *occ = (uint32_t *)alloc((size_t)bucket_lits * 4);
+        if (rc == ASP_OK) {
+            D.occ_off = off;
+            D.occ = occ;
+            cudaError_t e = launch_occurrences(D, (uint32_t)bucket_lits, off, occ, (uint32_t *)D.deps, D.trail, p->stream);
+            if (e != cudaSuccess) rc = cuda_fail(e, "occurrence lists");
         }
-        for (uint32_t v = 0; v < D.nv; v++) off[v + 1] += off[v];
-        occ.resize(off[D.nv]);
-        std::vector<uint32_t> fill(off.begin(), off.end() - 1);
-        for (int L = 2; L <= BUCKET_MAX; L++) {
-            const std::vector<uint32_t> &rows = H.bucket_rows[L];
-            for (size_t t = 0; t < rows.size(); t++)
-                occ[fill[rows[t] >> 1]++] = bucket_nogood_id((uint32_t)L, (uint32_t)(t / (size_t)L));
-        }
-        D.frontier = 1;
-        D.occ_off = upload(p, off, rc);
-        if (rc == ASP_OK) D.occ = upload(p, occ, rc);
     }
     if (rc == ASP_OK) rc = plan_grid(p, H);
     if (rc == ASP_OK) rc = plan_batch(p, H, 0);

@@ -1,5 +1,6 @@
 // Device-side data layout and small helpers of the solver (internal).
 #pragma once
+#include <cstddef>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -45,6 +46,11 @@ enum ViewMode : uint32_t { VIEW_PLAIN = 1, VIEW_PACKED = 2, VIEW_BYTES = 3 };
 
 constexpr unsigned long long NO_KEY = ~0ull;
 
+// Dynamic shared memory a program's view may take in the solve kernel (the
+// rest of the 227 KB holds the static arrays: claim list, unit queue, queue
+// of the narrow rounds).
+constexpr size_t SOLVE_SMEM_BUDGET = 196 * 1024;
+
 // learned heuristic: 16 features -> 64 hidden (ReLU) -> 1, parameters
 // W1[64][16], b1[64], w2[64], b2
 constexpr int N_FEATURES = 16, N_HIDDEN = 64;
@@ -65,6 +71,7 @@ struct Ctl {              // double-buffered control block (phase parity)
     int32_t status, err;
     int32_t conflict;
     uint32_t full;              // the next round sweeps every nogood (else the frontier)
+    uint32_t chased, pad;       // the last claims have been followed by narrow rounds
 };
 
 struct Acc {              // per-phase accumulators, indexed by phase % 4
@@ -171,10 +178,14 @@ struct Dev {
     const float *prior;       // heuristic 3: per-rule score computed at load
     uint32_t *trace;          // [trace_cap][TRACE_WORDS]
     uint32_t trace_cap;
+    // occurrence lists (Algorithm 2's Map): the ids of the bucket nogoods
+    // that hold literal l are occ[occ_off[l] .. occ_off[l + 1]); a phase
+    // with at most narrow_max claims to follow is run by one CTA through them
+    // (narrow_rounds; 0 = no lists)
+    uint32_t narrow_max;
     // frontier propagation (Algorithm 2's idea): a round checks only the
-    // bucket nogoods of the variables assigned in the previous round, found
-    // through occ_off/occ (per variable, the ids of the bucket nogoods it
-    // occurs in); full sweeps after (re)starts and backjumps
+    // bucket nogoods of the variables assigned in the previous round; full
+    // sweeps after (re)starts and backjumps
     uint32_t frontier;
     const uint32_t *occ_off, *occ;
     // frontier = 2 (frontier by bucket units): the sweep units of the static

@@ -6,16 +6,17 @@
 // cached blocks), and processes whose device memory is handed out up front
 // by a pool or a framework that owns all of it.  This entry point computes the
 // same closure as asp_debug_propagate, but all of its working memory (the
-// assignment codes, the round counters and the grid barrier) lives in one
-// fixed static device array defined below.  It reads the program's nogood
-// store (created earlier by asp_load_ground) and the caller's device buffers,
-// and allocates nothing.
+// assignment codes, the list of assigned literals, the round counters and the
+// grid barrier) lives in one fixed static device array defined below.  It
+// reads the program's nogood store and occurrence lists (created earlier by
+// asp_load_ground) and the caller's device buffers, and allocates nothing.
 //
 // The array is shared by every call in the process: calls that overlap on
 // the GPU (two streams, or two host threads) race on it and give wrong
 // results.  Each call re-initialises what must start at zero.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <mutex>
 
@@ -28,19 +29,30 @@ namespace aspgpu {
 constexpr uint32_t NOALLOC_CTL_WORDS = 64;
 // largest program the static array serves: 2^20 variables (4-bit codes)
 constexpr uint32_t NOALLOC_MAX_VARS = 1u << 20;
-constexpr uint32_t NOALLOC_WORDS = NOALLOC_CTL_WORDS + NOALLOC_MAX_VARS / 8u;
+constexpr uint32_t NOALLOC_CODES = NOALLOC_MAX_VARS / 8u;
+constexpr uint32_t NOALLOC_WORDS = NOALLOC_CTL_WORDS + NOALLOC_CODES + NOALLOC_MAX_VARS;
 
-// 512 KB of codes + 256 B of control words; every GPU that loads the
-// library holds it until the process exits.
+// 512 KB of codes, 4 MB of list and 256 B of control words; every GPU that
+// loads the library holds them until the process exits.
 static __device__ __align__(256) uint32_t g_noalloc_scratch[NOALLOC_WORDS];
 
 namespace {
 
 struct NaCtl {                 // first words of the scratch array
-    unsigned int count, gen, err, pad;
-    unsigned int nclaim[3];
-    unsigned int conflict;
+    unsigned int count, err, conflict;
+    // of the grid's rounds, by their number modulo 3 (a round clears the next
+    // one's, whose last readers are two barriers back): literals listed, conflict
+    unsigned int nclaim[3], conf[3];
+    // CTA 0's narrow rounds: number of the next round, literals it left to
+    // follow, conflict; and the counter of literals past its shared lists
+    unsigned int next, left, nconf, nover;
 };
+
+constexpr uint32_t NA_THREADS = 768, NA_LIST = 1024;
+// claims that CTA 0 follows alone: a round of the grid costs its barrier and
+// list copy (about 3 us) over the chain of loads of a narrow round, in which
+// 192 claims go at a time
+constexpr uint32_t NA_NARROW = 384;
 
 __device__ __forceinline__ unsigned long long na_timer()
 {
@@ -56,38 +68,37 @@ __device__ __forceinline__ uint32_t na_ld_acquire(const unsigned int *p)
     return v;
 }
 
-// grid barrier on the scratch control words; bounded wait (~20 s)
-__device__ bool na_sync(NaCtl *c)
+// CTA barrier that counts every thread on its own: warps arrive from loops
+// with different trip counts
+__device__ __forceinline__ void na_cta_sync() { asm volatile("barrier.sync 0;" ::: "memory"); }
+
+// grid barrier number gen on the scratch control words (its counter is zeroed
+// before each launch); bounded wait (~20 s)
+__device__ bool na_sync(NaCtl *c, uint32_t gen)
 {
     __shared__ int s_ok;
-    __syncthreads();
+    na_cta_sync();
     if (threadIdx.x == 0) {
         int ok = 1;
         if (gridDim.x > 1) {
-            unsigned g = na_ld_acquire(&c->gen);
-            __threadfence();
-            if (atomicAdd(&c->count, 1u) == gridDim.x - 1) {
-                atomicExch(&c->count, 0u);
-                __threadfence();
-                atomicAdd(&c->gen, 1u);
-            } else {
-                unsigned long long t0 = na_timer();
-                unsigned spins = 0;
-                while (na_ld_acquire(&c->gen) == g) {
-                    if (na_ld_acquire(&c->err)) { ok = 0; break; }
-                    if ((++spins & 1023u) == 0 && na_timer() - t0 > 20000000000ull) {
-                        atomicExch(&c->err, 1u);
-                        ok = 0;
-                        break;
-                    }
+            const uint32_t target = (gen + 1u) * gridDim.x;
+            asm volatile("red.release.gpu.global.add.u32 [%0], 1;" :: "l"(&c->count) : "memory");
+            unsigned long long t0 = 0;
+            for (unsigned spins = 1; (int)(na_ld_acquire(&c->count) - target) < 0; spins++) {
+                if ((spins & 255u) != 0u) continue;
+                const unsigned long long now = na_timer();
+                if (t0 == 0) t0 = now;
+                if (na_ld_acquire(&c->err) || now - t0 > 20000000000ull) {
+                    atomicExch(&c->err, 1u);
+                    ok = 0;
+                    break;
                 }
             }
+            __threadfence();
         }
-        __threadfence();
-        if (na_ld_acquire(&c->err)) ok = 0;
         s_ok = ok;
     }
-    __syncthreads();
+    na_cta_sync();
     return s_ok != 0;
 }
 
@@ -98,106 +109,237 @@ __device__ __forceinline__ uint32_t na_val(const uint32_t *asg, uint32_t v, uint
     return (c & fresh) ? 0u : (c & 3u);
 }
 
+// The CTA's literals listed in the current round: shared memory first, then
+// straight to the list (slots of counter *n after base).
+struct NaList {
+    uint32_t *list;            // of the scratch array
+    uint32_t base;             // its first free word
+    unsigned int *n;           // counter of the round
+    uint32_t *s_lit;           // [NA_LIST]
+    unsigned int *s_n;
+    unsigned int *conf;        // the round's conflict flag
+};
+
+__device__ __forceinline__ void na_push(const NaList &O, uint32_t l)
+{
+    const uint32_t i = atomicAdd(O.s_n, 1u);
+    if (i < NA_LIST) { O.s_lit[i] = l; return; }
+    const uint32_t pos = O.base + atomicAdd(O.n, 1u);
+    if (pos < NOALLOC_MAX_VARS) O.list[pos] = l;
+}
+
+// Copies the CTA's literals to the list, one global atomic a CTA.
+__device__ __forceinline__ void na_flush(const NaList &O)
+{
+    __shared__ uint32_t s_base;
+    na_cta_sync();
+    const uint32_t n = min(*O.s_n, NA_LIST);
+    if (threadIdx.x == 0) s_base = O.base + (n ? atomicAdd(O.n, n) : 0u);
+    na_cta_sync();
+    const uint32_t b = s_base;
+    for (uint32_t i = threadIdx.x; i < n; i += blockDim.x)
+        if (b + i < NOALLOC_MAX_VARS) O.list[b + i] = O.s_lit[i];
+    if (threadIdx.x == 0) *O.s_n = 0u;
+}
+
+__device__ __forceinline__ void na_conflict(NaCtl *c, const NaList &O)
+{
+    atomicExch(&c->conflict, 1u);
+    atomicExch(O.conf, 1u);
+}
+
 // claim the complement of literal l; conflict flag on a clash
-__device__ __forceinline__ void na_claim(uint32_t *asg, NaCtl *c, uint32_t l, uint32_t fresh, uint32_t slot)
+__device__ __forceinline__ void na_claim(uint32_t *asg, NaCtl *c, uint32_t l, uint32_t fresh, const NaList &O)
 {
     const uint32_t v = l >> 1, valbit = (l & 1u) ? V_T : V_F, sh = (v & 7u) * 4u;
     const uint32_t old = (atomicOr(asg + (v >> 3), (valbit | fresh) << sh) >> sh) & 3u;
-    if (old == 0u) atomicAdd(&c->nclaim[slot], 1u);
-    else if (!(old & valbit)) atomicExch(&c->conflict, 1u);
+    if (old == 0u) na_push(O, l ^ 1u);
+    else if (!(old & valbit)) na_conflict(c, O);
 }
 
-__global__ void __launch_bounds__(768, 1) noalloc_propagate_kernel(Dev D, const int8_t *partial, int8_t *closure,
-                                                                   int32_t *conflict_out, uint32_t *scratch)
+// Checks the bucket nogoods of the n literals at `from` (each holds since the
+// round before; no other nogood can have become unit or violated), four lanes
+// a literal, groups of four lanes [g, g + ng, ...).  The literal's own fresh
+// bit, of the other parity, is cleared meanwhile.  SHARED: `from` is in shared
+// memory.
+template <bool SHARED>
+__device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c, const uint32_t *from, uint32_t n, uint32_t g,
+                                          uint32_t ng, uint32_t fresh, uint32_t stale, const NaList &O)
 {
+    const uint32_t sub = threadIdx.x & 3u;
+    for (uint32_t i = g; i < n; i += ng) {
+        const uint32_t l0 = SHARED ? from[i] : __ldcg(from + i), y = l0 >> 1;
+        const uint32_t o0 = __ldg(D.occ_off + l0), o1 = __ldg(D.occ_off + l0 + 1u);
+        if (sub == 0u) atomicAnd(asg + (y >> 3), ~(stale << ((y & 7u) * 4u)));
+        for (uint32_t o = o0 + sub; o < o1; o += 4u) {
+            const uint32_t id = __ldg(D.occ + o), L = ((id >> 27) & 15u) + 1u, stride = D.bk_n[L];
+            const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
+            bool sat = false;
+            uint32_t n_un = 0, ul = 0;
+            for (uint32_t q0 = 0; q0 < L && !sat && n_un < 2u; q0 += 4u) {
+                uint32_t l[4], v[4];
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; q++) l[q] = q0 + q < L ? __ldg(base + (size_t)(q0 + q) * stride) : PAD_LIT;
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; q++) v[q] = l[q] != PAD_LIT ? na_val(asg, l[q] >> 1, fresh) : 3u;
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; q++) {
+                    if (l[q] == PAD_LIT) continue;
+                    sat |= v[q] == ((l[q] & 1u) ? V_T : V_F);
+                    if (v[q] == 0u) { n_un++; ul = l[q]; }
+                }
+            }
+            if (sat || n_un > 1u) continue;
+            if (n_un == 0u) na_conflict(c, O);
+            else na_claim(asg, c, ul, fresh, O);
+        }
+    }
+}
+
+// The fixpoint by following assignments: a round checks the nogoods of the
+// literals listed by the round before (first the caller's assignment), found
+// through the occurrence lists, instead of every nogood of the store; with at
+// most NA_NARROW of them CTA 0 goes on alone, with CTA barriers.  Nogoods in
+// no list (more than BUCKET_MAX literals) are checked in the grid's rounds,
+// and the last round is one.  A round is bound by its chain of dependent loads
+// (list, list bounds, nogood id, literals, codes, claim) and its barrier.
+__global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D, const int8_t *partial, int8_t *closure,
+                                                                          int32_t *conflict_out, uint32_t *scratch)
+{
+    __shared__ uint32_t s_lit[2][NA_LIST];
+    __shared__ unsigned int s_n[3], s_conf;
     NaCtl *c = reinterpret_cast<NaCtl *>(scratch);
-    uint32_t *asg = scratch + NOALLOC_CTL_WORDS;
+    uint32_t *asg = scratch + NOALLOC_CTL_WORDS, *list = asg + NOALLOC_CODES;
     const uint32_t nth = gridDim.x * blockDim.x, gt = blockIdx.x * blockDim.x + threadIdx.x;
-    const uint32_t lane = threadIdx.x & 31u, gw = gt >> 5, nw = nth >> 5;
+    const uint32_t lane = threadIdx.x & 31u, nw = nth >> 5;
+    // consecutive warps of the grid sit on different CTAs, so short lists
+    // spread over the SMs
+    const uint32_t gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     const uint32_t words = (D.nv + 7u) >> 3;
-    // the caller's partial assignment, committed (no fresh bits)
+    if (threadIdx.x == 0) s_n[0] = s_n[1] = s_n[2] = s_conf = 0u;
+    na_cta_sync();
+    NaList O{list, 0u, &c->nclaim[2], s_lit[0], &s_n[0], &c->conf[2]};
+    // the caller's partial assignment, committed (no fresh bits); round -1
+    const bool aligned = ((reinterpret_cast<uintptr_t>(partial) | reinterpret_cast<uintptr_t>(closure)) & 7u) == 0u;
     for (uint32_t w = gt; w < words; w += nth) {
+        unsigned long long x = 0;
+        if (aligned && 8u * w + 8u <= D.nv) x = reinterpret_cast<const unsigned long long *>(partial)[w];
+        else
+            for (uint32_t q = 0; q < 8u && 8u * w + q < D.nv; q++) x |= (unsigned long long)(uint8_t)partial[8u * w + q] << (8u * q);
         uint32_t m = 0;
-        for (uint32_t q = 0; q < 8u; q++) {
-            uint32_t v = 8u * w + q;
-            if (v < D.nv && partial[v]) m |= (partial[v] > 0 ? V_T : V_F) << (4u * q);
+        for (uint32_t q = 0; x >> (8u * q); q++) {
+            const int8_t p = (int8_t)(x >> (8u * q));
+            if (p) {
+                m |= (p > 0 ? V_T : V_F) << (4u * q);
+                na_push(O, mk_lit(8u * w + q, p < 0));
+            }
+            if (q == 7u) break;
         }
         asg[w] = m;
     }
-    if (!na_sync(c)) return;
-    // round 0 applies the unit nogoods; later rounds sweep the store
-    for (uint32_t r = 0;; r++) {
-        const uint32_t fresh = 4u << (r & 1u), slot = r % 3u;
-        // clear the fresh bits of round r-1 (the other parity)
-        const uint32_t old_fresh = 4u << ((r + 1u) & 1u);
-        const uint32_t clear = ~(old_fresh * 0x11111111u);
-        if (r > 0)
-            for (uint32_t w = gt; w < words; w += nth) atomicAnd(asg + w, clear);
-        if (gt == 0) c->nclaim[(r + 1u) % 3u] = 0u;
-        if (r == 0) {
+    na_flush(O);
+    uint32_t gen = 0, from = 0, to = 0;       // literals [from, to) are to be followed
+    bool ok = na_sync(c, gen++);
+    if (ok) to = __ldcg(&c->nclaim[2]);
+    // r: rounds so far (its parity names the fresh bit), k: the grid's rounds;
+    // the first also applies the unit nogoods
+    for (uint32_t r = 0, k = 0; ok; k++) {
+        const uint32_t fresh = 4u << (r & 1u), stale = 4u << ((r + 1u) & 1u), slot = k % 3u;
+        if (gt == 0) c->nclaim[(k + 1u) % 3u] = c->conf[(k + 1u) % 3u] = 0u;
+        O = NaList{list, to, &c->nclaim[slot], s_lit[0], &s_n[0], &c->conf[slot]};
+        if (k == 0)
             for (uint32_t i = gt; i < D.n_units; i += nth) {
                 const uint32_t l = __ldg(D.lits + D.units_base + i) & ~END_BIT;
                 const uint32_t v = na_val(asg, l >> 1, fresh);
-                if (v == 0u) na_claim(asg, c, l, fresh, slot);
-                else if (v == ((l & 1u) ? V_F : V_T)) atomicExch(&c->conflict, 1u);
+                if (v == 0u) na_claim(asg, c, l, fresh, O);
+                else if (v == ((l & 1u) ? V_F : V_T)) na_conflict(c, O);
             }
-        } else {
-            // buckets: one lane per nogood
-            for (uint32_t L = 2; L <= (uint32_t)BUCKET_MAX; L++) {
-                const uint32_t n = D.bk_n[L];
-                const uint32_t *base = D.lits + D.bk_base[L];
-                for (uint32_t k = gt; k < n; k += nth) {
-                    bool sat = false;
-                    uint32_t n_un = 0, ul = 0;
-                    for (uint32_t q = 0; q < L && !sat; q++) {
-                        const uint32_t l = __ldg(base + (size_t)q * n + k);
-                        const uint32_t v = na_val(asg, l >> 1, fresh);
-                        if (v == ((l & 1u) ? V_T : V_F)) sat = true;
-                        else if (v == 0u) { n_un++; ul = l; }
-                    }
-                    if (sat || n_un > 1u) continue;
-                    if (n_un == 0u) atomicExch(&c->conflict, 1u);
-                    else na_claim(asg, c, ul, fresh, slot);
-                }
+        na_follow<false>(D, asg, c, list + from, to - from, gw * 8u + (lane >> 2), nw * 8u, fresh, stale, O);
+        // long nogoods: one warp per nogood, lanes over literals
+        for (uint32_t i = gw; i < D.n_long; i += nw) {
+            __syncwarp();
+            const uint32_t id = __ldg(D.long_ids + i);
+            bool sat = false;
+            uint32_t n_un = 0, ul = 0;
+            for (uint32_t off = id;; off += 32u) {
+                const uint32_t w = __ldg(D.lits + off + lane);
+                const unsigned Bend = __ballot_sync(0xFFFFFFFFu, (w & END_BIT) != 0u);
+                const unsigned valid = Bend ? ((2u << (__ffs(Bend) - 1)) - 1u) : 0xFFFFFFFFu;
+                const uint32_t l = w & ~END_BIT;
+                const bool mine = (valid >> lane) & 1u;
+                const uint32_t v = mine ? na_val(asg, l >> 1, fresh) : 0u;
+                const unsigned Bopp = __ballot_sync(0xFFFFFFFFu, mine && v == ((l & 1u) ? V_T : V_F));
+                const unsigned Bun = __ballot_sync(0xFFFFFFFFu, mine && v == 0u);
+                const uint32_t first = __shfl_sync(0xFFFFFFFFu, l, Bun ? __ffs(Bun) - 1 : 0);
+                if (Bun && n_un == 0) ul = first;
+                n_un += (uint32_t)__popc(Bun);
+                if (Bopp) { sat = true; break; }
+                if (Bend || n_un > 1u) break;
             }
-            // long nogoods: one warp per nogood, lanes over literals
-            for (uint32_t i = gw; i < D.n_long; i += nw) {
-                const uint32_t id = __ldg(D.long_ids + i);
-                bool sat = false;
-                uint32_t n_un = 0, ul = 0;
-                for (uint32_t off = id;; off += 32u) {
-                    const uint32_t w = __ldg(D.lits + off + lane);
-                    const unsigned Bend = __ballot_sync(0xFFFFFFFFu, (w & END_BIT) != 0u);
-                    const unsigned valid = Bend ? ((2u << (__ffs(Bend) - 1)) - 1u) : 0xFFFFFFFFu;
-                    const uint32_t l = w & ~END_BIT;
-                    const bool mine = (valid >> lane) & 1u;
-                    const uint32_t v = mine ? na_val(asg, l >> 1, fresh) : 0u;
-                    const unsigned Bopp = __ballot_sync(0xFFFFFFFFu, mine && v == ((l & 1u) ? V_T : V_F));
-                    const unsigned Bun = __ballot_sync(0xFFFFFFFFu, mine && v == 0u);
-                    const uint32_t first = __shfl_sync(0xFFFFFFFFu, l, Bun ? __ffs(Bun) - 1 : 0);
-                    if (Bun && n_un == 0) ul = first;
-                    n_un += (uint32_t)__popc(Bun);
-                    if (Bopp) { sat = true; break; }
-                    if (Bend || n_un > 1u) break;
-                }
-                if (lane == 0 && !sat) {
-                    if (n_un == 0u) atomicExch(&c->conflict, 1u);
-                    else if (n_un == 1u) na_claim(asg, c, ul, fresh, slot);
-                }
+            if (lane == 0 && !sat) {
+                if (n_un == 0u) na_conflict(c, O);
+                else if (n_un == 1u) na_claim(asg, c, ul, fresh, O);
             }
         }
-        if (!na_sync(c)) break;
+        na_flush(O);
+        if (!(ok = na_sync(c, gen++))) break;
         // every thread sees the same counters after the barrier
-        const uint32_t claims = __ldcg(&c->nclaim[slot]);
-        const uint32_t conf = __ldcg(&c->conflict);
-        if (conf || (r > 0 && claims == 0u)) break;
-        if (!na_sync(c)) break;   // nobody may reset a slot still being read
+        const uint32_t n = __ldcg(&c->nclaim[slot]);
+        if (__ldcg(&c->conf[slot]) || n == 0u) break;
+        from = to;
+        to += n;
+        r++;
+        if (n > NA_NARROW) continue;
+        if (blockIdx.x == 0) {
+            // narrow rounds: a round's literals stay in shared memory, two
+            // lists in turn; if the last one lists too many they go to the
+            // list after `to`, for the grid
+            for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) s_lit[0][i] = __ldcg(list + from + i);
+            if (threadIdx.x == 0) c->nover = 0u;
+            uint32_t m = n, i = 0;
+            O.base = to;
+            O.n = &c->nover;
+            O.conf = &s_conf;
+            do {
+                na_cta_sync();
+                if (threadIdx.x == 0) s_n[(i + 2u) % 3u] = 0u;     // the next round's counter
+                O.s_lit = s_lit[(i + 1u) & 1u];
+                O.s_n = &s_n[(i + 1u) % 3u];
+                na_follow<true>(D, asg, c, s_lit[i & 1u], m, threadIdx.x >> 2, blockDim.x >> 2, 4u << ((r + i) & 1u),
+                                4u << ((r + i + 1u) & 1u), O);
+                na_cta_sync();
+                m = *O.s_n;
+                i++;
+            } while (m != 0u && m <= NA_NARROW && !s_conf);
+            if (m > NA_NARROW) na_flush(O);
+            na_cta_sync();
+            if (threadIdx.x == 0) {
+                s_n[0] = s_n[1] = s_n[2] = 0u;
+                c->next = r + i;
+                c->left = m > NA_NARROW ? m : 0u;
+                c->nconf = s_conf;
+            }
+        }
+        if (!(ok = na_sync(c, gen++))) break;
+        r = __ldcg(&c->next);
+        from = to;
+        to += __ldcg(&c->left);
+        if (__ldcg(&c->nconf) || (from == to && D.n_long == 0u)) break;
     }
-    for (uint32_t v = gt; v < D.nv; v += nth) {
-        const uint32_t code = (__ldcg(asg + (v >> 3)) >> ((v & 7u) * 4u)) & 3u;
-        closure[v] = code == V_T ? 1 : code == V_F ? -1 : code == 3u ? 2 : 0;
+    if (!ok && !gt) *conflict_out = -1;
+    if (!ok) return;
+    for (uint32_t w = gt; w < words; w += nth) {
+        const uint32_t m = __ldcg(asg + w);
+        unsigned long long x = 0;
+        for (uint32_t q = 0; q < 8u; q++) {
+            const uint32_t code = (m >> (4u * q)) & 3u;
+            x |= (unsigned long long)(uint8_t)(code == V_F ? -1 : code == 3u ? 2 : (int)code) << (8u * q);
+        }
+        if (aligned && 8u * w + 8u <= D.nv) reinterpret_cast<unsigned long long *>(closure)[w] = x;
+        else
+            for (uint32_t q = 0; q < 8u && 8u * w + q < D.nv; q++) closure[8u * w + q] = (int8_t)(x >> (8u * q));
     }
-    if (gt == 0) *conflict_out = __ldcg(&c->conflict) ? 1 : (__ldcg(&c->err) ? -1 : 0);
+    if (gt == 0) *conflict_out = __ldcg(&c->conflict) ? 1 : 0;
 }
 
 std::mutex g_noalloc_mu;
@@ -245,7 +387,7 @@ extern "C" int asp_propagate_noalloc(const asp_prog *p, const int8_t *d_partial,
             // (__launch_bounds__(768, 1)), so a grid of one CTA per SM always
             // fits a cooperative launch; the occupancy query confirms that
             // at least one block is resident per SM.
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, noalloc_propagate_kernel, 768, 0) != cudaSuccess ||
+            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, noalloc_propagate_kernel, NA_THREADS, 0) != cudaSuccess ||
                 per_sm < 1)
                 return internal_fail(ASP_E_CUDA, "the propagation kernel cannot be resident on an SM");
             g_noalloc_grid[dev] = sms;
@@ -254,6 +396,8 @@ extern "C" int asp_propagate_noalloc(const asp_prog *p, const int8_t *d_partial,
         scratch = g_noalloc_ptr[dev];
         grid = g_noalloc_grid[dev];
     }
+    // small programs take fewer CTAs: their barriers are shorter
+    grid = std::min<int>(grid, 1 + (int)(D->nv / 4096u));
     cudaStream_t st = internal_stream(p);
     // the control words start at zero on every call
     if (cudaMemsetAsync(scratch, 0, NOALLOC_CTL_WORDS * sizeof(uint32_t), st) != cudaSuccess)
@@ -261,7 +405,7 @@ extern "C" int asp_propagate_noalloc(const asp_prog *p, const int8_t *d_partial,
     Dev copy = *D;
     uint32_t *s = static_cast<uint32_t *>(scratch);
     void *args[] = {(void *)&copy, (void *)&d_partial, (void *)&d_closure, (void *)&d_conflict, (void *)&s};
-    if (cudaLaunchCooperativeKernel((void *)noalloc_propagate_kernel, dim3(grid), dim3(768), args, 0, st) != cudaSuccess)
+    if (cudaLaunchCooperativeKernel((void *)noalloc_propagate_kernel, dim3(grid), dim3(NA_THREADS), args, 0, st) != cudaSuccess)
         return internal_fail(ASP_E_CUDA, "launch failed");
     return ASP_OK;
 }

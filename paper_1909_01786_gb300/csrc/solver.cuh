@@ -1109,7 +1109,7 @@ __device__ __forceinline__ void frontier_round(const SweepCtx &X, uint32_t fr0, 
     for (uint32_t i = slot; i < count; i += X.nw) {
         const uint32_t v = dec ? X.dec_v : __ldcg(D.trail + fr0 + i) & TRAIL_VAR;
         if (v >= D.nv) continue;
-        const uint32_t o0 = __ldg(D.occ_off + v), o1 = __ldg(D.occ_off + v + 1u);
+        const uint32_t o0 = __ldg(D.occ_off + 2u * v), o1 = __ldg(D.occ_off + 2u * v + 2u);
         for (uint32_t ob = o0; ob < o1; ob += 32u) {
             const uint32_t o = ob + lane;
             const bool has = o < o1;
@@ -1962,14 +1962,14 @@ __device__ __forceinline__ View make_view(const Dev &D, uint32_t *vbase, uint32_
 }
 
 // Copy of a control struct read through L2 (other threads update it with
-// plain stores and atomics).
+// plain stores and atomics), by the 32 lanes of a warp.
 template <class T>
 __device__ __forceinline__ void ldcg_copy(T *dst, const T *src)
 {
     const uint32_t *s = reinterpret_cast<const uint32_t *>(src);
     uint32_t *d = reinterpret_cast<uint32_t *>(dst);
 #pragma unroll
-    for (uint32_t i = 0; i < sizeof(T) / 4u; i++) d[i] = __ldcg(s + i);
+    for (uint32_t i = threadIdx.x & 31u; i < sizeof(T) / 4u; i += 32u) d[i] = __ldcg(s + i);
 }
 
 __device__ __forceinline__ Smem make_smem(const Dev &D, unsigned long long *raw)
@@ -2005,6 +2005,274 @@ __device__ __forceinline__ bool group_sync(const Dev &D, uint32_t gen)
         return true;
     }
     return grid_sync(D.bar, gridDim.x, D.barrier_ns, gen);
+}
+
+// ------------------------------------------------------------ narrow rounds
+
+// Claims of the previous and of the current narrow round, cached in shared
+// memory (the trail holds all of them): e = trail entry, reason, and the
+// bounds of its literal's occurrence list unless the list's entries are among
+// the round's items; u = the reason's other variables, where it has at most
+// four literals.
+template <bool BATCH>
+struct NarrowQueue {
+    static constexpr uint32_t N = BATCH ? 48u : 256u, M = BATCH ? 192u : 1024u;
+    uint4 e[2][N];
+    uint32_t u[2][N][3];
+    uint32_t item[2][M];          // positions in D.occ to check
+    uint32_t n[3], m[3], conf[3]; // claims, items and conflict of round i: at (i + 1) % 3
+};
+
+// Entry k of a round's queue: its occurrence list goes to the items if it fits.
+template <bool BATCH>
+__device__ __forceinline__ void narrow_queue(NarrowQueue<BATCH> &Q, uint32_t buf, uint32_t slot, uint32_t k, uint32_t entry,
+                                             uint32_t id, uint32_t o0, uint32_t o1)
+{
+    if (k >= NarrowQueue<BATCH>::N) return;
+    const uint32_t c = o1 - o0;
+    if (c <= 64u && Q.m[slot] + c <= NarrowQueue<BATCH>::M) {
+        const uint32_t at = atomicAdd(&Q.m[slot], c);
+        if (at + c <= NarrowQueue<BATCH>::M) {
+            for (uint32_t j = 0; j < c; j++) Q.item[buf][at + j] = o0 + j;
+            o1 = o0;
+        } else {
+            // the items end before this list: the part inside must not be read
+            for (uint32_t j = at; j < NarrowQueue<BATCH>::M; j++) Q.item[buf][j] = 0xFFFFFFFFu;
+        }
+    }
+    Q.e[buf][k] = make_uint4(entry, id, o0, o1);
+}
+
+// OR into acc of word w of the bitmaps of variables u[0 .. C) other than x.
+// The words are loaded beside the levels that say whether they count.
+template <int C>
+__device__ __forceinline__ unsigned long long deps_or(const Dev &D, const uint32_t (&u)[C], uint32_t x, uint32_t w)
+{
+    int32_t lev[C];
+    unsigned long long word[C], acc = 0;
+#pragma unroll
+    for (int q = 0; q < C; q++) {
+        lev[q] = u[q] != x ? __ldcg(D.dl + u[q]) : 0;
+        word[q] = u[q] != x ? __ldcg(D.deps + (size_t)u[q] * D.WW + w) : 0ull;
+    }
+#pragma unroll
+    for (int q = 0; q < C; q++)
+        if (lev[q] > 1 && 64u * w < (uint32_t)lev[q]) acc |= word[q];
+    return acc;
+}
+
+// Dependency bitmap (Section 4.2, mk_dl_bitmap) of variable x, assigned by
+// bucket nogood id, by the 8 lanes `sub` of a group: each takes every eighth
+// word.  others: the nogood's other variables if it has at most four literals
+// and they are known (x where there are fewer), else null.
+__device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t id, const uint32_t *others, uint32_t nw, uint32_t sub)
+{
+    const uint32_t L = ((id >> 27) & 15u) + 1u, n = D.bk_n[L];
+    const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
+    if (others && L <= 4u) {
+        const uint32_t u[3] = {others[0], others[1], others[2]};
+        for (uint32_t w = sub; w < nw; w += 8u) D.deps[(size_t)x * D.WW + w] = deps_or<3>(D, u, x, w);
+        return;
+    }
+    for (uint32_t w = sub; w < nw; w += 8u) {
+        unsigned long long acc = 0;
+        for (uint32_t q0 = 0; q0 < L; q0 += 5u) {
+            uint32_t u[5];
+#pragma unroll
+            for (uint32_t q = 0; q < 5u; q++) u[q] = q0 + q < L ? __ldg(base + (size_t)(q0 + q) * n) >> 1 : x;
+            acc |= deps_or<5>(D, u, x, w);
+        }
+        D.deps[(size_t)x * D.WW + w] = acc;
+    }
+}
+
+// What a round counts and where its claims go.
+struct NarrowRound {
+    uint32_t cdl, fresh, buf, slot, out;      // buf, slot: of the next round's queue; out: trail index of its first claim
+    unsigned long long checks, visits;
+};
+
+__device__ __forceinline__ void narrow_count(const uint32_t l, uint32_t code, uint32_t fresh, bool &sat, uint32_t &n_un, uint32_t &ul)
+{
+    if (l == PAD_LIT) return;
+    const uint32_t val = eff_val(nib(code, l >> 1), fresh);
+    sat |= val == ((l & 1u) ? V_T : V_F);
+    if (val == 0u) { n_un++; ul = l; }
+}
+
+// Checks bucket nogood id: claims its unit literal's complement, or reports
+// the conflict.
+template <bool BATCH>
+__device__ __forceinline__ void narrow_check(const Dev &D, Acc *acc, NarrowQueue<BATCH> &Q, NarrowRound &R, uint32_t id)
+{
+    const uint32_t L = ((id >> 27) & 15u) + 1u, n = D.bk_n[L];
+    const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
+    bool sat = false;
+    uint32_t n_un = 0, ul = 0, l[4], c[4];
+#pragma unroll
+    for (uint32_t q = 0; q < 4u; q++) l[q] = q < L ? __ldg(base + (size_t)q * n) : PAD_LIT;
+#pragma unroll
+    for (uint32_t q = 0; q < 4u; q++) c[q] = l[q] != PAD_LIT ? __ldcg(D.asg + (l[q] >> 4)) : 0u;
+    if (L > 4u) {
+        // the rest beside the first four
+        uint32_t l2[BUCKET_MAX - 4], c2[BUCKET_MAX - 4];
+#pragma unroll
+        for (uint32_t q = 4; q < (uint32_t)BUCKET_MAX; q++) l2[q - 4u] = q < L ? __ldg(base + (size_t)q * n) : PAD_LIT;
+#pragma unroll
+        for (uint32_t q = 4; q < (uint32_t)BUCKET_MAX; q++) c2[q - 4u] = l2[q - 4u] != PAD_LIT ? __ldcg(D.asg + (l2[q - 4u] >> 4)) : 0u;
+#pragma unroll
+        for (uint32_t q = 4; q < (uint32_t)BUCKET_MAX; q++) narrow_count(l2[q - 4u], c2[q - 4u], R.fresh, sat, n_un, ul);
+    }
+#pragma unroll
+    for (uint32_t q = 0; q < 4u; q++) narrow_count(l[q], c[q], R.fresh, sat, n_un, ul);
+    R.checks += L;
+    R.visits++;
+    if (sat || n_un > 1u) return;
+    bool clash = n_un == 0u;
+    if (!clash) {
+        const uint32_t x = ul >> 1, valbit = (ul & 1u) ? V_T : V_F;
+        // the claimed literal's list bounds load beside the claim
+        const uint32_t a0 = __ldg(D.occ_off + (ul ^ 1u)), a1 = __ldg(D.occ_off + (ul ^ 1u) + 1u);
+        const int r = claim_var(D.asg, x, valbit, R.fresh);
+        if (r == 0) {
+            const uint32_t entry = x | (valbit == V_F ? TRAIL_F : 0u);
+            D.dl[x] = (int32_t)R.cdl;
+            D.reason[x] = id;
+            const uint32_t k = atomicAdd(&Q.n[R.slot], 1u), pos = R.out + k;
+            narrow_queue<BATCH>(Q, R.buf, R.slot, k, entry, id, a0, a1);
+            if (k < NarrowQueue<BATCH>::N && L <= 4u) {
+                uint32_t j = 0;
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; q++)
+                    if (l[q] != ul && j < 3u) Q.u[R.buf][k][j++] = l[q] != PAD_LIT ? l[q] >> 1 : x;
+            }
+            if (pos < D.nv) {
+                D.trail[pos] = entry;
+                if (D.tpos) D.tpos[x] = pos;
+            }
+        }
+        clash = r == 2;
+    }
+    if (clash) {
+        const unsigned long long key = ((unsigned long long)L << 32) | id;
+        atomicMin(&acc->ckey, key);
+        atomicMin(&acc->cslot[id % 3u], key);
+        Q.conf[R.slot] = 1u;
+    }
+}
+
+// Bitmaps of entries [i0, i0 + step, ...) of the n in queue buf (trail from qs).
+template <bool BATCH>
+__device__ __forceinline__ void narrow_bitmaps(const Dev &D, const NarrowQueue<BATCH> &Q, uint32_t buf, uint32_t qs, uint32_t n,
+                                               uint32_t i0, uint32_t step, uint32_t nw)
+{
+    for (uint32_t i = i0; i < n; i += step) {
+        if (i < NarrowQueue<BATCH>::N) {
+            const uint4 c = Q.e[buf][i];
+            narrow_deps(D, c.x & TRAIL_VAR, c.y, Q.u[buf][i], nw, threadIdx.x & 7u);
+        } else {
+            const uint32_t x = __ldcg(D.trail + qs + i) & TRAIL_VAR;
+            narrow_deps(D, x, __ldcg(D.reason + x), nullptr, nw, threadIdx.x & 7u);
+        }
+    }
+}
+
+// Propagation by one CTA, following the claims instead of sweeping the store
+// (Algorithm 2's Last/Next): the trail entries [first, tend) are the
+// assignments whose nogoods have not been checked yet (claims of the phase
+// before, or the decision, whose level and bitmap are in memory); every other
+// static nogood is as a sweep left it.  A round takes each entry's occurrence
+// list for the literal that now holds -- only those nogoods can have become
+// unit or violated -- and claims become the next round's entries, at
+// tbase, tbase + 1, ... of the trail.  Ends when a round claims nothing, on a
+// conflict, or when a round claims more than D.narrow_max (a sweep by every CTA
+// is then the faster way).
+//
+// Why: a search round assigns a few dozen variables (62 on average in the
+// 100k-atom program), and a sweep round costs its chain of barriers and loads
+// (15 us there on 152 CTAs) whatever its claims.  Here a round is bound by
+// four dependent loads (list entry, literals, codes, claim) and a CTA barrier.
+// A claim puts its list's positions into the next round's items, so a lane
+// checks one nogood whatever the lists' lengths; a third of the warps check
+// while the others compute the bitmaps of the round's entries (nothing in the
+// round reads those), from the variables that the claim left in shared memory.
+// The fresh bits alternate by round exactly as in sweeps: an entry's bit is
+// cleared while its round runs, when only the other parity's bit hides a
+// variable.  Returns the number of rounds; *n_claims is the number of claims,
+// *wide whether some are still to be checked.
+template <bool BATCH>
+__device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, Acc *acc, uint32_t cdl, uint32_t round, uint32_t first,
+                                                  uint32_t tend, uint32_t tbase, uint32_t *n_claims, bool *wide)
+{
+    __shared__ NarrowQueue<BATCH> Q;
+    constexpr uint32_t N = NarrowQueue<BATCH>::N, M = NarrowQueue<BATCH>::M;
+    const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarp = blockDim.x >> 5;
+    const uint32_t nw = cdl > 1u ? deps_words(D, cdl) : 0u;
+    // warps [0, wa) check nogoods, the others compute bitmaps; all do both
+    // when there is one warp, and all check at the root level
+    const bool split = nw && nwarp > 1u;
+    const uint32_t wa = split ? (nwarp + 1u) / 3u : nwarp;
+    if (tid == 0) Q.n[0] = Q.n[1] = Q.n[2] = Q.m[0] = Q.m[1] = Q.m[2] = Q.conf[0] = Q.conf[1] = Q.conf[2] = 0u;
+    cta_sync();
+    for (uint32_t i = tid; i < min(tend - first, N); i += blockDim.x) {
+        const uint32_t e = __ldcg(D.trail + first + i), l = mk_lit(e & TRAIL_VAR, (e & TRAIL_F) != 0u);
+        if ((l >> 1) >= D.nv) { atomicExch(&D.bar->err, 2u); Q.e[0][i] = make_uint4(0u, 0u, 0u, 0u); continue; }   // corrupt trail
+        narrow_queue<BATCH>(Q, 0u, 0u, i, e, 0u, __ldg(D.occ_off + l), __ldg(D.occ_off + l + 1u));
+    }
+    cta_sync();
+    uint32_t qs = first, qn = tend - first, it = 0;
+    NarrowRound R{cdl, 0u, 0u, 0u, tbase, 0ull, 0ull};
+    for (bool done = false; !done;) {
+        const uint32_t cur = it & 1u, stale = 4u << ((round + 1u) & 1u), items = min(Q.m[it % 3u], M);
+        R.fresh = 4u << (round & 1u);
+        R.buf = cur ^ 1u;
+        R.slot = (it + 1u) % 3u;
+        // cleared for the next round's claims; last read two barriers ago
+        if (tid == 0) Q.n[(it + 2u) % 3u] = Q.m[(it + 2u) % 3u] = Q.conf[(it + 2u) % 3u] = 0u;
+        if (warp < wa) {
+            for (uint32_t i = tid; i < items; i += wa * 32u) {
+                const uint32_t o = Q.item[cur][i];
+                if (o != 0xFFFFFFFFu) narrow_check<BATCH>(D, acc, Q, R, __ldg(D.occ + o));
+            }
+            for (uint32_t i = warp * 8u + (lane >> 2); i < qn; i += wa * 8u) {
+                uint32_t e, o0, o1;
+                if (i < N) {
+                    const uint4 c = Q.e[cur][i];
+                    e = c.x; o0 = c.z; o1 = c.w;
+                } else {
+                    e = __ldcg(D.trail + qs + i);
+                    const uint32_t l = mk_lit(e & TRAIL_VAR, (e & TRAIL_F) != 0u);
+                    if ((l >> 1) >= D.nv) { atomicExch(&D.bar->err, 2u); continue; }
+                    o0 = __ldg(D.occ_off + l); o1 = __ldg(D.occ_off + l + 1u);
+                }
+                const uint32_t y = e & TRAIL_VAR;
+                if ((lane & 3u) == 0u) atomicAnd(D.asg + (y >> 3), ~(stale << ((y & 7u) * 4u)));
+                for (uint32_t o = o0 + (lane & 3u); o < o1; o += 4u) narrow_check<BATCH>(D, acc, Q, R, __ldg(D.occ + o));
+            }
+        }
+        // bitmaps of this round's entries (the first round's have theirs)
+        if (nw && it > 0u && (!split || warp >= wa))
+            narrow_bitmaps<BATCH>(D, Q, cur, qs, qn, (split ? warp - wa : warp) * 4u + (lane >> 3), (split ? nwarp - wa : nwarp) * 4u, nw);
+        cta_sync();
+        const uint32_t n_new = Q.n[R.slot];
+        done = n_new == 0u || Q.conf[R.slot] || n_new > D.narrow_max || R.out + n_new >= D.nv;
+        qs = R.out;
+        qn = n_new;
+        R.out += n_new;
+        round++;
+        it++;
+    }
+    // the last claims' bitmaps, by every warp
+    if (nw) narrow_bitmaps<BATCH>(D, Q, it & 1u, qs, qn, warp * 4u + (lane >> 3), nwarp * 4u, nw);
+    cta_sync();
+    const uint32_t c32 = __reduce_add_sync(FULL_MASK, (unsigned)R.checks), v32 = __reduce_add_sync(FULL_MASK, (unsigned)R.visits);
+    if (lane == 0 && v32) {
+        atomicAdd(&acc->checks, (unsigned long long)c32);
+        atomicAdd(&acc->visits, (unsigned long long)v32);
+    }
+    *n_claims = R.out - tbase;
+    *wide = qn != 0u;
+    return it;
 }
 
 // Test-only failure injection: CTA D.stall_cta (thread 0) waits on a flag
@@ -2051,7 +2319,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
     }
     if (threadIdx.x == 0) { s_tlearned = 0ull; s_tbuckets = 0ull; s_wmax[0] = s_wmax[1] = 0ull; t_cta0 = globaltimer_ns(); }
 
-    if (threadIdx.x == 0) ldcg_copy(&sC, D.ctl);
+    if (threadIdx.x < 32u) ldcg_copy(&sC, D.ctl);
     if (D.heuristic == 2) {
         uint16_t *w = const_cast<uint16_t *>(reinterpret_cast<const uint16_t *>(S.mlp));
         for (uint32_t i = threadIdx.x; i < (uint32_t)MLP_PARAMS; i += blockDim.x) w[i] = __ldg(D.mlp + i);
@@ -2071,7 +2339,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
     cta_sync();
 
     for (uint32_t k = 0;; k++) {
-        if (threadIdx.x == 0) {
+        if (threadIdx.x < 32u) {
             ldcg_copy(&sC, D.ctl + (k & 1u));
             ldcg_copy(&sA, D.acc + ((k + 3u) & 3u));
         }
@@ -2093,7 +2361,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
 
         // the propagate-and-check sweep of ROUND and APPLY runs after the
         // switch (one copy of its code)
-        bool sw = false, sw_full = true;
+        bool sw = false, sw_full = true, nar = false;
         uint32_t sw_cdl = 0, sw_tbase = 0, sw_dec = 0xFFFFFFFFu, sw_fr0 = 0, sw_fr1 = 0;
         switch (C.op) {
         case OP_INIT: {
@@ -2202,8 +2470,10 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 }
                 break;
             }
-            if (A.nclaim == 0u && C.clean) {
+            const bool quiet = A.nclaim == 0u || C.chased;   // no claim is left to follow
+            if (quiet && C.clean) {
                 // fixpoint
+                if (leader) N.tb = tend;
                 if (D.mode == MODE_PROPAGATE) {
                     if (leader) { N.op = OP_DONE; N.status = 0; }
                     break;
@@ -2218,13 +2488,18 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 if (leader) N.op = OP_APPLY;
                 break;
             }
+            if (!quiet && !C.full && A.nclaim <= D.narrow_max) {
+                nar = true; sw_cdl = C.cdl; sw_fr0 = C.tb; sw_fr1 = sw_tbase = tend;
+                if (leader) atomicAdd(&D.stats->props, (unsigned long long)A.nclaim);
+                break;
+            }
             // frontier by units: this round's dirty units of the CTA
             if constexpr (UNITS && !BATCH) {
                 if (D.frontier >= 2u) build_unit_queue(D, cta, D.dirty + (C.round & 1u) * D.dirty_words, 0xFFFFFFFFu);
             }
             // make last round's claims visible: clear their fresh bit
             // (grid-wide) and put them in this CTA's view
-            for (uint32_t i = C.tc + gtid; i < tend; i += nthreads) {
+            for (uint32_t i = (C.chased ? tend : C.tb) + gtid; i < tend; i += nthreads) {
                 uint32_t v = __ldcg(D.trail + i) & TRAIL_VAR;
                 if (v >= D.nv) { atomicExch(&D.bar->err, 2u); continue; }   // corrupt trail: stop with an error
                 atomicAnd(D.asg + (v >> 3), ~(fresh_prev << ((v & 7u) * 4u)));
@@ -2240,11 +2515,11 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             cta_sync();
             sw = true; sw_cdl = C.cdl; sw_tbase = tend;
             sw_full = C.full != 0u || D.frontier == 0u || (!UNITS && D.frontier >= 2u);
-            sw_fr0 = C.tc; sw_fr1 = tend;
+            sw_fr0 = C.chased ? tend : C.tb; sw_fr1 = tend;
             if (leader) {
-                N.op = OP_ROUND; N.round = C.round + 1u; N.tc = tend; N.tb = tend; N.clean = 1; N.full = 0;
+                N.op = OP_ROUND; N.round = C.round + 1u; N.tc = tend; N.tb = tend; N.clean = 1; N.full = 0; N.chased = 0;
                 atomicAdd(&D.stats->rounds, 1ull);
-                atomicAdd(&D.stats->props, (unsigned long long)(tend - C.tc));
+                atomicAdd(&D.stats->props, (unsigned long long)A.nclaim);
                 if (sw_full) atomicAdd(&D.stats->checks, D.static_checks);
                 atomicAdd(&D.stats->visits, (sw_full ? D.static_nogoods : 0ull) + D.n_long + C.n_learned);
             }
@@ -2269,7 +2544,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 if (leader) {
                     // (frontier by units: completion claims mark no units, so
                     // the next round sweeps everything)
-                    N.op = OP_ROUND; N.round = C.round + 1u; N.tb = tend; N.tc = tend; N.clean = 0;
+                    N.op = OP_ROUND; N.round = C.round + 1u; N.tb = tend; N.clean = 0; N.chased = 0;
                     N.full = D.frontier >= 2u ? 1u : 0u;
                     atomicAdd(&D.stats->completions, 1ull);
                 }
@@ -2297,6 +2572,17 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 __threadfence();
                 atomicOr(D.asg + (bv >> 3), V_T << ((bv & 7u) * 4u));
             }
+            if (D.narrow_max) {
+                // the decision's consequences by narrow rounds: the store is at
+                // a fixpoint, so only the decision's nogoods can change it
+                nar = true; sw_cdl = L; sw_fr0 = tend; sw_fr1 = sw_tbase = tend + 1u;
+                if (leader) {
+                    N.cdl = L;
+                    atomicAdd(&D.stats->decisions, 1ull);
+                    if ((unsigned long long)L > D.stats->max_level) D.stats->max_level = L;
+                }
+                break;
+            }
             if (threadIdx.x == 0) view_set(V, bv, V_T);
             if (UNITS && D.frontier >= 2u) {
                 uint32_t *buf = D.dirty + (C.round & 1u) * D.dirty_words;
@@ -2317,7 +2603,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             sw_full = D.frontier == 0u || (!UNITS && D.frontier >= 2u);
             if (leader) {
                 N.op = OP_ROUND; N.cdl = L; N.round = C.round + 1u; N.tc = tend + 1u; N.tb = tend + 1u;
-                N.clean = 0; N.full = 0;
+                N.clean = 0; N.full = 0; N.chased = 0;
                 atomicAdd(&D.stats->decisions, 1ull);
                 atomicAdd(&D.stats->rounds, 1ull);
                 if (sw_full) atomicAdd(&D.stats->checks, D.static_checks);
@@ -2338,7 +2624,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             for (uint32_t i = newend + threadIdx.x; i < tend; i += blockDim.x)
                 view_clear(V, __ldcg(D.trail + i) & TRAIL_VAR);
             if (leader) {
-                N.op = OP_ROUND; N.cdl = C.target; N.tc = newend; N.tb = newend; N.clean = 0; N.full = 1;
+                N.op = OP_ROUND; N.cdl = C.target; N.tc = min(C.tc, newend); N.tb = newend; N.clean = 0; N.full = 1; N.chased = 0;
             }
             break;
         }
@@ -2514,6 +2800,23 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             if (leader) { N.op = OP_DONE; N.err = -6; }
             break;
         }
+        if (nar && cta0) {
+            // few claims (or the decision): CTA 0 follows them to the end, the
+            // others wait at the barrier; their views catch up with the trail
+            // at the next sweep.  A full-sweep program confirms the fixpoint
+            // with a sweep; so does a program with long or learned nogoods,
+            // which no list holds
+            cta_sync();
+            uint32_t n = 0;
+            bool wide = false;
+            const uint32_t its = narrow_rounds<BATCH>(D, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &wide);
+            if (leader) {
+                N.op = OP_ROUND; N.round = C.round + its; N.tb = sw_tbase;
+                N.chased = !wide; N.full = wide; N.clean = D.frontier != 0u && D.n_long + C.n_learned == 0u;
+                acc->nclaim = n;
+                atomicAdd(&D.stats->rounds, (unsigned long long)its);
+            }
+        }
         if (sw) {
             const unsigned long long ts = threadIdx.x == 0 ? globaltimer_ns() : 0ull;
             SweepCtx X{&D, V, fresh_cur, sw_cdl, sw_tbase, acc, true, true, sw_dec, cta, rank >> 5, size >> 5};
@@ -2583,6 +2886,6 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
 // The dynamic shared-memory limit is a property of each kernel, shared by
 // every program: it is set to the largest size any program may use, and
 // occupancy is computed for a program's own size.
-constexpr int MAX_DYN_SMEM = 220 * 1024;
+constexpr int MAX_DYN_SMEM = (int)SOLVE_SMEM_BUDGET;
 
 }  // namespace aspgpu
