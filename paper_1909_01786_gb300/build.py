@@ -14,11 +14,11 @@ LIB = os.path.join(OUT_DIR, "libaspgpu.so")
 INCLUDE = os.path.join(ROOT, "include")
 
 # (source, extra flags, object name): batch_kernel.cu is compiled once per
-# batch configuration and frontier mode, so the four instantiations of the
-# batch kernel compile in parallel
+# batch configuration and propagation schedule, so the five instantiations of
+# the batch kernel compile in parallel
 SOURCES = [("solve.cu", [], "solve"), ("solve_units.cu", [], "solve_units"), ("batch.cu", [], "batch")]
-SOURCES += [("batch_kernel.cu", [f"-DBATCH_CONFIG={c}", f"-DBATCH_UNITS={u}"], f"batch_kernel_c{c}_u{u}")
-            for c in (0, 1) for u in (0, 1)]
+SOURCES += [("batch_kernel.cu", [f"-DBATCH_CONFIG={c}", f"-DBATCH_LISTS={u}"], f"batch_kernel_c{c}_l{u}")
+            for c, u in ((0, 0), (0, 1), (1, 0), (1, 1), (2, 1))]
 SOURCES += [(f, [], f.split(".")[0]) for f in ("sweep.cu", "state.cu", "noalloc.cu", "mlp.cu", "api.cpp", "store.cpp",
                                                   "host_completion.cpp")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

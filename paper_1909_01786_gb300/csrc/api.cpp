@@ -22,12 +22,13 @@ int batch_threads(int config);
 cudaError_t launch_reset(const Dev &D, bool codes, cudaStream_t st);
 uint32_t input_blocks(const Dev &D);
 cudaError_t launch_input(const Dev &D, const int8_t *partial, uint32_t *counts, cudaStream_t st);
-cudaError_t launch_occurrences(const Dev &D, uint32_t n_lits, uint32_t *off, uint32_t *occ, uint32_t *count,
+cudaError_t launch_occurrences(const Dev &D, uint32_t n_lits, uint32_t *off, Occurrence *occ, uint32_t *rows, uint32_t *count,
                                uint32_t *sums, cudaStream_t st);
+uint32_t row_words(const Dev &D);
 cudaError_t launch_closure(const Dev &D, int8_t *closure, cudaStream_t st);
 int mlp_prior(const uint16_t *d_w, const std::vector<float> &features, int64_t n, float *d_out, cudaStream_t st);
-cudaError_t batch_configure(int config, bool units, size_t smem, int *blocks_per_sm);
-cudaError_t launch_batch(int config, bool units, const Dev *devs, const uint32_t *order, uint32_t n, unsigned int *queue, int grid,
+cudaError_t batch_configure(int config, bool lists, size_t smem, int *blocks_per_sm);
+cudaError_t launch_batch(int config, bool lists, const Dev *devs, const uint32_t *order, uint32_t n, unsigned int *queue, int grid,
                          size_t smem, cudaStream_t st);
 }  // namespace aspgpu
 
@@ -71,8 +72,7 @@ struct asp_prog {
     // the same program as one CTA solves it in a batch, for each batch
     // kernel configuration (256 threads, 3 per SM; 128 threads, 6 per SM)
     Dev D1[2]{};
-    UnitLists batch_units;              // frontier by units in batches
-    size_t smem1[2] = {0, 0};
+    size_t smem1[2] = {0, 0}, smem_base = 0;   // with the view; without
     int64_t n_nogoods = 0, n_literals = 0, n_units = 0, n_long = 0, store_bytes = 0;
     bool empty_nogood = false;
     // internal buffers for the blocking entry points
@@ -308,8 +308,9 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     const int max_grid = p->n_sms * per_sm;
     uint64_t total = 0;
     for (uint64_t x : H.group_lits) total += x;
-    // every SM for any real store; one CTA for tiny programs
-    int64_t want = (int64_t)(total / 2048) + 1;
+    // every SM for any real store; one CTA, which needs no grid barrier, for
+    // small programs
+    int64_t want = total <= 65536u ? 1 : (int64_t)(total / 2048) + 1;
     int g = (int)std::max<int64_t>(1, std::min<int64_t>(want, max_grid));
     if (p->opt.grid_ctas > 0) g = std::min(p->opt.grid_ctas, max_grid);
     p->grid = g;
@@ -318,6 +319,8 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     // about 8 us and 0.2 ns a literal of the CTA's part, against about 0.03 us
     // a claim
     if (D.occ) D.narrow_max = (uint32_t)std::min<uint64_t>(256u + total / (uint64_t)g / 128u, 1u << 20);
+    D.lists = D.occ && g == 1;
+    if (D.lists) D.narrow_max = 0xFFFFFFFFu;
     // groups [glo[i], glo[i+1]) for CTA i, balanced by literal count
     const uint32_t ng = (uint32_t)H.n_groups;
     std::vector<uint32_t> glo(g + 1, ng);
@@ -353,6 +356,9 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     int rc = choose_view(p, H, D, boff, alo, an, base_smem, max_smem);
     if (rc != ASP_OK) return rc;
     p->smem = base_smem + 4 * D.view_words;
+    // a copy of the codes for the narrow rounds where it fits beside the view
+    D.code_cache = p->smem + 4 * (size_t)D.asg_words <= max_smem;
+    if (D.code_cache) p->smem += 4 * (size_t)D.asg_words;
     if (D.frontier >= 2) {
         UnitLists U;
         rc = unit_lists(p, H, boff, D.G, ~0ull, U);
@@ -375,13 +381,9 @@ static int plan_grid(asp_prog *p, const HostStore &H)
 // configuration (3 or 6 CTAs in an SM's 228 KB, less reserved and static
 // shared memory).
 constexpr size_t BATCH_SMEM_BUDGET[2] = {68 * 1024, 30 * 1024};
-// frontier by units in batches: the unit lists of a program's single-CTA
-// partition are built for programs of at most this many sweep units (about
-// 20k atoms at 4 rules per atom), whatever the program's own frontier option,
-// so that the batch autotuner can choose between full sweeps and the unit
-// frontier
-constexpr uint64_t BATCH_MAX_UNITS = 1u << 14;
-
+// the same of the kernels that follow lists only (3, 6 or 1 CTAs per SM): a
+// program's codes are copied there if they fit
+constexpr size_t LISTS_SMEM_BUDGET[3] = {54 * 1024, 17 * 1024, 186 * 1024};
 static int plan_batch(asp_prog *p, const HostStore &H, int config)
 {
     Dev D1 = p->D;
@@ -391,27 +393,17 @@ static int plan_batch(asp_prog *p, const HostStore &H, int config)
     an[0] = 3 * D1.J;
     const size_t base = 8ull * D1.WW + 8ull * 32 + 4ull * 16 + MLP_SMEM_BYTES;
     D1.G = 1;
+    D1.lists = D1.code_cache = 0u;
     if (D1.occ) D1.narrow_max = (uint32_t)std::min<uint64_t>(64u + p->D.static_checks / 1024u, 1u << 20);
     int rc = choose_view(p, H, D1, boff, alo, an, base, BATCH_SMEM_BUDGET[config]);
     if (rc != ASP_OK) return rc;
     D1.cta_boff = upload(p, boff, rc);
     if (rc == ASP_OK) D1.cta_auxlo = upload(p, alo, rc);
     if (rc == ASP_OK) D1.cta_auxn = upload(p, an, rc);
-    if (rc == ASP_OK) {
-        // one program per CTA: the units of the whole store (the same for
-        // both configurations), for programs small enough for batches.  The
-        // descriptor keeps the program's own choice (the unit frontier if
-        // it asked for it and the lists exist, no chaining in batches); a
-        // batch's autotuner may switch every program with lists to it
-        if (config == 0) rc = unit_lists(p, H, boff, 1u, BATCH_MAX_UNITS, p->batch_units);
-        if (rc == ASP_OK) {
-            const uint32_t own = D1.frontier;
-            use_unit_lists(D1, p->batch_units);
-            D1.frontier = own >= 2u ? (p->batch_units.built ? 2u : 0u) : own;
-        }
-    }
+    if (D1.frontier >= 2u) D1.frontier = 0u;     // no unit lists for the one-CTA partition
     p->D1[config] = D1;
     p->smem1[config] = base + 4 * D1.view_words;
+    p->smem_base = base;
     return rc;
 }
 
@@ -422,11 +414,12 @@ struct asp_batch {
     std::vector<asp_prog *> progs;
     std::vector<int64_t> caps;
     int64_t max_models_each = 0;
-    int config = 0, grid = 0;
-    bool units = false;                 // the unit-frontier kernels (programs with unit lists use them)
+    int config = 0, kernel = 0, grid = 0;   // kernel: configuration of the instantiation in use
+    bool lists = true;                  // the kernels that follow occurrence lists only
+    bool wide = false;                  // configuration 0 of the lists kernels with 768 threads
     size_t smem = 0;
-    // autotuner trial times per program: configurations 0 and 1 with full
-    // sweeps, then with the unit frontier (0 = not tried, < 0 = cannot run)
+    // autotuner trial times per program: configurations 0 and 1 with
+    // sweeps, then with lists only (0 = not tried, < 0 = cannot run)
     double trial_ns[4] = {0.0, 0.0, 0.0, 0.0};
     uint32_t queued = 0;
     cudaStream_t stream = nullptr;
@@ -452,10 +445,13 @@ std::vector<Dev> batch_descriptors(const asp_batch *b, int config, bool trial = 
     for (size_t i = 0; i < b->progs.size(); i++) {
         asp_prog *p = b->progs[i];
         Dev d = p->D1[config];
-        // the batch's propagation schedule: the unit frontier for programs
-        // with lists, or no unit frontier at all
-        if (b->units && p->batch_units.built) d.frontier = 2u;
-        else if (!b->units && d.frontier >= 2u) d.frontier = 0u;
+        if (b->lists && d.occ) {
+            d.lists = 1u;
+            d.narrow_max = 0xFFFFFFFFu;
+            d.frontier = 0u;
+            d.view_atoms = d.view_words = 0u;
+            d.code_cache = p->smem_base + 4 * (size_t)d.asg_words <= LISTS_SMEM_BUDGET[b->wide && config == 0 ? 2 : config];
+        }
         d.mode = MODE_SOLVE;
         d.max_models = b->max_models_each;
         d.models_cap = b->caps[i];
@@ -478,10 +474,14 @@ std::vector<Dev> batch_descriptors(const asp_batch *b, int config, bool trial = 
 int batch_prepare(asp_batch *b, int config, const std::vector<uint32_t> &order, bool trial = false)
 {
     const size_t n = b->progs.size();
+    const int kernel = b->lists && b->wide && config == 0 ? 2 : config;
     size_t smem = 0;
-    for (asp_prog *p : b->progs) smem = std::max(smem, p->smem1[config]);
+    for (asp_prog *p : b->progs) {
+        const size_t cached = p->smem_base + 4 * (size_t)p->D.asg_words;
+        smem = std::max(smem, !b->lists ? p->smem1[config] : cached <= LISTS_SMEM_BUDGET[kernel] ? cached : p->smem_base);
+    }
     int per_sm = 0;
-    cudaError_t e = batch_configure(config, b->units, smem, &per_sm);
+    cudaError_t e = batch_configure(kernel, b->lists, smem, &per_sm);
     if (e != cudaSuccess) return cuda_fail(e, "batch configuration");
     if (per_sm < 1) return fail(ASP_E_CUDA, "batch kernel cannot be resident");
     const std::vector<Dev> devs = batch_descriptors(b, config, trial);
@@ -492,6 +492,7 @@ int batch_prepare(asp_batch *b, int config, const std::vector<uint32_t> &order, 
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);     // host vectors go out of scope
     if (e != cudaSuccess) return cuda_fail(e, "batch descriptors");
     b->config = config;
+    b->kernel = kernel;
     b->grid = (int)std::min<int64_t>((int64_t)b->progs[0]->n_sms * per_sm, (int64_t)order.size());
     b->smem = smem;
     b->queued = (uint32_t)order.size();
@@ -506,7 +507,7 @@ cudaError_t batch_enqueue(asp_batch *b)
     uint32_t *d_order = (uint32_t *)((char *)b->scratch + sizeof(Dev) * n);
     unsigned int *d_queue = (unsigned int *)((char *)d_order + 4 * n);
     cudaError_t e = cudaMemsetAsync(d_queue, 0, 64, b->stream);
-    if (e == cudaSuccess) e = launch_batch(b->config, b->units, d_devs, d_order, b->queued, d_queue, b->grid, b->smem, b->stream);
+    if (e == cudaSuccess) e = launch_batch(b->kernel, b->lists, d_devs, d_order, b->queued, d_queue, b->grid, b->smem, b->stream);
     return e;
 }
 
@@ -734,11 +735,13 @@ int asp_load_ground(int32_t n_atoms, int32_t n_rules, const int32_t *head,
     if (rc == ASP_OK && D.nv > 0) {
         // occurrence lists by literal, built on the device; the bitmaps and
         // the trail, not in use yet, hold its counters
-        uint32_t *off = (uint32_t *)alloc(((size_t)2 * D.nv + 1) * 4), *occ = (uint32_t *)alloc((size_t)bucket_lits * 4);
+        uint32_t *off = (uint32_t *)alloc(((size_t)2 * D.nv + 1) * 4), *rows = (uint32_t *)alloc((size_t)row_words(D) * 4);
+        Occurrence *occ = (Occurrence *)alloc((size_t)bucket_lits * sizeof(Occurrence));
         if (rc == ASP_OK) {
             D.occ_off = off;
             D.occ = occ;
-            cudaError_t e = launch_occurrences(D, (uint32_t)bucket_lits, off, occ, (uint32_t *)D.deps, D.trail, p->stream);
+            D.rows = rows;
+            cudaError_t e = launch_occurrences(D, (uint32_t)bucket_lits, off, occ, rows, (uint32_t *)D.deps, D.trail, p->stream);
             if (e != cudaSuccess) rc = cuda_fail(e, "occurrence lists");
         }
     }
@@ -1132,13 +1135,8 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
     b->max_models_each = max_models_each;
     b->caps.resize(n);
     for (int32_t i = 0; i < n; i++) b->caps[i] = models_cap ? models_cap[i] : 0;
-    // an explicit configuration keeps the programs' own choice of frontier;
-    // the autotuner tries both where the lists exist
-    bool lists = false;
-    for (int32_t i = 0; i < n; i++) {
-        b->units |= progs[i]->D1[0].frontier == 2u;
-        lists |= progs[i]->batch_units.built;
-    }
+    // an explicit configuration follows the occurrence lists; the autotuner
+    // tries the sweeps too
     auto bail = [&](int rc) { asp_batch_free(b); return rc; };
     // model buffers of every program
     for (int32_t i = 0; i < n; i++) {
@@ -1178,20 +1176,22 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
         const size_t S = std::min<size_t>((size_t)n, 256);
         std::vector<uint32_t> sample(S);
         for (size_t k = 0; k < S; k++) sample[k] = order[k * (size_t)n / S];
-        // schedules: the two kernel configurations, each with full sweeps
-        // and (where the programs have unit lists) with the unit frontier
+        // schedules: the two kernel configurations, each with sweeps and with
+        // lists only; with at most one program per SM the first lists
+        // kernel takes 768 threads
         double best = -1.0;
-        bool best_units = false;
-        for (int u = 0; u < (lists ? 2 : 1); u++) {
-            b->units = u == 1;
+        bool best_lists = true;
+        b->wide = n <= progs[0]->n_sms;
+        for (int u = 0; u < 2; u++) {
+            b->lists = u == 1;
             for (int c = 0; c < 2; c++) {
                 const double t = batch_trial(b, c, sample);
                 b->trial_ns[c + 2 * u] = t;
-                if (t >= 0.0 && (best < 0.0 || t < best)) { best = t; chosen = c; best_units = u == 1; }
+                if (t >= 0.0 && (best < 0.0 || t < best)) { best = t; chosen = c; best_lists = u == 1; }
             }
         }
         if (best < 0.0) return bail(fail(ASP_E_CUDA, "no batch configuration can run"));
-        b->units = best_units;
+        b->lists = best_lists;
     }
     int rc = batch_prepare(b, chosen, order);
     if (rc != ASP_OK) return bail(rc);
@@ -1246,9 +1246,9 @@ int asp_batch_info(const asp_batch *b, int32_t *config, int32_t *block_threads, 
 {
     if (!b) return fail(ASP_E_ARG, "bad argument");
     if (config) *config = b->config;
-    if (block_threads) *block_threads = batch_threads(b->config);
+    if (block_threads) *block_threads = batch_threads(b->kernel);
     if (grid) *grid = b->grid;
-    if (frontier) *frontier = b->units ? ASP_FRONTIER_UNITS : ASP_FRONTIER_FULL;
+    if (frontier) *frontier = b->lists ? ASP_FRONTIER_UNITS : ASP_FRONTIER_FULL;
     if (trial_ns)
         for (int i = 0; i < 4; i++) trial_ns[i] = b->trial_ns[i];
     return ASP_OK;

@@ -49,7 +49,7 @@ constexpr unsigned long long NO_KEY = ~0ull;
 // Dynamic shared memory a program's view may take in the solve kernel (the
 // rest of the 227 KB holds the static arrays: claim list, unit queue, queue
 // of the narrow rounds).
-constexpr size_t SOLVE_SMEM_BUDGET = 196 * 1024;
+constexpr size_t SOLVE_SMEM_BUDGET = 186 * 1024;
 
 // learned heuristic: 16 features -> 64 hidden (ReLU) -> 1, parameters
 // W1[64][16], b1[64], w2[64], b2
@@ -71,7 +71,8 @@ struct Ctl {              // double-buffered control block (phase parity)
     int32_t status, err;
     int32_t conflict;
     uint32_t full;              // the next round sweeps every nogood (else the frontier)
-    uint32_t chased, pad;       // the last claims have been followed by narrow rounds
+    uint32_t chased;            // the last claims have been followed by narrow rounds
+    uint32_t tcom;              // trail entries whose assignments are committed (tc: those in the views)
 };
 
 struct Acc {              // per-phase accumulators, indexed by phase % 4
@@ -122,6 +123,9 @@ struct DevStats {
 // waiting; stall is a flag that nothing sets (the test-only stalled CTA
 // waits on it).
 struct Barrier { unsigned long long count; unsigned int err, stall; };
+
+// An entry of the occurrence lists (see Dev::occ)
+struct __align__(32) Occurrence { uint32_t w[8]; };
 
 struct Dev {
     uint32_t na, J, nv, asg_words;
@@ -178,16 +182,22 @@ struct Dev {
     const float *prior;       // heuristic 3: per-rule score computed at load
     uint32_t *trace;          // [trace_cap][TRACE_WORDS]
     uint32_t trace_cap;
-    // occurrence lists (Algorithm 2's Map): the ids of the bucket nogoods
-    // that hold literal l are occ[occ_off[l] .. occ_off[l + 1]); a phase
-    // with at most narrow_max claims to follow is run by one CTA through them
-    // (narrow_rounds; 0 = no lists)
-    uint32_t narrow_max;
+    // occurrence lists (Algorithm 2's Map): the bucket nogoods that hold
+    // literal l are occ[occ_off[l] .. occ_off[l + 1]): id and the other
+    // literals (PAD_LIT past their number), or, for one of more than eight
+    // literals, id, END_BIT | length and the place of its literals in rows.
+    // A phase with at most narrow_max claims to follow is run by one CTA
+    // through them (narrow_rounds; 0 = no lists).
+    // lists: one CTA solves the program, and its bucket nogoods are checked
+    // through the lists only: no sweep, no view
+    // code_cache: narrow rounds work on a copy of the codes in shared memory
+    uint32_t narrow_max, lists, code_cache, pad4;
     // frontier propagation (Algorithm 2's idea): a round checks only the
     // bucket nogoods of the variables assigned in the previous round; full
     // sweeps after (re)starts and backjumps
     uint32_t frontier;
-    const uint32_t *occ_off, *occ;
+    const uint32_t *occ_off, *rows;
+    const Occurrence *occ;
     // frontier = 2 (frontier by bucket units): the sweep units of the static
     // partition are numbered globally, CTA g's being [cta_ubase[g],
     // cta_ubase[g+1]); occ_unit[occ_uoff[v] .. occ_uoff[v+1]) are the units

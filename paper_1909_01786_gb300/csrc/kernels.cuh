@@ -1,6 +1,6 @@
 // The solver kernels (device code in solver.cuh), instantiated per
-// translation unit: solve.cu and batch.cu without the frontier by units,
-// solve_units.cu and batch_units.cu with it.
+// translation unit: solve.cu without the frontier by units, solve_units.cu
+// with it, batch_kernel.cu per batch configuration.
 #pragma once
 #include "solver.cuh"
 
@@ -14,14 +14,17 @@ __global__ void __launch_bounds__(768, 1) solve_kernel(Dev D)
     extern __shared__ unsigned long long smem_raw[];
     const Smem S = make_smem(D, smem_raw);
     const View V = make_view(D, S.misc + 16, blockIdx.x);
-    solver_loop<false, UNITS>(D, S, V, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, blockIdx.x == 0,
+    solver_loop<false, UNITS, false>(D, S, V, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, blockIdx.x == 0,
                        blockIdx.x == 0 && threadIdx.x == 0, blockIdx.x);
 }
 
 // Batched solving: each CTA takes programs from a queue (the host orders it
-// largest first) and solves each alone, with the whole program's assignment
-// view in its shared memory and a CTA barrier as the phase barrier.
-template <int THREADS, int MIN_BLOCKS, bool UNITS>
+// largest first) and solves each alone, with a CTA barrier as the phase
+// barrier.  LISTS: bucket nogoods are followed through the occurrence lists
+// only (no sweep code, no view: the largest program of a batch of 20k-atom
+// ones took 26 sweeps of 0.9 ms by its one CTA); else sweeps with the whole
+// program's assignment view in shared memory, and lists for few claims.
+template <int THREADS, int MIN_BLOCKS, bool LISTS>
 __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) batch_kernel(const Dev *devs, const uint32_t *order, uint32_t n,
                                                                     unsigned int *queue)
 {
@@ -41,8 +44,6 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) batch_kernel(const Dev *d
         for (uint32_t w = threadIdx.x; w <= D.asg_words; w += blockDim.x) D.asg[w] = 0u;
         for (uint32_t v = threadIdx.x; v < D.nv; v += blockDim.x) D.dl[v] = 0;
         for (uint32_t j = threadIdx.x; j <= D.J; j += blockDim.x) D.act[j] = 0u;
-        if (D.frontier >= 2u)
-            for (uint32_t w = threadIdx.x; w < 2u * D.dirty_words; w += blockDim.x) D.dirty[w] = 0u;
         if (threadIdx.x == 0) {
             Ctl c;
             memset(&c, 0, sizeof(c));
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) batch_kernel(const Dev *d
         cta_sync();
         const Smem S = make_smem(D, smem_raw);
         const View V = make_view(D, S.misc + 16, 0);
-        solver_loop<true, UNITS>(D, S, V, threadIdx.x, blockDim.x, true, threadIdx.x == 0, 0);
+        solver_loop<true, false, LISTS>(D, S, V, threadIdx.x, blockDim.x, true, threadIdx.x == 0, 0);
         cta_sync();
     }
 }

@@ -22,6 +22,7 @@
 
 #include "aspgpu.h"
 #include "device.cuh"
+#include "follow.cuh"
 #include "store.h"
 
 namespace aspgpu {
@@ -158,41 +159,33 @@ __device__ __forceinline__ void na_claim(uint32_t *asg, NaCtl *c, uint32_t l, ui
 }
 
 // Checks the bucket nogoods of the n literals at `from` (each holds since the
-// round before; no other nogood can have become unit or violated), four lanes
-// a literal, groups of four lanes [g, g + ng, ...).  The literal's own fresh
-// bit, of the other parity, is cleared meanwhile.  SHARED: `from` is in shared
-// memory.
+// round before; no other nogood can have become unit or violated): warps w,
+// w + nw, ... take eight literals at a time and share out their lists
+// (warp_lists, quad_check).  A literal's own fresh bit, of the other parity,
+// is cleared meanwhile.  SHARED: `from` is in shared memory.
 template <bool SHARED>
-__device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c, const uint32_t *from, uint32_t n, uint32_t g,
-                                          uint32_t ng, uint32_t fresh, uint32_t stale, const NaList &O)
+__device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c, const uint32_t *from, uint32_t n, uint32_t w,
+                                          uint32_t nw, uint32_t fresh, uint32_t stale, const NaList &O)
 {
-    const uint32_t sub = threadIdx.x & 3u;
-    for (uint32_t i = g; i < n; i += ng) {
-        const uint32_t l0 = SHARED ? from[i] : __ldcg(from + i), y = l0 >> 1;
-        const uint32_t o0 = __ldg(D.occ_off + l0), o1 = __ldg(D.occ_off + l0 + 1u);
-        if (sub == 0u) atomicAnd(asg + (y >> 3), ~(stale << ((y & 7u) * 4u)));
-        for (uint32_t o = o0 + sub; o < o1; o += 4u) {
-            const uint32_t id = __ldg(D.occ + o), L = ((id >> 27) & 15u) + 1u, stride = D.bk_n[L];
-            const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
-            bool sat = false;
-            uint32_t n_un = 0, ul = 0;
-            for (uint32_t q0 = 0; q0 < L && !sat && n_un < 2u; q0 += 4u) {
-                uint32_t l[4], v[4];
-#pragma unroll
-                for (uint32_t q = 0; q < 4u; q++) l[q] = q0 + q < L ? __ldg(base + (size_t)(q0 + q) * stride) : PAD_LIT;
-#pragma unroll
-                for (uint32_t q = 0; q < 4u; q++) v[q] = l[q] != PAD_LIT ? na_val(asg, l[q] >> 1, fresh) : 3u;
-#pragma unroll
-                for (uint32_t q = 0; q < 4u; q++) {
-                    if (l[q] == PAD_LIT) continue;
-                    sat |= v[q] == ((l[q] & 1u) ? V_T : V_F);
-                    if (v[q] == 0u) { n_un++; ul = l[q]; }
-                }
-            }
-            if (sat || n_un > 1u) continue;
-            if (n_un == 0u) na_conflict(c, O);
-            else na_claim(asg, c, ul, fresh, O);
+    const uint32_t lane = threadIdx.x & 31u;
+    const Codes<false> codes{asg};
+    for (uint32_t i0 = w * 8u; i0 < n; i0 += nw * 8u) {
+        const uint32_t i = i0 + lane;
+        uint32_t o0 = 0, count = 0;
+        if (lane < 8u && i < n) {
+            const uint32_t l = SHARED ? from[i] : __ldcg(from + i), y = l >> 1;
+            o0 = __ldg(D.occ_off + l);
+            count = __ldg(D.occ_off + l + 1u) - o0;
+            atomicAnd(asg + (y >> 3), ~(stale << ((y & 7u) * 4u)));
         }
+        warp_lists(o0, count, [&](uint32_t o, uint32_t) {
+            const QuadCheck r = quad_check(D, codes, fresh, o);
+            if ((lane & 3u) == 0u && !r.sat && r.n_un < 2u) {
+                if (r.n_un == 0u) na_conflict(c, O);
+                else na_claim(asg, c, r.ul, fresh, O);
+            }
+            __syncwarp();
+        });
     }
 }
 
@@ -254,7 +247,7 @@ __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D,
                 if (v == 0u) na_claim(asg, c, l, fresh, O);
                 else if (v == ((l & 1u) ? V_F : V_T)) na_conflict(c, O);
             }
-        na_follow<false>(D, asg, c, list + from, to - from, gw * 8u + (lane >> 2), nw * 8u, fresh, stale, O);
+        na_follow<false>(D, asg, c, list + from, to - from, gw, nw, fresh, stale, O);
         // long nogoods: one warp per nogood, lanes over literals
         for (uint32_t i = gw; i < D.n_long; i += nw) {
             __syncwarp();
@@ -305,7 +298,7 @@ __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D,
                 if (threadIdx.x == 0) s_n[(i + 2u) % 3u] = 0u;     // the next round's counter
                 O.s_lit = s_lit[(i + 1u) & 1u];
                 O.s_n = &s_n[(i + 1u) % 3u];
-                na_follow<true>(D, asg, c, s_lit[i & 1u], m, threadIdx.x >> 2, blockDim.x >> 2, 4u << ((r + i) & 1u),
+                na_follow<true>(D, asg, c, s_lit[i & 1u], m, threadIdx.x >> 5, blockDim.x >> 5, 4u << ((r + i) & 1u),
                                 4u << ((r + i + 1u) & 1u), O);
                 na_cta_sync();
                 m = *O.s_n;

@@ -27,6 +27,7 @@
 #include <cstdint>
 
 #include "device.cuh"
+#include "follow.cuh"
 #include "mlp.cuh"
 #include "store.h"
 
@@ -1113,7 +1114,7 @@ __device__ __forceinline__ void frontier_round(const SweepCtx &X, uint32_t fr0, 
         for (uint32_t ob = o0; ob < o1; ob += 32u) {
             const uint32_t o = ob + lane;
             const bool has = o < o1;
-            const uint32_t id = has ? __ldg(D.occ + o) : 0u;
+            const uint32_t id = has ? __ldg(&D.occ[o].w[0]) : 0u;
             const uint32_t L = has ? ((id >> 27) & 15u) + 1u : 0u, k = id & 0x7FFFFFFu;
             const uint32_t *base = has ? D.lits + D.bk_base[L] + k : D.lits;
             const uint32_t n = has ? D.bk_n[L] : 0u;
@@ -1171,7 +1172,7 @@ __device__ __forceinline__ void frontier_round(const SweepCtx &X, uint32_t fr0, 
 
 // The CTA's unit table (s_ubase) from the static partition, once per
 // launch; callers synchronise the CTA before the first sweep.
-__device__ __forceinline__ void unit_table(const Dev &D, uint32_t cta)
+__device__ __forceinline__ void unit_table(const Dev &D, uint32_t cta, bool lists = false)
 {
     if (threadIdx.x != 0) return;
     s_unit = 0u;
@@ -1179,6 +1180,7 @@ __device__ __forceinline__ void unit_table(const Dev &D, uint32_t cta)
     s_nq = 0u;
     s_unit2[0] = 0u;
     s_unit2[1] = 0u;
+    if (lists) return;
     const uint32_t G1 = D.G + 1u;
     uint32_t acc = 0;
     for (uint32_t L = 2; L <= (uint32_t)BUCKET_MAX; L++) {
@@ -1195,14 +1197,12 @@ __device__ __forceinline__ void unit_table(const Dev &D, uint32_t cta)
 // Propagate-and-check over this CTA's ranges of every bucket (full), or
 // over the frontier -- the nogoods of the previous round's assignments
 // (frontier = 1) or the dirty bucket units (frontier = 2), taken from the
-// CTA's queue (DQ = 1, the single-program solver) or straight from the
-// round's dirty bitmap, one 32-unit word per warp (DQ = 2, one program per
-// CTA: every word belongs to the CTA) -- then (grid-wide) the static long
-// nogoods and the learned nogoods.  dbuf: the round's dirty bitmap (DQ = 2).
+// CTA's queue (DQ = 1) -- then (grid-wide) the static long nogoods and the
+// learned nogoods.  DQ = 2: the latter alone (the bucket nogoods are followed
+// through the occurrence lists).
 template <int DQ>
 __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bool full = true,
-                                      uint32_t fr0 = 0u, uint32_t fr1 = 0u, uint32_t pass = 0u,
-                                      uint32_t *dbuf = nullptr)
+                                      uint32_t fr0 = 0u, uint32_t fr1 = 0u, uint32_t pass = 0u)
 {
     SweepCtx X = X0;
     // Listed claims take their trail slots at the end of the sweep, after
@@ -1236,7 +1236,7 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
     uint32_t units = full ? ubase[BUCKET_MAX + 1] : 0u;
     // frontier by units: the queue (or, if it overflowed, every unit of the
     // CTA); the literals and nogoods of the units checked are counted here
-    bool queued = false, count_units = false, words = false;
+    bool queued = false, count_units = false;
     if constexpr (DQ == 1) {
         if (!full && D.frontier >= 2u) {
             const uint32_t nq = s_nq;
@@ -1246,14 +1246,6 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
             X.chain = queued && D.frontier == 3u;
         }
     }
-    if constexpr (DQ == 2) {
-        if (!full && D.frontier >= 2u) {
-            words = true;
-            units = D.dirty_words;
-            count_units = true;
-        }
-    }
-    uint32_t pending = 0u, wbase = 0u;        // DQ = 2: units of the warp's word not yet run
     // frontier = 3: waves of the queue; wave w pops positions [lo, units)
     // with its own counter, and the units claims of wave w queued form wave
     // w + 1 (up to DQ_WAVES waves)
@@ -1267,15 +1259,12 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
     const uint32_t wpc = blockDim.x >> 5, slot = (X.gw % wpc) * (X.nw / wpc) + X.gw / wpc;
     for (uint32_t i = slot; i < nl; i += X.nw) {
         uint32_t id = i < D.n_long ? __ldg(D.long_ids + i) : __ldcg(D.learned_ids + (i - D.n_long));
-        classify_long<(DQ != 0)>(X, id, checks, D.nwatch ? D.nwatch + i : nullptr);
+        classify_long<(DQ == 1)>(X, id, checks, D.nwatch ? D.nwatch + i : nullptr);
     }
     const unsigned long long t1 = wtimer ? globaltimer_ns() : 0ull;
-    for (;;) {
+    for (; DQ != 2;) {
         uint32_t u = 0;
-        if (words && pending) {
-            u = wbase + (uint32_t)__ffs(pending) - 1u;
-            pending &= pending - 1u;
-        } else {
+        {
             if (lane == 0) {
                 if constexpr (DQ == 1) u = X.chain ? lo + atomicAdd(&s_wave[wave], 1u) : atomicAdd(uctr, 1u);
                 else u = atomicAdd(uctr, 1u);
@@ -1304,16 +1293,6 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
             if constexpr (DQ == 1) {
                 if (queued) u = s_dq[u];
             }
-            if constexpr (DQ == 2) {
-                if (words) {
-                    // take the word's bits and clear them in one atomic
-                    uint32_t b = 0u;
-                    if (lane == 0) b = atomicExch(dbuf + u, 0u);
-                    pending = __shfl_sync(FULL_MASK, b, 0);
-                    wbase = u * 32u;
-                    continue;
-                }
-            }
         }
         uint32_t L = 2;
 #pragma unroll
@@ -1322,16 +1301,16 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
         const uint32_t first = ubase[L];
         const uint32_t b0 = s_krange[L][0], b1 = s_krange[L][1];
         const uint32_t k0 = b0 + (u - first) * unit_groups(L) * 32u;
-        if (D.view_mode == VIEW_BYTES) run_unit_view<true, (DQ != 0)>(X, L, k0, b1);
-        else if (D.view_mode == VIEW_PACKED) run_unit_view<false, (DQ != 0)>(X, L, k0, b1);
-        else run_unit<(DQ != 0)>(X, L, k0, b1);
+        if (D.view_mode == VIEW_BYTES) run_unit_view<true, (DQ == 1)>(X, L, k0, b1);
+        else if (D.view_mode == VIEW_PACKED) run_unit_view<false, (DQ == 1)>(X, L, k0, b1);
+        else run_unit<(DQ == 1)>(X, L, k0, b1);
         if (count_units && lane == 0) {
             const uint32_t n = min(b1 - k0, unit_groups(L) * 32u);
             checks += (unsigned long long)L * n;
             uvisits += n;
         }
     }
-    if (!full && D.frontier == 1u) {
+    if (DQ != 2 && !full && D.frontier == 1u && fr0 != fr1) {
         unsigned long long fchecks = 0;           // per lane (classify_long's are per warp)
         frontier_round(X, fr0, fr1, fchecks);
         checks += __reduce_add_sync(FULL_MASK, (unsigned)fchecks);
@@ -1429,6 +1408,7 @@ struct Smem {
     unsigned long long *red;    // [32]
     uint32_t *misc;             // [16]
     const __nv_bfloat16 *mlp;   // [MLP_PARAMS] after the view (heuristic 2)
+    uint32_t *codes;            // [asg_words] after that (code_cache)
 };
 
 // The 16 features of candidate rule j (inputs of the learned heuristic):
@@ -1474,14 +1454,23 @@ __device__ __forceinline__ void decide(const Dev &D, const Smem &S, Acc *acc, ui
                                        uint32_t cdl, uint32_t tend)
 {
     unsigned long long best = 0;
-    for (uint32_t j = gtid; j < D.J; j += nthreads) {
-        uint32_t h = (uint32_t)__ldg(D.rule_head + j);
-        uint32_t b = D.na + 3u * j, t = b + 1u, n = b + 2u;
-        uint32_t ch = nib(__ldcg(D.asg + (h >> 3)), h) & 3u;
-        uint32_t cb = nib(__ldcg(D.asg + (b >> 3)), b) & 3u;
-        uint32_t ct = nib(__ldcg(D.asg + (t >> 3)), t) & 3u;
-        uint32_t cn = nib(__ldcg(D.asg + (n >> 3)), n) & 3u;
-        if (ch == 0u && cb == 0u && ct == V_T && cn != V_F) {
+    // the codes of b, t and n (three neighbours) of four rules load together;
+    // the head's only for the few rules that these let pass
+    for (uint32_t j4 = gtid; j4 < D.J; j4 += 4u * nthreads) {
+        unsigned long long w[4];
+#pragma unroll
+        for (uint32_t q = 0; q < 4u; q++) {
+            const uint32_t b = D.na + 3u * min(j4 + q * nthreads, D.J - 1u);
+            w[q] = (((unsigned long long)__ldcg(D.asg + ((b + 2u) >> 3)) << 32) | __ldcg(D.asg + (b >> 3))) >> ((b & 7u) * 4u);
+        }
+        uint32_t pass = 0;
+#pragma unroll
+        for (uint32_t q = 0; q < 4u; q++)
+            if ((w[q] & 3u) == 0u && ((w[q] >> 4) & 3u) == V_T && ((w[q] >> 8) & 3u) != V_F && j4 + q * nthreads < D.J) pass |= 1u << q;
+        for (; pass; pass &= pass - 1u) {
+            const uint32_t j = j4 + ((uint32_t)__ffs(pass) - 1u) * nthreads;
+            const uint32_t h = (uint32_t)__ldg(D.rule_head + j);
+            if ((nib(__ldcg(D.asg + (h >> 3)), h) & 3u) != 0u) continue;
             unsigned long long key;
             if (D.trace) {
                 // sample about one candidate in eight per decision point
@@ -1541,6 +1530,53 @@ __device__ __forceinline__ void decide(const Dev &D, const Smem &S, Acc *acc, ui
         unsigned long long x = lane < (blockDim.x >> 5) ? S.red[lane] : 0ull;
         x = shfl_max_u64(x);
         if (lane == 0 && x) atomicMax(&acc->dkey, x);
+    }
+}
+
+// One pass of the immediate-consequence operator of the reduct on D.lm;
+// whether this thread added an atom.  The assignment M is total and violates
+// no nogood, so M is a model of the reduct, the least model stays inside M, and
+// a rule can fire only if its body holds in M, which is the value of b_j: the
+// other rules (most) are passed over by that one code, four at a time, and no
+// negative body is read.
+__device__ __forceinline__ bool least_model_pass(const Dev &D, uint32_t gtid, uint32_t nthreads)
+{
+    bool more = false;
+    for (uint32_t j4 = gtid; j4 < D.J; j4 += 4u * nthreads) {
+        uint32_t w[4], pass = 0;
+#pragma unroll
+        for (uint32_t q = 0; q < 4u; q++) {
+            const uint32_t b = D.na + 3u * min(j4 + q * nthreads, D.J - 1u);
+            w[q] = nib(__ldcg(D.asg + (b >> 3)), b) & 3u;
+        }
+#pragma unroll
+        for (uint32_t q = 0; q < 4u; q++)
+            if (w[q] == V_T && j4 + q * nthreads < D.J) pass |= 1u << q;
+        for (; pass; pass &= pass - 1u) {
+            const uint32_t j = j4 + ((uint32_t)__ffs(pass) - 1u) * nthreads, h = (uint32_t)__ldg(D.rule_head + j);
+            if ((__ldcg(D.lm + (h >> 5)) >> (h & 31u)) & 1u) continue;
+            bool ok = true;
+            const uint32_t q1 = __ldg(D.rpos_off + j + 1);
+            for (uint32_t q = __ldg(D.rpos_off + j); ok && q < q1; q++) {
+                const uint32_t a = __ldg(D.rpos + q);
+                ok = (__ldcg(D.lm + (a >> 5)) >> (a & 31u)) & 1u;
+            }
+            if (ok) {
+                atomicOr(D.lm + (h >> 5), 1u << (h & 31u));
+                more = true;
+            }
+        }
+    }
+    return more;
+}
+
+// The smallest true atom outside the least model, into acc->minU.
+__device__ __forceinline__ void unfounded_min(const Dev &D, Acc *acc, uint32_t gtid, uint32_t nthreads)
+{
+    for (uint32_t p = gtid; p < D.na; p += nthreads) {
+        const bool inM = (nib(__ldcg(D.asg + (p >> 3)), p) & 3u) == V_T;
+        const bool inLM = (__ldcg(D.lm + (p >> 5)) >> (p & 31u)) & 1u;
+        if (inM && !inLM) atomicMin(&acc->minU, p);
     }
 }
 
@@ -1979,6 +2015,7 @@ __device__ __forceinline__ Smem make_smem(const Dev &D, unsigned long long *raw)
     S.red = S.bm + D.WW;
     S.misc = reinterpret_cast<uint32_t *>(S.red + 32);
     S.mlp = reinterpret_cast<const __nv_bfloat16 *>(S.misc + 16 + D.view_words);
+    S.codes = S.misc + 16 + D.view_words + (2 * MLP_PARAMS + 15) / 16 * 4;
     return S;
 }
 
@@ -2010,37 +2047,35 @@ __device__ __forceinline__ bool group_sync(const Dev &D, uint32_t gen)
 // ------------------------------------------------------------ narrow rounds
 
 // Claims of the previous and of the current narrow round, cached in shared
-// memory (the trail holds all of them): e = trail entry, reason, and the
-// bounds of its literal's occurrence list unless the list's entries are among
-// the round's items; u = the reason's other variables, where it has at most
-// four literals.
-template <bool BATCH>
+// memory (the trail holds all of them): e = trail entry, reason, and its
+// literal's occurrence list [z, w) unless the list is among the round's items;
+// u = the reason's variables, where it has at most eight literals (the entry's
+// own variable where there are fewer).
+template <uint32_t ENTRIES, uint32_t ITEMS>
 struct NarrowQueue {
-    static constexpr uint32_t N = BATCH ? 48u : 256u, M = BATCH ? 192u : 1024u;
-    uint4 e[2][N];
-    uint32_t u[2][N][3];
-    uint32_t item[2][M];          // positions in D.occ to check
-    uint32_t n[3], m[3], conf[3]; // claims, items and conflict of round i: at (i + 1) % 3
+    static constexpr uint32_t N = ENTRIES, M = ITEMS;
+    uint4 e[2][N], u[2][N][2];
+    uint2 item[2][M];             // position in D.occ, variable it is the list of
+    // of round i, at (i + 1) % 3: claims, items, conflict, lists not among the items
+    uint32_t n[3], m[3], conf[3], rest[3];
 };
 
-// Entry k of a round's queue: its occurrence list goes to the items if it fits.
-template <bool BATCH>
-__device__ __forceinline__ void narrow_queue(NarrowQueue<BATCH> &Q, uint32_t buf, uint32_t slot, uint32_t k, uint32_t entry,
-                                             uint32_t id, uint32_t o0, uint32_t o1)
+// Entry k of a round's queue (k and at: its place among the items, drawn by
+// the caller) by `lanes` lanes, this one the sub-th.
+template <class Queue>
+__device__ __forceinline__ void narrow_queue(Queue &Q, uint32_t buf, uint32_t slot, uint32_t k, uint32_t at, uint32_t entry,
+                                             uint32_t id, uint32_t o0, uint32_t o1, uint32_t sub, uint32_t lanes)
 {
-    if (k >= NarrowQueue<BATCH>::N) return;
     const uint32_t c = o1 - o0;
-    if (c <= 64u && Q.m[slot] + c <= NarrowQueue<BATCH>::M) {
-        const uint32_t at = atomicAdd(&Q.m[slot], c);
-        if (at + c <= NarrowQueue<BATCH>::M) {
-            for (uint32_t j = 0; j < c; j++) Q.item[buf][at + j] = o0 + j;
-            o1 = o0;
-        } else {
-            // the items end before this list: the part inside must not be read
-            for (uint32_t j = at; j < NarrowQueue<BATCH>::M; j++) Q.item[buf][j] = 0xFFFFFFFFu;
-        }
+    const bool fits = k < Queue::N && at <= Queue::M && c <= Queue::M - at;
+    if (fits)
+        for (uint32_t j = sub; j < c; j += lanes) Q.item[buf][at + j] = make_uint2(o0 + j, entry & TRAIL_VAR);
+    else
+        for (uint32_t j = at + sub; j < Queue::M && j - at < c; j += lanes) Q.item[buf][j] = make_uint2(0xFFFFFFFFu, 0u);   // drawn, not used
+    if (sub == 0u) {
+        if (k < Queue::N) Q.e[buf][k] = make_uint4(entry, id, o0, fits ? o0 : o1);
+        if (!fits) Q.rest[slot] = 1u;
     }
-    Q.e[buf][k] = make_uint4(entry, id, o0, o1);
 }
 
 // OR into acc of word w of the bitmaps of variables u[0 .. C) other than x.
@@ -2063,17 +2098,24 @@ __device__ __forceinline__ unsigned long long deps_or(const Dev &D, const uint32
 
 // Dependency bitmap (Section 4.2, mk_dl_bitmap) of variable x, assigned by
 // bucket nogood id, by the 8 lanes `sub` of a group: each takes every eighth
-// word.  others: the nogood's other variables if it has at most four literals
-// and they are known (x where there are fewer), else null.
-__device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t id, const uint32_t *others, uint32_t nw, uint32_t sub)
+// word.  vars: the nogood's variables if it has at most eight literals and
+// they are known, else null.
+__device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t id, const uint4 *vars, uint32_t nw, uint32_t sub)
 {
     const uint32_t L = ((id >> 27) & 15u) + 1u, n = D.bk_n[L];
-    const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
-    if (others && L <= 4u) {
-        const uint32_t u[3] = {others[0], others[1], others[2]};
-        for (uint32_t w = sub; w < nw; w += 8u) D.deps[(size_t)x * D.WW + w] = deps_or<3>(D, u, x, w);
+    if (vars && L <= 8u) {
+        const uint4 v = vars[0];
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+        if (L <= 4u) {
+            for (uint32_t w = sub; w < nw; w += 8u) D.deps[(size_t)x * D.WW + w] = deps_or<4>(D, u, x, w);
+        } else {
+            const uint4 t = vars[1];
+            const uint32_t u2[4] = {t.x, t.y, t.z, t.w};
+            for (uint32_t w = sub; w < nw; w += 8u) D.deps[(size_t)x * D.WW + w] = deps_or<4>(D, u, x, w) | deps_or<4>(D, u2, x, w);
+        }
         return;
     }
+    const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
     for (uint32_t w = sub; w < nw; w += 8u) {
         unsigned long long acc = 0;
         for (uint32_t q0 = 0; q0 < L; q0 += 5u) {
@@ -2089,87 +2131,79 @@ __device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t i
 // What a round counts and where its claims go.
 struct NarrowRound {
     uint32_t cdl, fresh, buf, slot, out;      // buf, slot: of the next round's queue; out: trail index of its first claim
-    unsigned long long checks, visits;
+    uint32_t checks, visits;
 };
 
-__device__ __forceinline__ void narrow_count(const uint32_t l, uint32_t code, uint32_t fresh, bool &sat, uint32_t &n_un, uint32_t &ul)
+// Checks occurrence o (0xFFFFFFFF: none) of a literal of variable y by a quad
+// of lanes; its first lane claims the unit literal's complement, or reports
+// the conflict, and all four write the claim's queue entry.  CACHED: the codes
+// are the CTA's copy, and a claim goes to global memory too, where nothing of
+// the round waits for it.  All 32 lanes call it.
+template <bool CACHED, class Queue>
+__device__ __forceinline__ void narrow_check(const Dev &D, const Codes<CACHED> &codes, Acc *acc, Queue &Q, NarrowRound &R, uint32_t o,
+                                             uint32_t y)
 {
-    if (l == PAD_LIT) return;
-    const uint32_t val = eff_val(nib(code, l >> 1), fresh);
-    sat |= val == ((l & 1u) ? V_T : V_F);
-    if (val == 0u) { n_un++; ul = l; }
-}
-
-// Checks bucket nogood id: claims its unit literal's complement, or reports
-// the conflict.
-template <bool BATCH>
-__device__ __forceinline__ void narrow_check(const Dev &D, Acc *acc, NarrowQueue<BATCH> &Q, NarrowRound &R, uint32_t id)
-{
-    const uint32_t L = ((id >> 27) & 15u) + 1u, n = D.bk_n[L];
-    const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
-    bool sat = false;
-    uint32_t n_un = 0, ul = 0, l[4], c[4];
-#pragma unroll
-    for (uint32_t q = 0; q < 4u; q++) l[q] = q < L ? __ldg(base + (size_t)q * n) : PAD_LIT;
-#pragma unroll
-    for (uint32_t q = 0; q < 4u; q++) c[q] = l[q] != PAD_LIT ? __ldcg(D.asg + (l[q] >> 4)) : 0u;
-    if (L > 4u) {
-        // the rest beside the first four
-        uint32_t l2[BUCKET_MAX - 4], c2[BUCKET_MAX - 4];
-#pragma unroll
-        for (uint32_t q = 4; q < (uint32_t)BUCKET_MAX; q++) l2[q - 4u] = q < L ? __ldg(base + (size_t)q * n) : PAD_LIT;
-#pragma unroll
-        for (uint32_t q = 4; q < (uint32_t)BUCKET_MAX; q++) c2[q - 4u] = l2[q - 4u] != PAD_LIT ? __ldcg(D.asg + (l2[q - 4u] >> 4)) : 0u;
-#pragma unroll
-        for (uint32_t q = 4; q < (uint32_t)BUCKET_MAX; q++) narrow_count(l2[q - 4u], c2[q - 4u], R.fresh, sat, n_un, ul);
-    }
-#pragma unroll
-    for (uint32_t q = 0; q < 4u; q++) narrow_count(l[q], c[q], R.fresh, sat, n_un, ul);
-    R.checks += L;
-    R.visits++;
-    if (sat || n_un > 1u) return;
-    bool clash = n_un == 0u;
-    if (!clash) {
-        const uint32_t x = ul >> 1, valbit = (ul & 1u) ? V_T : V_F;
-        // the claimed literal's list bounds load beside the claim
-        const uint32_t a0 = __ldg(D.occ_off + (ul ^ 1u)), a1 = __ldg(D.occ_off + (ul ^ 1u) + 1u);
-        const int r = claim_var(D.asg, x, valbit, R.fresh);
-        if (r == 0) {
-            const uint32_t entry = x | (valbit == V_F ? TRAIL_F : 0u);
-            D.dl[x] = (int32_t)R.cdl;
-            D.reason[x] = id;
-            const uint32_t k = atomicAdd(&Q.n[R.slot], 1u), pos = R.out + k;
-            narrow_queue<BATCH>(Q, R.buf, R.slot, k, entry, id, a0, a1);
-            if (k < NarrowQueue<BATCH>::N && L <= 4u) {
-                uint32_t j = 0;
-#pragma unroll
-                for (uint32_t q = 0; q < 4u; q++)
-                    if (l[q] != ul && j < 3u) Q.u[R.buf][k][j++] = l[q] != PAD_LIT ? l[q] >> 1 : x;
+    const uint32_t sub = threadIdx.x & 3u, quad = threadIdx.x & 28u;
+    const QuadCheck r = quad_check(D, codes, R.fresh, o);
+    const uint32_t x = r.ul >> 1, valbit = (r.ul & 1u) ? V_T : V_F;
+    uint32_t k = 0xFFFFFFFFu, at = 0u, a0 = 0u, a1 = 0u;
+    if (sub == 0u && o != 0xFFFFFFFFu) {
+        const uint32_t L = ((r.id >> 27) & 15u) + 1u;
+        R.checks += L;
+        R.visits++;
+        if (!r.sat && r.n_un < 2u) {
+            bool clash = r.n_un == 0u;
+            if (!clash) {
+                // the claimed literal's list bounds load beside the claim
+                a0 = __ldg(D.occ_off + (r.ul ^ 1u));
+                a1 = __ldg(D.occ_off + (r.ul ^ 1u) + 1u);
+                const int c = claim_var(codes.w, x, valbit, R.fresh);
+                if (CACHED && c != 1) atomicOr(D.asg + (x >> 3), (valbit | R.fresh) << ((x & 7u) * 4u));
+                if (c == 0) {
+                    k = atomicAdd(&Q.n[R.slot], 1u);
+                    at = atomicAdd(&Q.m[R.slot], a1 - a0);
+                    D.dl[x] = (int32_t)R.cdl;
+                    D.reason[x] = r.id;
+                    const uint32_t pos = R.out + k;
+                    if (pos < D.nv) {
+                        D.trail[pos] = x | (valbit == V_F ? TRAIL_F : 0u);
+                        if (D.tpos) D.tpos[x] = pos;
+                    }
+                }
+                clash = c == 2;
             }
-            if (pos < D.nv) {
-                D.trail[pos] = entry;
-                if (D.tpos) D.tpos[x] = pos;
+            if (clash) {
+                const unsigned long long key = ((unsigned long long)L << 32) | r.id;
+                atomicMin(&acc->ckey, key);
+                atomicMin(&acc->cslot[r.id % 3u], key);
+                Q.conf[R.slot] = 1u;
             }
         }
-        clash = r == 2;
     }
-    if (clash) {
-        const unsigned long long key = ((unsigned long long)L << 32) | id;
-        atomicMin(&acc->ckey, key);
-        atomicMin(&acc->cslot[id % 3u], key);
-        Q.conf[R.slot] = 1u;
+    k = __shfl_sync(FULL_MASK, k, quad);
+    if (!__any_sync(FULL_MASK, k != 0xFFFFFFFFu)) return;
+    at = __shfl_sync(FULL_MASK, at, quad);
+    a0 = __shfl_sync(FULL_MASK, a0, quad);
+    a1 = __shfl_sync(FULL_MASK, a1, quad);
+    if (k != 0xFFFFFFFFu) {
+        narrow_queue(Q, R.buf, R.slot, k, at, x | (valbit == V_F ? TRAIL_F : 0u), r.id, a0, a1, sub, 4u);
+        // the reason's variables for the bitmap, two per lane of the quad
+        if (k < Queue::N && !r.len)
+            reinterpret_cast<uint2 *>(&Q.u[R.buf][k][0])[sub] =
+                make_uint2(sub == 0u ? y : r.l[0] == PAD_LIT ? x : r.l[0] >> 1, r.l[1] == PAD_LIT ? x : r.l[1] >> 1);
     }
+    __syncwarp();
 }
 
 // Bitmaps of entries [i0, i0 + step, ...) of the n in queue buf (trail from qs).
-template <bool BATCH>
-__device__ __forceinline__ void narrow_bitmaps(const Dev &D, const NarrowQueue<BATCH> &Q, uint32_t buf, uint32_t qs, uint32_t n,
-                                               uint32_t i0, uint32_t step, uint32_t nw)
+template <class Queue>
+__device__ __forceinline__ void narrow_bitmaps(const Dev &D, const Queue &Q, uint32_t buf, uint32_t qs, uint32_t n, uint32_t i0,
+                                               uint32_t step, uint32_t nw)
 {
     for (uint32_t i = i0; i < n; i += step) {
-        if (i < NarrowQueue<BATCH>::N) {
+        if (i < Queue::N) {
             const uint4 c = Q.e[buf][i];
-            narrow_deps(D, c.x & TRAIL_VAR, c.y, Q.u[buf][i], nw, threadIdx.x & 7u);
+            narrow_deps(D, c.x & TRAIL_VAR, c.y, &Q.u[buf][i][0], nw, threadIdx.x & 7u);
         } else {
             const uint32_t x = __ldcg(D.trail + qs + i) & TRAIL_VAR;
             narrow_deps(D, x, __ldcg(D.reason + x), nullptr, nw, threadIdx.x & 7u);
@@ -2190,72 +2224,91 @@ __device__ __forceinline__ void narrow_bitmaps(const Dev &D, const NarrowQueue<B
 //
 // Why: a search round assigns a few dozen variables (62 on average in the
 // 100k-atom program), and a sweep round costs its chain of barriers and loads
-// (15 us there on 152 CTAs) whatever its claims.  Here a round is bound by
-// four dependent loads (list entry, literals, codes, claim) and a CTA barrier.
-// A claim puts its list's positions into the next round's items, so a lane
-// checks one nogood whatever the lists' lengths; a third of the warps check
-// while the others compute the bitmaps of the round's entries (nothing in the
+// (15 us there on 152 CTAs) whatever its claims.  Here a round is bound by a
+// chain of list entry, codes, claim (two loads and an atomic from L2, about
+// 0.6 us) and the instructions around it.  A claim puts its list's positions
+// into the next round's items, so a quad of lanes checks one nogood whatever
+// the lists' lengths (a program whose codes fit keeps a copy of them in shared
+// memory, which halves the chain); two thirds of the warps check while the others compute the bitmaps of the round's entries (nothing in the
 // round reads those), from the variables that the claim left in shared memory.
 // The fresh bits alternate by round exactly as in sweeps: an entry's bit is
 // cleared while its round runs, when only the other parity's bit hides a
 // variable.  Returns the number of rounds; *n_claims is the number of claims,
-// *wide whether some are still to be checked.
-template <bool BATCH>
-__device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, Acc *acc, uint32_t cdl, uint32_t round, uint32_t first,
-                                                  uint32_t tend, uint32_t tbase, uint32_t *n_claims, bool *wide)
+// *n_left that of the last ones, still to be checked.
+template <bool CACHED, class Queue>
+__device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache, Queue &Q, Acc *acc, uint32_t cdl, uint32_t round,
+                                                  uint32_t first, uint32_t tend, uint32_t tbase, uint32_t *n_claims, uint32_t *n_left)
 {
-    __shared__ NarrowQueue<BATCH> Q;
-    constexpr uint32_t N = NarrowQueue<BATCH>::N, M = NarrowQueue<BATCH>::M;
+    constexpr uint32_t N = Queue::N, M = Queue::M;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarp = blockDim.x >> 5;
     const uint32_t nw = cdl > 1u ? deps_words(D, cdl) : 0u;
+    const Codes<CACHED> codes{CACHED ? cache : D.asg};
     // warps [0, wa) check nogoods, the others compute bitmaps; all do both
     // when there is one warp, and all check at the root level
     const bool split = nw && nwarp > 1u;
-    const uint32_t wa = split ? (nwarp + 1u) / 3u : nwarp;
-    if (tid == 0) Q.n[0] = Q.n[1] = Q.n[2] = Q.m[0] = Q.m[1] = Q.m[2] = Q.conf[0] = Q.conf[1] = Q.conf[2] = 0u;
+    const uint32_t wa = split ? max(1u, nwarp * 2u / 3u) : nwarp;
+    if (tid < 3u) Q.n[tid] = Q.m[tid] = Q.conf[tid] = Q.rest[tid] = 0u;
+    if (CACHED)
+        for (uint32_t w = tid; w < D.asg_words; w += blockDim.x) cache[w] = __ldcg(D.asg + w);
     cta_sync();
+    if (tid == 0 && tend - first > N) Q.rest[0] = 1u;
     for (uint32_t i = tid; i < min(tend - first, N); i += blockDim.x) {
         const uint32_t e = __ldcg(D.trail + first + i), l = mk_lit(e & TRAIL_VAR, (e & TRAIL_F) != 0u);
         if ((l >> 1) >= D.nv) { atomicExch(&D.bar->err, 2u); Q.e[0][i] = make_uint4(0u, 0u, 0u, 0u); continue; }   // corrupt trail
-        narrow_queue<BATCH>(Q, 0u, 0u, i, e, 0u, __ldg(D.occ_off + l), __ldg(D.occ_off + l + 1u));
+        const uint32_t a0 = __ldg(D.occ_off + l), a1 = __ldg(D.occ_off + l + 1u);
+        narrow_queue(Q, 0u, 0u, i, atomicAdd(&Q.m[0], a1 - a0), e, 0u, a0, a1, 0u, 1u);
     }
     cta_sync();
     uint32_t qs = first, qn = tend - first, it = 0;
-    NarrowRound R{cdl, 0u, 0u, 0u, tbase, 0ull, 0ull};
+    NarrowRound R{cdl, 0u, 0u, 0u, tbase, 0u, 0u};
     for (bool done = false; !done;) {
-        const uint32_t cur = it & 1u, stale = 4u << ((round + 1u) & 1u), items = min(Q.m[it % 3u], M);
+        const uint32_t cur = it & 1u, stale = 4u << ((round + 1u) & 1u), items = min(Q.m[it % 3u], M), rest = Q.rest[it % 3u];
         R.fresh = 4u << (round & 1u);
         R.buf = cur ^ 1u;
         R.slot = (it + 1u) % 3u;
         // cleared for the next round's claims; last read two barriers ago
-        if (tid == 0) Q.n[(it + 2u) % 3u] = Q.m[(it + 2u) % 3u] = Q.conf[(it + 2u) % 3u] = 0u;
+        if (tid == 0) Q.n[(it + 2u) % 3u] = Q.m[(it + 2u) % 3u] = Q.conf[(it + 2u) % 3u] = Q.rest[(it + 2u) % 3u] = 0u;
         if (warp < wa) {
-            for (uint32_t i = tid; i < items; i += wa * 32u) {
-                const uint32_t o = Q.item[cur][i];
-                if (o != 0xFFFFFFFFu) narrow_check<BATCH>(D, acc, Q, R, __ldg(D.occ + o));
+            for (uint32_t i0 = warp * 8u; i0 < items; i0 += wa * 8u) {
+                const uint32_t i = i0 + (lane >> 2);
+                const uint2 t = i < items ? Q.item[cur][i] : make_uint2(0xFFFFFFFFu, 0u);
+                narrow_check(D, codes, acc, Q, R, t.x, t.y);
             }
-            for (uint32_t i = warp * 8u + (lane >> 2); i < qn; i += wa * 8u) {
-                uint32_t e, o0, o1;
-                if (i < N) {
-                    const uint4 c = Q.e[cur][i];
-                    e = c.x; o0 = c.z; o1 = c.w;
-                } else {
-                    e = __ldcg(D.trail + qs + i);
-                    const uint32_t l = mk_lit(e & TRAIL_VAR, (e & TRAIL_F) != 0u);
-                    if ((l >> 1) >= D.nv) { atomicExch(&D.bar->err, 2u); continue; }
-                    o0 = __ldg(D.occ_off + l); o1 = __ldg(D.occ_off + l + 1u);
+            // lists past the items, and entries past the queue
+            for (uint32_t i0 = warp * 8u; rest && i0 < qn; i0 += wa * 8u) {
+                const uint32_t i = i0 + lane;
+                uint32_t y = 0, o = 0, o1 = 0;
+                if (lane < 8u && i < qn) {
+                    if (i < N) {
+                        const uint4 c = Q.e[cur][i];
+                        y = c.x & TRAIL_VAR; o = c.z; o1 = c.w;
+                    } else {
+                        const uint32_t e = __ldcg(D.trail + qs + i), l = mk_lit(e & TRAIL_VAR, (e & TRAIL_F) != 0u);
+                        y = e & TRAIL_VAR;
+                        if (y >= D.nv) { atomicExch(&D.bar->err, 2u); y = 0u; }
+                        else { o = __ldg(D.occ_off + l); o1 = __ldg(D.occ_off + l + 1u); }
+                    }
                 }
-                const uint32_t y = e & TRAIL_VAR;
-                if ((lane & 3u) == 0u) atomicAnd(D.asg + (y >> 3), ~(stale << ((y & 7u) * 4u)));
-                for (uint32_t o = o0 + (lane & 3u); o < o1; o += 4u) narrow_check<BATCH>(D, acc, Q, R, __ldg(D.occ + o));
+                warp_lists(o, o1 - o, [&](uint32_t oc, uint32_t li) {
+                    narrow_check(D, codes, acc, Q, R, oc, __shfl_sync(FULL_MASK, y, li));
+                });
             }
+        }
+        // the entries' fresh bits, from the last warps backwards (they
+        // have the fewest items)
+        for (uint32_t i = blockDim.x - 1u - tid; i < qn; i += blockDim.x) {
+            const uint32_t y = (i < N ? Q.e[cur][i].x : __ldcg(D.trail + qs + i)) & TRAIL_VAR;
+            if (y >= D.nv) continue;
+            const uint32_t clear = ~(stale << ((y & 7u) * 4u));
+            if (CACHED) atomicAnd(cache + (y >> 3), clear);
+            atomicAnd(D.asg + (y >> 3), clear);
         }
         // bitmaps of this round's entries (the first round's have theirs)
         if (nw && it > 0u && (!split || warp >= wa))
-            narrow_bitmaps<BATCH>(D, Q, cur, qs, qn, (split ? warp - wa : warp) * 4u + (lane >> 3), (split ? nwarp - wa : nwarp) * 4u, nw);
+            narrow_bitmaps(D, Q, cur, qs, qn, (split ? warp - wa : warp) * 4u + (lane >> 3), (split ? nwarp - wa : nwarp) * 4u, nw);
         cta_sync();
         const uint32_t n_new = Q.n[R.slot];
-        done = n_new == 0u || Q.conf[R.slot] || n_new > D.narrow_max || R.out + n_new >= D.nv;
+        done = n_new == 0u || Q.conf[R.slot] || n_new > D.narrow_max || R.out + n_new > D.nv;
         qs = R.out;
         qn = n_new;
         R.out += n_new;
@@ -2263,15 +2316,15 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, Acc *acc, uint32
         it++;
     }
     // the last claims' bitmaps, by every warp
-    if (nw) narrow_bitmaps<BATCH>(D, Q, it & 1u, qs, qn, warp * 4u + (lane >> 3), nwarp * 4u, nw);
+    if (nw) narrow_bitmaps(D, Q, it & 1u, qs, qn, warp * 4u + (lane >> 3), nwarp * 4u, nw);
     cta_sync();
-    const uint32_t c32 = __reduce_add_sync(FULL_MASK, (unsigned)R.checks), v32 = __reduce_add_sync(FULL_MASK, (unsigned)R.visits);
+    const uint32_t c32 = __reduce_add_sync(FULL_MASK, R.checks), v32 = __reduce_add_sync(FULL_MASK, R.visits);
     if (lane == 0 && v32) {
         atomicAdd(&acc->checks, (unsigned long long)c32);
         atomicAdd(&acc->visits, (unsigned long long)v32);
     }
     *n_claims = R.out - tbase;
-    *wide = qn != 0u;
+    *n_left = qn;
     return it;
 }
 
@@ -2296,13 +2349,14 @@ __device__ __forceinline__ void injected_stall(const Dev &D)
 // next control block.  UNITS: compiled with the frontier by units (used by
 // programs with frontier = 2; the kernels without it keep the sweeps free of
 // the unit marks).
-template <bool BATCH, bool UNITS>
+template <bool BATCH, bool UNITS, bool LISTS>
 __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const View &V, uint32_t rank,
                                             uint32_t size, bool cta0, bool leader, uint32_t cta)
 {
     __shared__ Ctl sC;
     __shared__ Acc sA;
     const uint32_t gtid = rank, nthreads = size;
+    const bool lists = LISTS || D.lists;
     // leader-only counters (shared memory, not registers of every thread),
     // written to the stats when the search ends
     __shared__ unsigned long long t_start, t_phase, n_conf, n_phases, ns_bar, ns_sw, ns_an, ns_de, ns_st;
@@ -2325,8 +2379,8 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
         for (uint32_t i = threadIdx.x; i < (uint32_t)MLP_PARAMS; i += blockDim.x) w[i] = __ldg(D.mlp + i);
     }
     cta_sync();
-    view_reload(D, V, 4u << (sC.round & 1u));
-    unit_table(D, cta);
+    if (!lists) view_reload(D, V, 4u << (sC.round & 1u));
+    unit_table(D, cta, lists);
     if constexpr (UNITS && !BATCH) {
         // frontier by units: the CTA's unit range, no unit queued yet
         if (threadIdx.x == 0 && D.frontier >= 2u) {
@@ -2383,7 +2437,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 }
             }
             if (leader) {
-                N.op = OP_ROUND; N.round = C.round + 1u; N.tb = tend; N.tc = C.tc; N.clean = 0; N.full = 1;
+                N.op = OP_ROUND; N.round = C.round + 1u; N.tb = tend; N.tc = C.tc; N.tcom = C.tc; N.clean = 0; N.full = 1;
             }
             break;
         }
@@ -2470,7 +2524,9 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 }
                 break;
             }
-            const bool quiet = A.nclaim == 0u || C.chased;   // no claim is left to follow
+            // without sweeps the caller's partial assignment is followed too
+            const bool input = lists && D.mode == MODE_PROPAGATE && C.round == 1u;
+            const bool quiet = (A.nclaim == 0u || C.chased) && !input;   // no assignment is left to follow
             if (quiet && C.clean) {
                 // fixpoint
                 if (leader) N.tb = tend;
@@ -2488,8 +2544,8 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 if (leader) N.op = OP_APPLY;
                 break;
             }
-            if (!quiet && !C.full && A.nclaim <= D.narrow_max) {
-                nar = true; sw_cdl = C.cdl; sw_fr0 = C.tb; sw_fr1 = sw_tbase = tend;
+            if (!quiet && (lists || (!C.full && A.nclaim <= D.narrow_max))) {
+                nar = true; sw_cdl = C.cdl; sw_fr0 = input ? 0u : C.tb; sw_fr1 = sw_tbase = tend;
                 if (leader) atomicAdd(&D.stats->props, (unsigned long long)A.nclaim);
                 break;
             }
@@ -2504,7 +2560,9 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 if (v >= D.nv) { atomicExch(&D.bar->err, 2u); continue; }   // corrupt trail: stop with an error
                 atomicAnd(D.asg + (v >> 3), ~(fresh_prev << ((v & 7u) * 4u)));
             }
-            if (tend - C.tc > 4096u) {
+            if (lists) {
+                // no view
+            } else if (tend - C.tc > 4096u) {
                 view_reload(D, V, fresh_cur);
             } else {
                 for (uint32_t i = C.tc + threadIdx.x; i < tend; i += blockDim.x) {
@@ -2514,10 +2572,10 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             }
             cta_sync();
             sw = true; sw_cdl = C.cdl; sw_tbase = tend;
-            sw_full = C.full != 0u || D.frontier == 0u || (!UNITS && D.frontier >= 2u);
+            sw_full = !lists && (C.full != 0u || D.frontier == 0u || (!UNITS && D.frontier >= 2u));
             sw_fr0 = C.chased ? tend : C.tb; sw_fr1 = tend;
             if (leader) {
-                N.op = OP_ROUND; N.round = C.round + 1u; N.tc = tend; N.tb = tend; N.clean = 1; N.full = 0; N.chased = 0;
+                N.op = OP_ROUND; N.round = C.round + 1u; N.tc = tend; N.tb = tend; N.tcom = tend; N.clean = 1; N.full = 0; N.chased = 0;
                 atomicAdd(&D.stats->rounds, 1ull);
                 atomicAdd(&D.stats->props, (unsigned long long)A.nclaim);
                 if (sw_full) atomicAdd(&D.stats->checks, D.static_checks);
@@ -2544,7 +2602,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 if (leader) {
                     // (frontier by units: completion claims mark no units, so
                     // the next round sweeps everything)
-                    N.op = OP_ROUND; N.round = C.round + 1u; N.tb = tend; N.clean = 0; N.chased = 0;
+                    N.op = OP_ROUND; N.round = C.round + 1u; N.tb = tend; N.tcom = tend; N.clean = 0; N.chased = 0;
                     N.full = D.frontier >= 2u ? 1u : 0u;
                     atomicAdd(&D.stats->completions, 1ull);
                 }
@@ -2572,7 +2630,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 __threadfence();
                 atomicOr(D.asg + (bv >> 3), V_T << ((bv & 7u) * 4u));
             }
-            if (D.narrow_max) {
+            if (lists || D.narrow_max) {
                 // the decision's consequences by narrow rounds: the store is at
                 // a fixpoint, so only the decision's nogoods can change it
                 nar = true; sw_cdl = L; sw_fr0 = tend; sw_fr1 = sw_tbase = tend + 1u;
@@ -2585,17 +2643,8 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             }
             if (threadIdx.x == 0) view_set(V, bv, V_T);
             if (UNITS && D.frontier >= 2u) {
-                uint32_t *buf = D.dirty + (C.round & 1u) * D.dirty_words;
                 if constexpr (UNITS && !BATCH) {
-                    build_unit_queue(D, cta, buf, bv);
-                } else if (threadIdx.x < 32u) {
-                    // one program per CTA: the decision variable's units go
-                    // into the bitmap the sweep takes its words from
-                    const uint32_t o0 = __ldg(D.occ_uoff + bv), o1 = __ldg(D.occ_uoff + bv + 1u);
-                    for (uint32_t o = o0 + threadIdx.x; o < o1; o += 32u) {
-                        const uint32_t u = __ldg(D.occ_unit + o);
-                        atomicOr(buf + (u >> 5), 1u << (u & 31u));
-                    }
+                    build_unit_queue(D, cta, D.dirty + (C.round & 1u) * D.dirty_words, bv);
                 }
             }
             cta_sync();
@@ -2603,7 +2652,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             sw_full = D.frontier == 0u || (!UNITS && D.frontier >= 2u);
             if (leader) {
                 N.op = OP_ROUND; N.cdl = L; N.round = C.round + 1u; N.tc = tend + 1u; N.tb = tend + 1u;
-                N.clean = 0; N.full = 0; N.chased = 0;
+                N.tcom = tend + 1u; N.clean = 0; N.full = 0; N.chased = 0;
                 atomicAdd(&D.stats->decisions, 1ull);
                 atomicAdd(&D.stats->rounds, 1ull);
                 if (sw_full) atomicAdd(&D.stats->checks, D.static_checks);
@@ -2621,10 +2670,11 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 atomicAnd(D.asg + (v >> 3), ~(0xFu << ((v & 7u) * 4u)));
                 D.dl[v] = 0;
             }
-            for (uint32_t i = newend + threadIdx.x; i < tend; i += blockDim.x)
-                view_clear(V, __ldcg(D.trail + i) & TRAIL_VAR);
+            if (!lists)
+                for (uint32_t i = newend + threadIdx.x; i < tend; i += blockDim.x)
+                    view_clear(V, __ldcg(D.trail + i) & TRAIL_VAR);
             if (leader) {
-                N.op = OP_ROUND; N.cdl = C.target; N.tc = min(C.tc, newend); N.tb = newend; N.clean = 0; N.full = 1; N.chased = 0;
+                N.op = OP_ROUND; N.cdl = C.target; N.tc = min(C.tc, newend); N.tb = newend; N.tcom = newend; N.clean = 0; N.full = 1; N.chased = 0;
             }
             break;
         }
@@ -2633,39 +2683,30 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             const uint32_t words = (D.na + 31u) >> 5;
             for (uint32_t w = gtid; w < words; w += nthreads) D.lm[w] = 0u;
             if (leader) { N.op = OP_STAB_ITER; N.stab_first = 1; N.tb = tend; }
+            if (BATCH || gridDim.x == 1u) {
+                // one CTA: every pass in this phase
+                __shared__ uint32_t s_more;
+                do {
+                    cta_sync();
+                    if (threadIdx.x == 0) s_more = 0u;
+                    cta_sync();
+                    if (least_model_pass(D, gtid, nthreads)) s_more = 1u;
+                    cta_sync();
+                } while (s_more);
+                unfounded_min(D, acc, gtid, nthreads);
+                if (leader) N.op = OP_STAB_RESULT;
+            }
             break;
         }
         case OP_STAB_ITER: {
             kind = 3;
             if (!C.stab_first && A.flag == 0u) {
                 // least model reached: look for true atoms outside it
-                for (uint32_t p = gtid; p < D.na; p += nthreads) {
-                    bool inM = (nib(__ldcg(D.asg + (p >> 3)), p) & 3u) == V_T;
-                    bool inLM = (__ldcg(D.lm + (p >> 5)) >> (p & 31u)) & 1u;
-                    if (inM && !inLM) atomicMin(&acc->minU, p);
-                }
+                unfounded_min(D, acc, gtid, nthreads);
                 if (leader) N.op = OP_STAB_RESULT;
                 break;
             }
-            // one pass of T over the reduct: rules whose negative body avoids
-            // M and whose positive body lies in the current set
-            for (uint32_t j = gtid; j < D.J; j += nthreads) {
-                uint32_t h = (uint32_t)__ldg(D.rule_head + j);
-                if ((__ldcg(D.lm + (h >> 5)) >> (h & 31u)) & 1u) continue;
-                bool ok = true;
-                for (uint32_t q = __ldg(D.rneg_off + j); ok && q < __ldg(D.rneg_off + j + 1); q++) {
-                    uint32_t a = __ldg(D.rneg + q);
-                    if ((nib(__ldcg(D.asg + (a >> 3)), a) & 3u) == V_T) ok = false;
-                }
-                for (uint32_t q = __ldg(D.rpos_off + j); ok && q < __ldg(D.rpos_off + j + 1); q++) {
-                    uint32_t a = __ldg(D.rpos + q);
-                    if (!((__ldcg(D.lm + (a >> 5)) >> (a & 31u)) & 1u)) ok = false;
-                }
-                if (ok) {
-                    atomicOr(D.lm + (h >> 5), 1u << (h & 31u));
-                    atomicOr(&acc->flag, 1u);
-                }
-            }
+            if (least_model_pass(D, gtid, nthreads)) atomicOr(&acc->flag, 1u);
             if (leader) { N.op = OP_STAB_ITER; N.stab_first = 0; }
             break;
         }
@@ -2806,23 +2847,27 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             // at the next sweep.  A full-sweep program confirms the fixpoint
             // with a sweep; so does a program with long or learned nogoods,
             // which no list holds
+            // (several CTAs share an SM in batches, with their views beside it)
+            constexpr uint32_t QN = !BATCH ? 192u : LISTS ? 96u : 24u;
+            __shared__ NarrowQueue<QN, 4u * QN> Q;
             cta_sync();
-            uint32_t n = 0;
-            bool wide = false;
-            const uint32_t its = narrow_rounds<BATCH>(D, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &wide);
+            uint32_t n = 0, left = 0;
+            const uint32_t its = D.code_cache
+                ? narrow_rounds<true>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left)
+                : narrow_rounds<false>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left);
             if (leader) {
-                N.op = OP_ROUND; N.round = C.round + its; N.tb = sw_tbase;
-                N.chased = !wide; N.full = wide; N.clean = D.frontier != 0u && D.n_long + C.n_learned == 0u;
+                N.op = OP_ROUND; N.round = C.round + its; N.tb = sw_tbase; N.tcom = sw_tbase + n - left;
+                N.chased = left == 0u; N.full = left != 0u;
+                N.clean = (lists || D.frontier != 0u) && D.n_long + C.n_learned == 0u;
                 acc->nclaim = n;
                 atomicAdd(&D.stats->rounds, (unsigned long long)its);
             }
         }
         if (sw) {
             const unsigned long long ts = threadIdx.x == 0 ? globaltimer_ns() : 0ull;
-            SweepCtx X{&D, V, fresh_cur, sw_cdl, sw_tbase, acc, true, true, sw_dec, cta, rank >> 5, size >> 5};
-            if (UNITS && D.frontier >= 2u) X.dmark = D.dirty + ((C.round + 1u) & 1u) * D.dirty_words;
-            sweep<UNITS ? (BATCH ? 2 : 1) : 0>(X, C.n_learned, sw_full, sw_fr0, sw_fr1, 0u,
-                                               D.frontier >= 2u ? D.dirty + (C.round & 1u) * D.dirty_words : nullptr);
+            SweepCtx X{&D, V, fresh_cur, sw_cdl, sw_tbase, acc, true, !lists, sw_dec, cta, rank >> 5, size >> 5};
+            if (UNITS && !lists && D.frontier >= 2u) X.dmark = D.dirty + ((C.round + 1u) & 1u) * D.dirty_words;
+            sweep<LISTS ? 2 : UNITS ? 1 : 0>(X, C.n_learned, sw_full, sw_fr0, sw_fr1);
             if (threadIdx.x == 0) atomicMax(&acc->tsweep, globaltimer_ns() - ts);
         }
 
@@ -2849,7 +2894,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             else if (kind == 2) ns_de += dt;
             else ns_st += dt;
             n_phases++;
-            __threadfence();
+            if (!BATCH && gridDim.x > 1u) __threadfence();
         }
         const unsigned long long tb0 = threadIdx.x == 0 ? globaltimer_ns() : 0ull;
         if (threadIdx.x == 0) atomicMax(&acc->tbusy, tb0 - t_cta0);
@@ -2860,7 +2905,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
     }
     if (leader) {
         const Ctl F = sC;
-        D.stats->pad = F.tc;
+        D.stats->pad = F.tcom;
         D.stats->ns_total = globaltimer_ns() - t_start;
         D.stats->ns_sweep = ns_sw;
         D.stats->ns_analysis = ns_an;

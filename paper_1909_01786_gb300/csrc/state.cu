@@ -130,15 +130,6 @@ __global__ void __launch_bounds__(256) closure_kernel(Dev D, int8_t *closure)
 // literals (and words of the scan) of one block of the occurrence kernels
 constexpr uint32_t OCC_BLOCK = 2048;
 
-// Bucket nogood id of word i of the literal array.
-__device__ __forceinline__ uint32_t word_nogood(const Dev &D, uint32_t i)
-{
-    uint32_t L = 2;
-    for (uint32_t q = 3; q <= (uint32_t)BUCKET_MAX; q++)
-        if (i >= D.bk_base[q]) L = q;
-    return bucket_nogood_id(L, (i - D.bk_base[L]) % D.bk_n[L]);
-}
-
 __global__ void __launch_bounds__(256) occ_count_kernel(Dev D, uint32_t n_lits, uint32_t *count)
 {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_lits; i += gridDim.x * blockDim.x)
@@ -207,23 +198,58 @@ __global__ void __launch_bounds__(256) occ_offsets_kernel(const uint32_t *count,
     }
 }
 
-__global__ void __launch_bounds__(256) occ_fill_kernel(Dev D, uint32_t n_lits, const uint32_t *off, uint32_t *count, uint32_t *occ)
+// First word of bucket L's literals in the rows of the nogoods of more than
+// eight literals.
+struct RowBase { uint32_t at[BUCKET_MAX + 1]; };
+
+__global__ void __launch_bounds__(256) occ_fill_kernel(Dev D, uint32_t n_lits, RowBase R, const uint32_t *off, uint32_t *count,
+                                                       Occurrence *occ, uint32_t *rows)
 {
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_lits; i += gridDim.x * blockDim.x) {
+        uint32_t L = 2;
+        for (uint32_t q = 3; q <= (uint32_t)BUCKET_MAX; q++)
+            if (i >= D.bk_base[q]) L = q;
+        const uint32_t n = D.bk_n[L], r = i - D.bk_base[L], q = r / n, k = r % n;
+        const uint32_t *base = D.lits + D.bk_base[L] + k;
         const uint32_t l = __ldg(D.lits + i);
-        occ[off[l] + atomicSub(count + l, 1u) - 1u] = word_nogood(D, i);
+        uint32_t w[8] = {bucket_nogood_id(L, k), PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT};
+        if (L <= 8u) {
+#pragma unroll
+            for (uint32_t j = 1; j < 8u; j++)
+                if (j < L) w[j] = __ldg(base + (size_t)(q + j < L ? q + j : q + j - L) * n);
+        } else {
+            w[1] = END_BIT | L;
+            w[2] = R.at[L] + k * L;
+            rows[w[2] + q] = l;
+        }
+        uint4 *e = reinterpret_cast<uint4 *>(occ + (off[l] + atomicSub(count + l, 1u) - 1u));
+        e[0] = make_uint4(w[0], w[1], w[2], w[3]);
+        e[1] = make_uint4(w[4], w[5], w[6], w[7]);
     }
 }
 
 }  // namespace
 
-// For every literal l the ids of the bucket nogoods that hold it: occ[off[l]
-// .. off[l + 1]), off of 2 nv + 1 words, n_lits ids.  count: 2 nv words,
-// sums: one word per 2048 of them.  (On the host this was a random pass over
-// the store, 0.1 s for 8M literals.)
-cudaError_t launch_occurrences(const Dev &D, uint32_t n_lits, uint32_t *off, uint32_t *occ, uint32_t *count,
+// Words of the rows of the bucket nogoods of more than eight literals.
+uint32_t row_words(const Dev &D)
+{
+    uint32_t w = 0;
+    for (uint32_t L = 9; L <= (uint32_t)BUCKET_MAX; L++) w += L * D.bk_n[L];
+    return w;
+}
+
+// The occurrence lists (device.cuh): off of 2 nv + 1 words, n_lits entries,
+// row_words(D) words of rows.  count: 2 nv words, sums: one word per 2048 of
+// them.  (On the host this was a random pass over the store, 0.1 s for 8M
+// literals.)
+cudaError_t launch_occurrences(const Dev &D, uint32_t n_lits, uint32_t *off, Occurrence *occ, uint32_t *rows, uint32_t *count,
                                uint32_t *sums, cudaStream_t st)
 {
+    RowBase R{};
+    for (uint32_t L = 9, w = 0; L <= (uint32_t)BUCKET_MAX; L++) {
+        R.at[L] = w;
+        w += L * D.bk_n[L];
+    }
     const uint32_t n = 2u * D.nv, blocks = (n + OCC_BLOCK - 1u) / OCC_BLOCK;
     const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>((n_lits + 255u) / 256u, 4864u));
     cudaError_t e = cudaMemsetAsync(count, 0, (size_t)n * 4, st);
@@ -232,7 +258,7 @@ cudaError_t launch_occurrences(const Dev &D, uint32_t n_lits, uint32_t *off, uin
     occ_sums_kernel<<<blocks, 256, 0, st>>>(count, n, sums);
     occ_base_kernel<<<1, 256, 0, st>>>(sums, blocks);
     occ_offsets_kernel<<<blocks, 256, 0, st>>>(count, n, sums, off);
-    occ_fill_kernel<<<grid, 256, 0, st>>>(D, n_lits, off, count, occ);
+    occ_fill_kernel<<<grid, 256, 0, st>>>(D, n_lits, R, off, count, occ, rows);
     return cudaGetLastError();
 }
 
