@@ -16,7 +16,7 @@ INCLUDE = os.path.join(ROOT, "include")
 # (source, extra flags, object name): batch_kernel.cu is compiled once per
 # batch configuration and propagation schedule, so the five instantiations of
 # the batch kernel compile in parallel
-SOURCES = [("solve.cu", [], "solve"), ("solve_units.cu", [], "solve_units"), ("batch.cu", [], "batch")]
+SOURCES = [("solve.cu", [], "solve"), ("batch.cu", [], "batch")]
 SOURCES += [("batch_kernel.cu", [f"-DBATCH_CONFIG={c}", f"-DBATCH_LISTS={u}"], f"batch_kernel_c{c}_l{u}")
             for c, u in ((0, 0), (0, 1), (1, 0), (1, 1), (2, 1))]
 SOURCES += [(f, [], f.split(".")[0]) for f in ("sweep.cu", "state.cu", "noalloc.cu", "mlp.cu", "api.cpp", "store.cpp",

@@ -30,6 +30,8 @@ int mlp_prior(const uint16_t *d_w, const std::vector<float> &features, int64_t n
 cudaError_t batch_configure(int config, bool lists, size_t smem, int *blocks_per_sm);
 cudaError_t launch_batch(int config, bool lists, const Dev *devs, const uint32_t *order, uint32_t n, unsigned int *queue, int grid,
                          size_t smem, cudaStream_t st);
+cudaError_t launch_batch_pack(const Dev *devs, uint32_t n, const long long *results, long long *places,
+                              unsigned long long *models, int64_t packed, cudaStream_t st);
 }  // namespace aspgpu
 
 using namespace aspgpu;
@@ -50,14 +52,6 @@ static int cuda_fail(cudaError_t e, const char *what)
 {
     return fail(ASP_E_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
-
-// device arrays of a frontier by units (see unit_lists)
-struct UnitLists {
-    const uint32_t *ubase = nullptr, *uoff = nullptr, *unit = nullptr;
-    uint32_t *dirty = nullptr;
-    uint32_t words = 0;
-    bool built = false;
-};
 
 struct asp_prog {
     asp_options opt{};
@@ -210,89 +204,6 @@ static int choose_view(asp_prog *p, const HostStore &H, Dev &D, const std::vecto
     return ASP_OK;
 }
 
-// Frontier by units (frontier = 2) over a static partition of G CTAs
-// (bucket L's nogoods [boff[L*(G+1)+g], boff[L*(G+1)+g+1]) belong to CTA
-// g): the sweep units numbered globally (CTA g's units are [ubase[g],
-// ubase[g+1]), in the order the device's unit table gives them: bucket by
-// bucket, unit_groups(L) groups of 32 nogoods each), for every variable the
-// units whose nogoods hold it, and the two dirty bitmaps.  Sets *built =
-// false (and allocates nothing) if the partition has more than max_units.
-
-static int unit_lists(asp_prog *p, const HostStore &H, const std::vector<uint32_t> &boff, uint32_t G,
-                      uint64_t max_units, UnitLists &out)
-{
-    const Dev &D = p->D;
-    const uint32_t G1 = G + 1u;
-    std::vector<uint32_t> ubase(G1, 0u), lbase((size_t)G * (BUCKET_MAX + 1), 0u);
-    for (uint32_t c = 0; c < G; c++) {
-        uint32_t acc = 0;
-        for (int L = 2; L <= BUCKET_MAX; L++) {
-            lbase[(size_t)c * (BUCKET_MAX + 1) + L] = acc;
-            const uint32_t n = boff[L * G1 + c + 1] - boff[L * G1 + c];
-            const uint32_t groups = (n + 31u) >> 5, per = unit_groups((uint32_t)L);
-            acc += (groups + per - 1u) / per;
-        }
-        ubase[c + 1] = ubase[c] + acc;
-    }
-    const uint32_t total = ubase[G];
-    out.built = false;
-    if (total > max_units) return ASP_OK;
-    // every (variable, unit) pair once: nogoods are visited in unit order,
-    // so a repeat of a pair is always adjacent to its first visit
-    std::vector<uint32_t> off((size_t)D.nv + 1, 0u), last((size_t)D.nv, 0xFFFFFFFFu), occ;
-    for (int pass = 0; pass < 2; pass++) {
-        std::fill(last.begin(), last.end(), 0xFFFFFFFFu);
-        std::vector<uint32_t> fill;
-        if (pass == 1) {
-            for (uint32_t v = 0; v < D.nv; v++) off[v + 1] += off[v];
-            occ.resize(off[D.nv]);
-            fill.assign(off.begin(), off.end() - 1);
-        }
-        for (uint32_t c = 0; c < G; c++) {
-            for (int L = 2; L <= BUCKET_MAX; L++) {
-                const std::vector<uint32_t> &rows = H.bucket_rows[L];
-                const uint32_t k0 = boff[L * G1 + c], k1 = boff[L * G1 + c + 1];
-                const uint32_t first = ubase[c] + lbase[(size_t)c * (BUCKET_MAX + 1) + L];
-                const uint32_t per = unit_groups((uint32_t)L) * 32u;
-                for (uint32_t k = k0; k < k1; k++) {
-                    const uint32_t u = first + (k - k0) / per;
-                    for (int q = 0; q < L; q++) {
-                        const uint32_t v = rows[(size_t)k * L + q] >> 1;
-                        if (last[v] == u) continue;
-                        last[v] = u;
-                        if (pass == 0) off[v + 1]++;
-                        else occ[fill[v]++] = u;
-                    }
-                }
-            }
-        }
-    }
-    int rc = ASP_OK;
-    out.ubase = upload(p, ubase, rc);
-    if (rc == ASP_OK) out.uoff = upload(p, off, rc);
-    if (rc == ASP_OK) out.unit = upload(p, occ, rc);
-    if (rc != ASP_OK) return rc;
-    out.words = (total + 31u) / 32u + 1u;
-    out.dirty = (uint32_t *)dalloc(p, (size_t)out.words * 2 * 4);
-    if (!out.dirty) return fail(ASP_E_OOM, "device allocation failed (dirty bitmaps)");
-    cudaError_t e = cudaMemsetAsync(out.dirty, 0, (size_t)out.words * 2 * 4, p->stream);
-    if (e != cudaSuccess) return cuda_fail(e, "clear dirty bitmaps");
-    out.built = true;
-    return ASP_OK;
-}
-
-// (a partition without lists sweeps everything; one with lists keeps the
-// requested unit mode, 2 or 3)
-static void use_unit_lists(Dev &D, const UnitLists &U)
-{
-    D.frontier = U.built ? (D.frontier >= 2u ? D.frontier : 2u) : 0u;
-    D.cta_ubase = U.ubase;
-    D.occ_uoff = U.uoff;
-    D.occ_unit = U.unit;
-    D.dirty = U.dirty;
-    D.dirty_words = U.words;
-}
-
 // Grid size, the static partition of the buckets over the CTAs along groups
 // (an atom with its rules; a constraint), each CTA's slice of auxiliary
 // variables kept in shared memory, and the shared-memory layout.
@@ -315,11 +226,12 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     if (p->opt.grid_ctas > 0) g = std::min(p->opt.grid_ctas, max_grid);
     p->grid = g;
     D.G = (uint32_t)g;
-    // one CTA follows up to this many claims in the time a sweep round takes:
-    // about 8 us and 0.2 ns a literal of the CTA's part, against about 0.03 us
-    // a claim
-    if (D.occ) D.narrow_max = (uint32_t)std::min<uint64_t>(256u + total / (uint64_t)g / 128u, 1u << 20);
-    D.lists = D.occ && g == 1;
+    // claims of a round that one CTA follows in the time of a round of the
+    // grid (about 6 us), and that the grid follows in the time of a sweep (a
+    // claim checks about three nogoods of 32 bytes each, at random)
+    D.narrow_max = 256u;
+    D.list_max = (uint32_t)(total / 128u);
+    D.lists = g == 1;
     if (D.lists) D.narrow_max = 0xFFFFFFFFu;
     // groups [glo[i], glo[i+1]) for CTA i, balanced by literal count
     const uint32_t ng = (uint32_t)H.n_groups;
@@ -359,12 +271,6 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     // a copy of the codes for the narrow rounds where it fits beside the view
     D.code_cache = p->smem + 4 * (size_t)D.asg_words <= max_smem;
     if (D.code_cache) p->smem += 4 * (size_t)D.asg_words;
-    if (D.frontier >= 2) {
-        UnitLists U;
-        rc = unit_lists(p, H, boff, D.G, ~0ull, U);
-        if (rc != ASP_OK) return rc;
-        use_unit_lists(D, U);
-    }
     D.cta_boff = upload(p, boff, rc);
     if (rc == ASP_OK) D.cta_auxlo = upload(p, alo, rc);
     if (rc == ASP_OK) D.cta_auxn = upload(p, an, rc);
@@ -394,13 +300,13 @@ static int plan_batch(asp_prog *p, const HostStore &H, int config)
     const size_t base = 8ull * D1.WW + 8ull * 32 + 4ull * 16 + MLP_SMEM_BYTES;
     D1.G = 1;
     D1.lists = D1.code_cache = 0u;
-    if (D1.occ) D1.narrow_max = (uint32_t)std::min<uint64_t>(64u + p->D.static_checks / 1024u, 1u << 20);
+    D1.narrow_max = (uint32_t)std::min<uint64_t>(64u + p->D.static_checks / 1024u, 1u << 20);
+    D1.list_max = D1.narrow_max;
     int rc = choose_view(p, H, D1, boff, alo, an, base, BATCH_SMEM_BUDGET[config]);
     if (rc != ASP_OK) return rc;
     D1.cta_boff = upload(p, boff, rc);
     if (rc == ASP_OK) D1.cta_auxlo = upload(p, alo, rc);
     if (rc == ASP_OK) D1.cta_auxn = upload(p, an, rc);
-    if (D1.frontier >= 2u) D1.frontier = 0u;     // no unit lists for the one-CTA partition
     p->D1[config] = D1;
     p->smem1[config] = base + 4 * D1.view_words;
     p->smem_base = base;
@@ -424,10 +330,20 @@ struct asp_batch {
     uint32_t queued = 0;
     cudaStream_t stream = nullptr;
     bool own_stream = false;
-    void *scratch = nullptr;
+    void *scratch = nullptr;            // descriptors | results | places | models | order | queue
     size_t scratch_bytes = 0;
+    int64_t packed = 0;                 // model words of the scratch
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
+
+    size_t n() const { return progs.size(); }
+    Dev *devs() const { return (Dev *)scratch; }
+    long long *results() const { return (long long *)(devs() + n()); }           // [n][4]
+    long long *places() const { return results() + 4 * n(); }                    // [n]
+    unsigned long long *models() const { return (unsigned long long *)(places() + n()); }
+    uint32_t *order() const { return (uint32_t *)(models() + packed); }
+    unsigned int *queue() const { return (unsigned int *)(order() + n()); }
+    size_t bytes() const { return sizeof(Dev) * n() + 8 * (5 * n() + (size_t)packed) + 4 * n() + 64; }
 };
 
 namespace {
@@ -445,10 +361,9 @@ std::vector<Dev> batch_descriptors(const asp_batch *b, int config, bool trial = 
     for (size_t i = 0; i < b->progs.size(); i++) {
         asp_prog *p = b->progs[i];
         Dev d = p->D1[config];
-        if (b->lists && d.occ) {
+        if (b->lists) {
             d.lists = 1u;
             d.narrow_max = 0xFFFFFFFFu;
-            d.frontier = 0u;
             d.view_atoms = d.view_words = 0u;
             d.code_cache = p->smem_base + 4 * (size_t)d.asg_words <= LISTS_SMEM_BUDGET[b->wide && config == 0 ? 2 : config];
         }
@@ -456,7 +371,7 @@ std::vector<Dev> batch_descriptors(const asp_batch *b, int config, bool trial = 
         d.max_models = b->max_models_each;
         d.models_cap = b->caps[i];
         d.models = p->d_models;
-        d.result = p->d_result;
+        d.result = b->results() + 4 * i;
         d.conflict_budget = p->opt.conflict_budget;
         d.time_budget_ns = p->opt.time_budget_ms > 0 ? p->opt.time_budget_ms * 1000000ll : 0;
         if (trial) {
@@ -485,10 +400,8 @@ int batch_prepare(asp_batch *b, int config, const std::vector<uint32_t> &order, 
     if (e != cudaSuccess) return cuda_fail(e, "batch configuration");
     if (per_sm < 1) return fail(ASP_E_CUDA, "batch kernel cannot be resident");
     const std::vector<Dev> devs = batch_descriptors(b, config, trial);
-    Dev *d_devs = (Dev *)b->scratch;
-    uint32_t *d_order = (uint32_t *)((char *)b->scratch + sizeof(Dev) * n);
-    e = cudaMemcpyAsync(d_devs, devs.data(), sizeof(Dev) * n, cudaMemcpyHostToDevice, b->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(d_order, order.data(), 4 * order.size(), cudaMemcpyHostToDevice, b->stream);
+    e = cudaMemcpyAsync(b->devs(), devs.data(), sizeof(Dev) * n, cudaMemcpyHostToDevice, b->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(b->order(), order.data(), 4 * order.size(), cudaMemcpyHostToDevice, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);     // host vectors go out of scope
     if (e != cudaSuccess) return cuda_fail(e, "batch descriptors");
     b->config = config;
@@ -502,12 +415,8 @@ int batch_prepare(asp_batch *b, int config, const std::vector<uint32_t> &order, 
 // enqueue one batch launch as prepared: reset the queue counter, launch
 cudaError_t batch_enqueue(asp_batch *b)
 {
-    const size_t n = b->progs.size();
-    Dev *d_devs = (Dev *)b->scratch;
-    uint32_t *d_order = (uint32_t *)((char *)b->scratch + sizeof(Dev) * n);
-    unsigned int *d_queue = (unsigned int *)((char *)d_order + 4 * n);
-    cudaError_t e = cudaMemsetAsync(d_queue, 0, 64, b->stream);
-    if (e == cudaSuccess) e = launch_batch(b->kernel, b->lists, d_devs, d_order, b->queued, d_queue, b->grid, b->smem, b->stream);
+    cudaError_t e = cudaMemsetAsync(b->queue(), 0, 64, b->stream);
+    if (e == cudaSuccess) e = launch_batch(b->kernel, b->lists, b->devs(), b->order(), b->queued, b->queue(), b->grid, b->smem, b->stream);
     return e;
 }
 
@@ -1159,7 +1068,11 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
         b->own_stream = true;
     }
     asp_prog *p0 = progs[0];
-    b->scratch_bytes = sizeof(Dev) * (size_t)n + 4 * (size_t)n + 64;
+    // room for every program's models, up to 64 MB (what does not fit is copied
+    // program by program)
+    for (int32_t i = 0; i < n; i++) b->packed += std::min<int64_t>(b->caps[i] * (((int64_t)progs[i]->D.na + 63) / 64), 1ll << 40);
+    b->packed = std::min<int64_t>(b->packed, 8ll << 20);
+    b->scratch_bytes = b->bytes();
     if (p0->opt.dev_alloc) b->scratch = p0->opt.dev_alloc(b->scratch_bytes, p0->opt.alloc_ctx);
     else if (cudaMalloc(&b->scratch, b->scratch_bytes) != cudaSuccess) { cudaGetLastError(); b->scratch = nullptr; }
     if (!b->scratch) return bail(fail(ASP_E_OOM, "device allocation failed (batch descriptors)"));
@@ -1199,6 +1112,7 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
     cudaError_t e = cudaStreamBeginCapture(b->stream, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
         cudaError_t e2 = batch_enqueue(b);
+        if (e2 == cudaSuccess) e2 = launch_batch_pack(b->devs(), (uint32_t)n, b->results(), b->places(), b->models(), b->packed, b->stream);
         e = cudaStreamEndCapture(b->stream, &b->graph);
         if (e == cudaSuccess) e = e2;
     }
@@ -1215,24 +1129,39 @@ int asp_batch_run(asp_batch *b, int32_t *statuses, int64_t *n_models, uint64_t *
     const int32_t n = (int32_t)b->progs.size();
     for (int32_t i = 0; i < n; i++)
         if (b->caps[i] > 0 && (!models || !models[i])) return fail(ASP_E_ARG, "null model buffer");
+    // every program's result in one copy, the models (packed on the device)
+    // in another: a copy per program took 8 us each
+    std::vector<long long> res((size_t)n * 5);
     cudaError_t e = cudaGraphLaunch(b->exec, b->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(res.data(), b->results(), res.size() * 8, cudaMemcpyDeviceToHost, b->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return cuda_fail(e, "batch solve");
+    const long long *place = res.data() + 4 * (size_t)n;
+    auto model_words = [&](int32_t i) -> int64_t {
+        return std::min<int64_t>(res[4 * (size_t)i + 1], b->caps[i]) * (((int64_t)b->progs[i]->D.na + 63) / 64);
+    };
+    int64_t used = 0;
+    for (int32_t i = 0; i < n; i++)
+        if (place[i] >= 0) used = std::max<int64_t>(used, place[i] + model_words(i));
+    std::vector<uint64_t> rows((size_t)used);
+    if (used > 0) {
+        e = cudaMemcpyAsync(rows.data(), b->models(), (size_t)used * 8, cudaMemcpyDeviceToHost, b->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(b->stream);
+        if (e != cudaSuccess) return cuda_fail(e, "batch models");
+    }
     bool device_error = false, capacity = false;
     for (int32_t i = 0; i < n; i++) {
-        asp_prog *p = b->progs[i];
-        long long res[4];
-        e = cudaMemcpy(res, p->d_result, sizeof(res), cudaMemcpyDeviceToHost);
-        if (e != cudaSuccess) return cuda_fail(e, "batch result");
-        statuses[i] = (int32_t)res[0];
-        n_models[i] = res[1];
-        device_error |= res[2] != 0;
-        const int64_t cap = b->caps[i];
-        const int64_t words = ((int64_t)p->D.na + 63) / 64;
-        const int64_t copy = std::min<int64_t>(res[1], cap);
-        capacity |= res[1] > cap && cap > 0;
-        if (copy > 0 && words > 0) {
-            e = cudaMemcpy(models[i], p->d_models, (size_t)(copy * words) * 8, cudaMemcpyDeviceToHost);
+        const long long *r = res.data() + 4 * (size_t)i;
+        statuses[i] = (int32_t)r[0];
+        n_models[i] = r[1];
+        device_error |= r[2] != 0;
+        capacity |= r[1] > b->caps[i] && b->caps[i] > 0;
+        const int64_t words = model_words(i);
+        if (words <= 0) continue;
+        if (place[i] >= 0) {
+            std::memcpy(models[i], rows.data() + place[i], (size_t)words * 8);
+        } else {
+            e = cudaMemcpy(models[i], b->progs[i]->d_models, (size_t)words * 8, cudaMemcpyDeviceToHost);
             if (e != cudaSuccess) return cuda_fail(e, "batch models");
         }
     }

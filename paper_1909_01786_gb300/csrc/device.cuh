@@ -70,9 +70,8 @@ struct Ctl {              // double-buffered control block (phase parity)
     long long n_models;
     int32_t status, err;
     int32_t conflict;
-    uint32_t full;              // the next round sweeps every nogood (else the frontier)
-    uint32_t chased;            // the last claims have been followed by narrow rounds
-    uint32_t tcom;              // trail entries whose assignments are committed (tc: those in the views)
+    uint32_t full;              // the next round sweeps every nogood
+    uint32_t pad, tcom;                     // trail entries whose assignments are committed (tc: those in the views)
 };
 
 struct Acc {              // per-phase accumulators, indexed by phase % 4
@@ -84,9 +83,8 @@ struct Acc {              // per-phase accumulators, indexed by phase % 4
     uint32_t flag;              // something changed (least-model iteration)
     uint32_t minU;              // smallest unfounded true atom
     uint32_t nlits;             // literals appended to the loop nogood
-    unsigned long long checks;  // literals classified by long/learned sweeps (and by unit
-                                // frontiers' bucket units)
-    unsigned long long visits;  // bucket nogoods classified by unit frontiers
+    unsigned long long checks;  // literals classified outside full sweeps of the buckets
+    unsigned long long visits;  // bucket nogoods classified through the occurrence lists
     unsigned long long tbusy;   // max over CTAs of the time from phase start to barrier arrival
     unsigned long long tsweep;  // max over CTAs of the time in the sweep
     unsigned long long tlong;   // max over warps of the sweep's long and learned nogoods
@@ -187,27 +185,18 @@ struct Dev {
     // literals (PAD_LIT past their number), or, for one of more than eight
     // literals, id, END_BIT | length and the place of its literals in rows.
     // A phase with at most narrow_max claims to follow is run by one CTA
-    // through them (narrow_rounds; 0 = no lists).
+    // through them (narrow_rounds), one with at most list_max by the grid
+    // (list_round), one with more is a sweep.
     // lists: one CTA solves the program, and its bucket nogoods are checked
     // through the lists only: no sweep, no view
     // code_cache: narrow rounds work on a copy of the codes in shared memory
-    uint32_t narrow_max, lists, code_cache, pad4;
-    // frontier propagation (Algorithm 2's idea): a round checks only the
-    // bucket nogoods of the variables assigned in the previous round; full
-    // sweeps after (re)starts and backjumps
+    uint32_t narrow_max, list_max, lists, code_cache;
+    // frontier propagation (Algorithm 2's idea; any value but 0): once the
+    // claims of a round are followed through the lists the static buckets are
+    // at their fixpoint, without a sweep that confirms it
     uint32_t frontier;
     const uint32_t *occ_off, *rows;
     const Occurrence *occ;
-    // frontier = 2 (frontier by bucket units): the sweep units of the static
-    // partition are numbered globally, CTA g's being [cta_ubase[g],
-    // cta_ubase[g+1]); occ_unit[occ_uoff[v] .. occ_uoff[v+1]) are the units
-    // whose nogoods hold variable v.  A claim sets the bits of v's units in
-    // the next round's dirty bitmap (two bitmaps of dirty_words words,
-    // alternating by round); each round's sweep checks the units whose bit
-    // is set and clears them.
-    const uint32_t *cta_ubase, *occ_uoff, *occ_unit;
-    uint32_t *dirty;
-    uint32_t dirty_words, pad3;
     uint32_t *asg;
     int32_t *dl;
     uint32_t *reason;

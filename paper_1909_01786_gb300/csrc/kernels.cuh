@@ -1,22 +1,8 @@
-// The solver kernels (device code in solver.cuh), instantiated per
-// translation unit: solve.cu without the frontier by units, solve_units.cu
-// with it, batch_kernel.cu per batch configuration.
+// The batch kernel (device code in solver.cuh), instantiated in batch_kernel.cu.
 #pragma once
 #include "solver.cuh"
 
 namespace aspgpu {
-
-// The single-program solver: one persistent cooperative kernel over the
-// whole grid runs Algorithm 1.
-template <bool UNITS>
-__global__ void __launch_bounds__(768, 1) solve_kernel(Dev D)
-{
-    extern __shared__ unsigned long long smem_raw[];
-    const Smem S = make_smem(D, smem_raw);
-    const View V = make_view(D, S.misc + 16, blockIdx.x);
-    solver_loop<false, UNITS, false>(D, S, V, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x, blockIdx.x == 0,
-                       blockIdx.x == 0 && threadIdx.x == 0, blockIdx.x);
-}
 
 // Batched solving: each CTA takes programs from a queue (the host orders it
 // largest first) and solves each alone, with a CTA barrier as the phase
@@ -62,7 +48,7 @@ __global__ void __launch_bounds__(THREADS, MIN_BLOCKS) batch_kernel(const Dev *d
         cta_sync();
         const Smem S = make_smem(D, smem_raw);
         const View V = make_view(D, S.misc + 16, 0);
-        solver_loop<true, false, LISTS>(D, S, V, threadIdx.x, blockDim.x, true, threadIdx.x == 0, 0);
+        solver_loop<true, LISTS>(D, S, V, threadIdx.x, blockDim.x, true, threadIdx.x == 0, 0);
         cta_sync();
     }
 }

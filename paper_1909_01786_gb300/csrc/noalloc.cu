@@ -160,8 +160,8 @@ __device__ __forceinline__ void na_claim(uint32_t *asg, NaCtl *c, uint32_t l, ui
 
 // Checks the bucket nogoods of the n literals at `from` (each holds since the
 // round before; no other nogood can have become unit or violated): warps w,
-// w + nw, ... take eight literals at a time and share out their lists
-// (warp_lists, quad_check).  A literal's own fresh bit, of the other parity,
+// w + nw, ... take up to eight literals at a time (fewer when there are fewer
+// than eight a warp) and share out their lists (warp_lists, quad_check).  A literal's own fresh bit, of the other parity,
 // is cleared meanwhile.  SHARED: `from` is in shared memory.
 template <bool SHARED>
 __device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c, const uint32_t *from, uint32_t n, uint32_t w,
@@ -169,10 +169,11 @@ __device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c,
 {
     const uint32_t lane = threadIdx.x & 31u;
     const Codes<false> codes{asg};
-    for (uint32_t i0 = w * 8u; i0 < n; i0 += nw * 8u) {
+    const uint32_t each = min(8u, (n + nw - 1u) / nw);
+    for (uint32_t i0 = w * each; i0 < n; i0 += nw * each) {
         const uint32_t i = i0 + lane;
         uint32_t o0 = 0, count = 0;
-        if (lane < 8u && i < n) {
+        if (lane < each && i < n) {
             const uint32_t l = SHARED ? from[i] : __ldcg(from + i), y = l >> 1;
             o0 = __ldg(D.occ_off + l);
             count = __ldg(D.occ_off + l + 1u) - o0;

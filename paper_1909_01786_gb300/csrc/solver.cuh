@@ -321,19 +321,11 @@ struct SweepCtx {
     Acc *acc;              // this phase's accumulators
     bool do_claim;
     bool use_view;
-    uint32_t dec_v;        // decision variable set in this phase (its level
-                           // and bitmap are known here before they reach memory)
     uint32_t cta;          // this CTA's part of the static partition
     uint32_t gw, nw;       // warp index and warp count of the solving group
     // inside a sweep: claims are listed in shared memory and copied to the
     // trail once at the end of the sweep (one global atomic per CTA)
     bool listed = false;
-    // frontier by units: the next round's dirty bitmap (null otherwise)
-    uint32_t *dmark = nullptr;
-    // frontier by units with chaining in the round (frontier = 3): a claim
-    // queues the CTA's own units that hold its variable for a later wave of
-    // the same sweep
-    bool chain = false;
 };
 
 constexpr uint32_t CLAIM_BUF = 256;
@@ -352,108 +344,6 @@ __shared__ unsigned int s_unit, s_unit2[2];
 __shared__ unsigned long long s_tlearned, s_tbuckets;
 // the same two parts, max over the CTA's warps in the current sweep
 __shared__ unsigned long long s_wmax[2];
-// frontier by units (single-program solver only): this round's queue of the
-// CTA's bucket units (local unit indices) and its length
-constexpr uint32_t DQ_CAP = 1024;
-__shared__ uint32_t s_dq[DQ_CAP];
-__shared__ unsigned int s_nq;
-// frontier = 3: units already in this round's queue (local units below
-// DQ_BITS), the per-wave pop counters, and the CTA's global unit range
-constexpr uint32_t DQ_BITS = 4096, DQ_WAVES = 4;
-__shared__ uint32_t s_dqbits[DQ_BITS / 32];
-__shared__ unsigned int s_wave[DQ_WAVES];
-__shared__ uint32_t s_ub[3];
-
-// Queue local unit `local` once per round (frontier = 3); the caller keeps
-// it below DQ_BITS.
-__device__ __forceinline__ void dq_push_once(uint32_t local)
-{
-    const uint32_t bit = 1u << (local & 31u);
-    if (atomicOr(&s_dqbits[local >> 5], bit) & bit) return;
-    const uint32_t pos = atomicAdd(&s_nq, 1u);
-    if (pos < DQ_CAP) s_dq[pos] = local;
-}
-
-// frontier = 3: after a claim of x is published in the CTA's view, queue
-// the CTA's own units that hold x for the next wave of this sweep (units of
-// other CTAs, and any that do not fit, are checked next round through the
-// dirty bitmap).  All 32 lanes call it with the same x.
-__device__ __forceinline__ void warp_push_units(const SweepCtx &X, uint32_t x)
-{
-    const Dev &D = *X.D;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t ub0 = s_ub[0], ub1 = s_ub[1];
-    const uint32_t o0 = __ldg(D.occ_uoff + x), o1 = __ldg(D.occ_uoff + x + 1u);
-    for (uint32_t o = o0 + lane; o < o1; o += 32u) {
-        const uint32_t u = __ldg(D.occ_unit + o);
-        if (u >= ub0 && u < ub1 && u - ub0 < DQ_BITS) dq_push_once(u - ub0);
-    }
-}
-
-// The same from one lane.
-__device__ __forceinline__ void lane_push_units(const SweepCtx &X, uint32_t x)
-{
-    const Dev &D = *X.D;
-    const uint32_t ub0 = s_ub[0], ub1 = s_ub[1];
-    const uint32_t o0 = __ldg(D.occ_uoff + x), o1 = __ldg(D.occ_uoff + x + 1u);
-    for (uint32_t o = o0; o < o1; o++) {
-        const uint32_t u = __ldg(D.occ_unit + o);
-        if (u >= ub0 && u < ub1 && u - ub0 < DQ_BITS) dq_push_once(u - ub0);
-    }
-}
-
-// Frontier by units: this CTA's bucket units to check in the round -- those
-// whose bit is set in the round's dirty bitmap `buf` (set by the claims of
-// the previous claiming phase; the bits read are cleared) and, in a decision
-// phase, those holding the decision variable dec_v.  Warp 0 writes the queue
-// (s_nq > DQ_CAP: it overflowed, and the CTA sweeps all its units); the
-// caller synchronises the CTA before the sweep.
-__device__ __forceinline__ void build_unit_queue(const Dev &D, uint32_t cta, uint32_t *buf, uint32_t dec_v)
-{
-    if (threadIdx.x >= 32u) return;
-    const uint32_t lane = threadIdx.x;
-    const uint32_t ub0 = __ldg(D.cta_ubase + cta), ub1 = __ldg(D.cta_ubase + cta + 1u);
-    if (ub1 > ub0) {
-        const uint32_t w_first = ub0 >> 5, w_last = (ub1 - 1u) >> 5;
-        for (uint32_t w0 = w_first; w0 <= w_last; w0 += 32u) {
-            const uint32_t w = w0 + lane;
-            uint32_t bits = 0u;
-            if (w <= w_last) {
-                uint32_t own = ~0u;
-                if (w == w_first) own &= ~0u << (ub0 & 31u);
-                if (w == w_last && (ub1 & 31u)) own &= (1u << (ub1 & 31u)) - 1u;
-                bits = __ldcg(buf + w) & own;
-                if (bits) atomicAnd(buf + w, ~bits);
-            }
-            while (bits) {
-                const uint32_t b = (uint32_t)__ffs(bits) - 1u;
-                bits &= bits - 1u;
-                const uint32_t local = w * 32u + b - ub0;
-                if (D.frontier == 3u && local < DQ_BITS) {
-                    dq_push_once(local);
-                } else {
-                    const uint32_t pos = atomicAdd(&s_nq, 1u);
-                    if (pos < DQ_CAP) s_dq[pos] = local;
-                }
-            }
-        }
-    }
-    if (dec_v != 0xFFFFFFFFu) {
-        const uint32_t o0 = __ldg(D.occ_uoff + dec_v), o1 = __ldg(D.occ_uoff + dec_v + 1u);
-        for (uint32_t o = o0 + lane; o < o1; o += 32u) {
-            const uint32_t u = __ldg(D.occ_unit + o);
-            if (u >= ub0 && u < ub1) {
-                if (D.frontier == 3u && u - ub0 < DQ_BITS) {
-                    dq_push_once(u - ub0);
-                } else {
-                    const uint32_t pos = atomicAdd(&s_nq, 1u);
-                    if (pos < DQ_CAP) s_dq[pos] = u - ub0;
-                }
-            }
-        }
-    }
-}
-
 __device__ __forceinline__ void report_conflict(const SweepCtx &X, uint32_t id, uint32_t len)
 {
     const unsigned long long key = ((unsigned long long)len << 32) | id;
@@ -479,33 +369,6 @@ __device__ __forceinline__ void record_claim(const SweepCtx &X, uint32_t v, uint
     }
 }
 
-// Frontier by units: the bucket units holding variable x are checked in the
-// next round; set their bits in that round's dirty bitmap.  All 32 lanes call
-// it with the same x.
-__device__ __forceinline__ void warp_mark_units(const SweepCtx &X, uint32_t x)
-{
-    if (!X.dmark) return;
-    const Dev &D = *X.D;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t o0 = __ldg(D.occ_uoff + x), o1 = __ldg(D.occ_uoff + x + 1u);
-    for (uint32_t o = o0 + lane; o < o1; o += 32u) {
-        const uint32_t u = __ldg(D.occ_unit + o);
-        atomicOr(X.dmark + (u >> 5), 1u << (u & 31u));
-    }
-}
-
-// The same from one lane.
-__device__ __forceinline__ void lane_mark_units(const SweepCtx &X, uint32_t x)
-{
-    if (!X.dmark) return;
-    const Dev &D = *X.D;
-    const uint32_t o0 = __ldg(D.occ_uoff + x), o1 = __ldg(D.occ_uoff + x + 1u);
-    for (uint32_t o = o0; o < o1; o++) {
-        const uint32_t u = __ldg(D.occ_unit + o);
-        atomicOr(X.dmark + (u >> 5), 1u << (u & 31u));
-    }
-}
-
 // One lane per literal u of a reason (has = false on lanes holding none):
 // the warp ORs Deps[u] over lanes with level > 1 and writes Deps[x]
 // (Section 4.2, mk_dl_bitmap).  All 32 lanes call it.
@@ -516,14 +379,13 @@ __device__ __forceinline__ void warp_or_deps(const SweepCtx &X, bool has, uint32
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t L = X.cdl;
     const uint32_t nw = deps_words(D, L);
-    const bool is_dec = has && u == X.dec_v;
     // a decision's bitmap is the bit of its own level: with the level, the
     // reason tells whether the bitmap words need loading at all (a learned
     // nogood of fwd-learning holds decisions only)
-    int32_t Lu = !has ? 0 : is_dec ? (int32_t)L : __ldcg(D.dl + u);
-    const uint32_t ru = (has && !is_dec) ? __ldcg(D.reason + u) : 0u;
+    int32_t Lu = has ? __ldcg(D.dl + u) : 0;
+    const uint32_t ru = has ? __ldcg(D.reason + u) : 0u;
     uint32_t nwu = (has && Lu > 1) ? deps_words(D, (uint32_t)Lu) : 0u;
-    const bool dec = is_dec || (has && Lu > 1 && ru == R_DECISION);
+    const bool dec = has && Lu > 1 && ru == R_DECISION;
     const uint32_t dbit = level_bit(D, dec ? (uint32_t)Lu : L);
     for (uint32_t w = 0; w < nw; w++) {
         unsigned long long c = w >= nwu ? 0ull
@@ -552,35 +414,28 @@ __device__ __forceinline__ void lane_deps(const SweepCtx &X, const uint32_t (&va
 {
     const Dev &D = *X.D;
     const uint32_t nw = deps_words(D, X.cdl);
-    const uint32_t dbit = level_bit(D, X.cdl);
     int32_t Lu[L];
 #pragma unroll
-    for (int q = 0; q < L; q++) {
-        uint32_t u = var[q];
-        Lu[q] = (u == x) ? 0 : (u == X.dec_v) ? (int32_t)X.cdl : __ldcg(D.dl + u);
-    }
+    for (int q = 0; q < L; q++) Lu[q] = var[q] == x ? 0 : __ldcg(D.dl + var[q]);
     for (uint32_t w = 0; w < nw; w++) {
         unsigned long long acc = 0;
 #pragma unroll
         for (int q = 0; q < L; q++) {
             uint32_t u = var[q];
-            if (Lu[q] > 1 && w < deps_words(D, (uint32_t)Lu[q]))
-                acc |= (u == X.dec_v) ? (w == (dbit >> 6) ? (1ull << (dbit & 63u)) : 0ull)
-                                      : __ldcg(D.deps + (size_t)u * D.WW + w);
+            if (Lu[q] > 1 && w < deps_words(D, (uint32_t)Lu[q])) acc |= __ldcg(D.deps + (size_t)u * D.WW + w);
         }
         D.deps[(size_t)x * D.WW + w] = acc;
     }
 }
 
-// Dependency bitmaps (Section 4.2, mk_dl_bitmap) -- and, with the frontier
-// by units, the unit marks -- of every claim of a group of 32 nogoods at
-// once: the claims take equal shares of the warp's lanes (32 / p2 lanes
-// each, p2 the claim count rounded up to a power of two), and the lanes of a
-// claim split its bitmap words and its occurrence list, so the group costs
-// the two dependent loads of one claim whatever the number of claims.  All 32
-// lanes call it; won: this lane's nogood claimed x; tl: its literals as view
-// entries.  Returns whether the group made a claim.
-template <int L, bool MARK>
+// Dependency bitmaps (Section 4.2, mk_dl_bitmap) of every claim of a group of
+// 32 nogoods at once: the claims take equal shares of the warp's lanes (32 / p2
+// lanes each, p2 the claim count rounded up to a power of two), and the lanes
+// of a claim split its bitmap words, so the group costs the two dependent
+// loads of one claim whatever the number of claims.  All 32 lanes call it; won:
+// this lane's nogood claimed x; tl: its literals as view entries.  Returns
+// whether the group made a claim.
+template <int L>
 __device__ __forceinline__ bool group_claims(const SweepCtx &X, bool won, const uint32_t (&tl)[L], uint32_t x)
 {
     const Dev &D = *X.D;
@@ -600,84 +455,18 @@ __device__ __forceinline__ bool group_claims(const SweepCtx &X, bool won, const 
     for (int q = 0; q < L; q++) var[q] = X.V.var(__shfl_sync(FULL_MASK, tl[q], src) >> 2);
     const uint32_t xs = __shfl_sync(FULL_MASK, x, src);
     if (c >= nc) return true;
-    // unit marks: the bounds of the claim's unit list load with the levels,
-    // and its first entry for this lane with the bitmap words, so the marks
-    // add no dependent load to the claim
-    uint32_t o0 = 0u, o1 = 0u;
-    if constexpr (MARK) {
-        if (X.dmark) {
-            o0 = __ldg(D.occ_uoff + xs);
-            o1 = __ldg(D.occ_uoff + xs + 1u);
-        }
-    }
-    if (X.cdl > 1u) {
-        const uint32_t nw = deps_words(D, X.cdl);
-        const uint32_t dbit = level_bit(D, X.cdl);
-        int32_t Lu[L];
-        bool has_dec = false;
+    const uint32_t nw = deps_words(D, X.cdl);
+    int32_t Lu[L];
 #pragma unroll
-        for (int q = 0; q < L; q++) {
-            const uint32_t u = var[q];
-            has_dec |= u != xs && u == X.dec_v;
-            Lu[q] = (u != xs && u != X.dec_v) ? __ldcg(D.dl + u) : 0;
-        }
-        uint32_t first = 0xFFFFFFFFu;
-        if constexpr (MARK) {
-            if (o0 + sub < o1) first = __ldg(D.occ_unit + o0 + sub);
-        }
-        for (uint32_t w = sub; w < nw; w += gs) {
-            unsigned long long acc = (has_dec && w == (dbit >> 6)) ? (1ull << (dbit & 63u)) : 0ull;
+    for (int q = 0; q < L; q++) Lu[q] = var[q] != xs ? __ldcg(D.dl + var[q]) : 0;
+    for (uint32_t w = sub; w < nw; w += gs) {
+        unsigned long long acc = 0;
 #pragma unroll
-            for (int q = 0; q < L; q++)
-                if (Lu[q] > 1 && 64u * w < (uint32_t)Lu[q]) acc |= __ldcg(D.deps + (size_t)var[q] * D.WW + w);
-            D.deps[(size_t)xs * D.WW + w] = acc;
-        }
-        if constexpr (MARK) {
-            if (first != 0xFFFFFFFFu) atomicOr(X.dmark + (first >> 5), 1u << (first & 31u));
-            for (uint32_t o = o0 + sub + gs; o < o1; o += gs) {
-                const uint32_t u = __ldg(D.occ_unit + o);
-                atomicOr(X.dmark + (u >> 5), 1u << (u & 31u));
-            }
-        }
-        return true;
-    }
-    if constexpr (MARK) {
-        for (uint32_t o = o0 + sub; o < o1; o += gs) {
-            const uint32_t u = __ldg(D.occ_unit + o);
-            atomicOr(X.dmark + (u >> 5), 1u << (u & 31u));
-        }
+        for (int q = 0; q < L; q++)
+            if (Lu[q] > 1 && 64u * w < (uint32_t)Lu[q]) acc |= __ldcg(D.deps + (size_t)var[q] * D.WW + w);
+        D.deps[(size_t)xs * D.WW + w] = acc;
     }
     return true;
-}
-
-// Dependency bitmap of x (claimed by one lane) computed by the whole warp,
-// for a nogood of L <= BUCKET_MAX literals known at run time (var[q] for
-// q < L): every lane loads the levels of the nogood's other variables and
-// ORs the bitmap words w = lane, lane + 32, ... over those with level > 1
-// (Section 4.2, mk_dl_bitmap).  All 32 lanes call it with the same arguments.
-__device__ __forceinline__ void warp_deps_dyn(const SweepCtx &X, const uint32_t (&var)[BUCKET_MAX], uint32_t L,
-                                              uint32_t x)
-{
-    const Dev &D = *X.D;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t nw = deps_words(D, X.cdl);
-    const uint32_t dbit = level_bit(D, X.cdl);
-    int32_t Lu[BUCKET_MAX];
-    bool has_dec = false;
-#pragma unroll
-    for (int q = 0; q < BUCKET_MAX; q++) {
-        const uint32_t u = var[q];
-        const bool in = (uint32_t)q < L;
-        has_dec |= in && u != x && u == X.dec_v;
-        Lu[q] = (in && u != x && u != X.dec_v) ? __ldcg(D.dl + u) : 0;
-    }
-    for (uint32_t w = lane; w < nw; w += 32u) {
-        unsigned long long acc = (has_dec && w == (dbit >> 6)) ? (1ull << (dbit & 63u)) : 0ull;
-#pragma unroll
-        for (int q = 0; q < BUCKET_MAX; q++)
-            if (Lu[q] > 1 && 64u * w < (uint32_t)Lu[q]) acc |= __ldcg(D.deps + (size_t)var[q] * D.WW + w);
-        D.deps[(size_t)x * D.WW + w] = acc;
-    }
 }
 
 // U groups of 32 nogoods of bucket L, lane = nogood k0 + t*stride + lane.
@@ -686,7 +475,7 @@ __device__ __forceinline__ void warp_deps_dyn(const SweepCtx &X, const uint32_t 
 // some literal's complement holds, violated if all hold, unit if exactly one
 // is unassigned and the rest hold (Section 2).  Repeats while a claim of
 // this warp changed the view.
-template <int L, int U, bool MARK>
+template <int L, int U>
 __device__ __forceinline__ void bucket_tasks(const SweepCtx &X, uint32_t k0, uint32_t k1, uint32_t stride)
 {
     const Dev &D = *X.D;
@@ -728,7 +517,6 @@ __device__ __forceinline__ void bucket_tasks(const SweepCtx &X, uint32_t k0, uin
             if (r == 2) { report_conflict(X, id, (uint32_t)L); continue; }
             if (r != 0) continue;
             record_claim(X, x, valbit, id);
-            if constexpr (MARK) lane_mark_units(X, x);
             if (X.cdl > 1u) {
                 uint32_t var[L];
 #pragma unroll
@@ -782,10 +570,9 @@ struct Row { uint32_t q[L]; };
 // classifies it again from the current view (a claim of this CTA may have
 // changed it since the count), reports a violation, or claims the variable
 // of its one unassigned literal; then the group's claims get their
-// dependency bitmaps (and, with the frontier by units, their unit marks),
-// and are published in the view.  All 32 lanes call it.  Returns whether
+// dependency bitmaps and are published in the view.  All 32 lanes call it.  Returns whether
 // this lane claimed.
-template <int L, bool BYTES, bool MARK>
+template <int L, bool BYTES>
 __device__ __forceinline__ bool group_claim_path(const SweepCtx &X, const Row<L> &r, uint32_t k, bool cand)
 {
     const Dev &D = *X.D;
@@ -816,19 +603,16 @@ __device__ __forceinline__ bool group_claim_path(const SweepCtx &X, const Row<L>
             }
         }
     }
-    if (L > 8 && won && (MARK || X.cdl > 1u)) {
+    if (L > 8 && won && X.cdl > 1u) {
         // long buckets (few claims): the claiming lane alone
-        if constexpr (MARK) lane_mark_units(X, x);
-        if (X.cdl > 1u) {
-            uint32_t var[L];
+        uint32_t var[L];
 #pragma unroll
-            for (int q = 0; q < L; q++) var[q] = X.V.var(r.q[q] >> 2);
-            lane_deps<L>(X, var, x);
-        }
+        for (int q = 0; q < L; q++) var[q] = X.V.var(r.q[q] >> 2);
+        lane_deps<L>(X, var, x);
     }
-    if (L <= 8 && (X.cdl > 1u || (MARK && X.dmark))) {
-        // bitmaps (and unit marks) of this group's claims, all at once
-        if (group_claims<L, MARK>(X, won, r.q, x)) {
+    if (L <= 8 && X.cdl > 1u) {
+        // bitmaps of this group's claims, all at once
+        if (group_claims<L>(X, won, r.q, x)) {
             __threadfence_block();
             __syncwarp();
         }
@@ -837,22 +621,6 @@ __device__ __forceinline__ bool group_claim_path(const SweepCtx &X, const Row<L>
         __threadfence_block();
         X.V.put(e, valbit);
     }
-    if constexpr (MARK) {
-        if (X.chain) {
-            // frontier = 3: the CTA's units that hold the claims, for the
-            // next wave (after the claims are in the view)
-            if (L > 8) {
-                if (won) lane_push_units(X, x);
-            } else {
-                unsigned m = __ballot_sync(FULL_MASK, won);
-                while (m) {
-                    const int src = __ffs(m) - 1;
-                    m &= m - 1u;
-                    warp_push_units(X, __shfl_sync(FULL_MASK, x, src));
-                }
-            }
-        }
-    }
     return won;
 }
 
@@ -860,7 +628,7 @@ __device__ __forceinline__ bool group_claim_path(const SweepCtx &X, const Row<L>
 // and BYTES): every literal is in the view, one shared-memory load and
 // three integer operations classify it.  Lanes past the end of the range
 // load the range's last nogood and drop the result.
-template <int L, int U, bool BYTES, bool MARK>
+template <int L, int U, bool BYTES>
 __device__ __forceinline__ void bucket_tasks_view(const SweepCtx &X, uint32_t k0, uint32_t k1)
 {
     const Dev &D = *X.D;
@@ -908,52 +676,51 @@ __device__ __forceinline__ void bucket_tasks_view(const SweepCtx &X, uint32_t k0
                 for (int q = 0; q < L; q++) r.q[q] = sel_if(t == tt, lit[tt][q], r.q[q]);
             }
             const uint32_t k = k0 + (uint32_t)t * 32u + lane;
-            pub |= group_claim_path<L, BYTES, MARK>(X, r, k, k < k1 && (c & 0xFFu) <= 1u);
+            pub |= group_claim_path<L, BYTES>(X, r, k, k < k1 && (c & 0xFFu) <= 1u);
         }
         if (!X.do_claim || !__any_sync(FULL_MASK, pub)) break;
     }
 }
 
 
-template <bool BYTES, bool MARK>
+template <bool BYTES>
 __device__ __forceinline__ void run_unit_view(const SweepCtx &X, uint32_t L, uint32_t k0, uint32_t k1)
 {
     switch (L) {
-    case 2: bucket_tasks_view<2, unit_groups(2), BYTES, MARK>(X, k0, k1); break;
-    case 3: bucket_tasks_view<3, unit_groups(3), BYTES, MARK>(X, k0, k1); break;
-    case 4: bucket_tasks_view<4, unit_groups(4), BYTES, MARK>(X, k0, k1); break;
-    case 5: bucket_tasks_view<5, unit_groups(5), BYTES, MARK>(X, k0, k1); break;
-    case 6: bucket_tasks_view<6, unit_groups(6), BYTES, MARK>(X, k0, k1); break;
-    case 7: bucket_tasks_view<7, unit_groups(7), BYTES, MARK>(X, k0, k1); break;
-    case 8: bucket_tasks_view<8, unit_groups(8), BYTES, MARK>(X, k0, k1); break;
-    case 9: bucket_tasks_view<9, unit_groups(9), BYTES, MARK>(X, k0, k1); break;
-    case 10: bucket_tasks_view<10, unit_groups(10), BYTES, MARK>(X, k0, k1); break;
-    case 11: bucket_tasks_view<11, unit_groups(11), BYTES, MARK>(X, k0, k1); break;
-    case 12: bucket_tasks_view<12, unit_groups(12), BYTES, MARK>(X, k0, k1); break;
-    case 13: bucket_tasks_view<13, unit_groups(13), BYTES, MARK>(X, k0, k1); break;
-    case 14: bucket_tasks_view<14, unit_groups(14), BYTES, MARK>(X, k0, k1); break;
-    default: bucket_tasks_view<15, unit_groups(15), BYTES, MARK>(X, k0, k1); break;
+    case 2: bucket_tasks_view<2, unit_groups(2), BYTES>(X, k0, k1); break;
+    case 3: bucket_tasks_view<3, unit_groups(3), BYTES>(X, k0, k1); break;
+    case 4: bucket_tasks_view<4, unit_groups(4), BYTES>(X, k0, k1); break;
+    case 5: bucket_tasks_view<5, unit_groups(5), BYTES>(X, k0, k1); break;
+    case 6: bucket_tasks_view<6, unit_groups(6), BYTES>(X, k0, k1); break;
+    case 7: bucket_tasks_view<7, unit_groups(7), BYTES>(X, k0, k1); break;
+    case 8: bucket_tasks_view<8, unit_groups(8), BYTES>(X, k0, k1); break;
+    case 9: bucket_tasks_view<9, unit_groups(9), BYTES>(X, k0, k1); break;
+    case 10: bucket_tasks_view<10, unit_groups(10), BYTES>(X, k0, k1); break;
+    case 11: bucket_tasks_view<11, unit_groups(11), BYTES>(X, k0, k1); break;
+    case 12: bucket_tasks_view<12, unit_groups(12), BYTES>(X, k0, k1); break;
+    case 13: bucket_tasks_view<13, unit_groups(13), BYTES>(X, k0, k1); break;
+    case 14: bucket_tasks_view<14, unit_groups(14), BYTES>(X, k0, k1); break;
+    default: bucket_tasks_view<15, unit_groups(15), BYTES>(X, k0, k1); break;
     }
 }
 
-template <bool MARK>
 __device__ __forceinline__ void run_unit(const SweepCtx &X, uint32_t L, uint32_t k0, uint32_t k1)
 {
     switch (L) {
-    case 2: bucket_tasks<2, unit_groups(2), MARK>(X, k0, k1, 32u); break;
-    case 3: bucket_tasks<3, unit_groups(3), MARK>(X, k0, k1, 32u); break;
-    case 4: bucket_tasks<4, unit_groups(4), MARK>(X, k0, k1, 32u); break;
-    case 5: bucket_tasks<5, unit_groups(5), MARK>(X, k0, k1, 32u); break;
-    case 6: bucket_tasks<6, unit_groups(6), MARK>(X, k0, k1, 32u); break;
-    case 7: bucket_tasks<7, unit_groups(7), MARK>(X, k0, k1, 32u); break;
-    case 8: bucket_tasks<8, unit_groups(8), MARK>(X, k0, k1, 32u); break;
-    case 9: bucket_tasks<9, unit_groups(9), MARK>(X, k0, k1, 32u); break;
-    case 10: bucket_tasks<10, unit_groups(10), MARK>(X, k0, k1, 32u); break;
-    case 11: bucket_tasks<11, unit_groups(11), MARK>(X, k0, k1, 32u); break;
-    case 12: bucket_tasks<12, unit_groups(12), MARK>(X, k0, k1, 32u); break;
-    case 13: bucket_tasks<13, unit_groups(13), MARK>(X, k0, k1, 32u); break;
-    case 14: bucket_tasks<14, unit_groups(14), MARK>(X, k0, k1, 32u); break;
-    default: bucket_tasks<15, unit_groups(15), MARK>(X, k0, k1, 32u); break;
+    case 2: bucket_tasks<2, unit_groups(2)>(X, k0, k1, 32u); break;
+    case 3: bucket_tasks<3, unit_groups(3)>(X, k0, k1, 32u); break;
+    case 4: bucket_tasks<4, unit_groups(4)>(X, k0, k1, 32u); break;
+    case 5: bucket_tasks<5, unit_groups(5)>(X, k0, k1, 32u); break;
+    case 6: bucket_tasks<6, unit_groups(6)>(X, k0, k1, 32u); break;
+    case 7: bucket_tasks<7, unit_groups(7)>(X, k0, k1, 32u); break;
+    case 8: bucket_tasks<8, unit_groups(8)>(X, k0, k1, 32u); break;
+    case 9: bucket_tasks<9, unit_groups(9)>(X, k0, k1, 32u); break;
+    case 10: bucket_tasks<10, unit_groups(10)>(X, k0, k1, 32u); break;
+    case 11: bucket_tasks<11, unit_groups(11)>(X, k0, k1, 32u); break;
+    case 12: bucket_tasks<12, unit_groups(12)>(X, k0, k1, 32u); break;
+    case 13: bucket_tasks<13, unit_groups(13)>(X, k0, k1, 32u); break;
+    case 14: bucket_tasks<14, unit_groups(14)>(X, k0, k1, 32u); break;
+    default: bucket_tasks<15, unit_groups(15)>(X, k0, k1, 32u); break;
     }
 }
 
@@ -970,7 +737,6 @@ __device__ __forceinline__ void run_unit(const SweepCtx &X, uint32_t L, uint32_t
 // nogood is checked every round by one warp, so the watches need no
 // per-variable lists and stay valid across backjumps.  Equal positions
 // (a nogood of one literal) always scan.
-template <bool MARK>
 __device__ __forceinline__ void classify_long(const SweepCtx &X, uint32_t id, unsigned long long &checks,
                                               uint2 *wslot)
 {
@@ -1065,7 +831,6 @@ __device__ __forceinline__ void classify_long(const SweepCtx &X, uint32_t id, un
     won = __shfl_sync(FULL_MASK, won, 0);
     if (!won) return;
     const uint32_t x = ulit >> 1;
-    if constexpr (MARK) warp_mark_units(X, x);
     if (X.cdl > 1u) {
         __threadfence_block();
         bool first = true;
@@ -1084,89 +849,115 @@ __device__ __forceinline__ void classify_long(const SweepCtx &X, uint32_t id, un
         __threadfence_block();
         view_set(X.V, x, (ulit & 1u) ? V_T : V_F);
     }
-    if constexpr (MARK) {
-        if (X.chain) {
-            __syncwarp();
-            warp_push_units(X, x);
+}
+
+// OR into acc of word w of the bitmaps of variables u[0 .. C) other than x.
+// The words are loaded beside the levels that say whether they count.
+template <int C>
+__device__ __forceinline__ unsigned long long deps_or(const Dev &D, const uint32_t (&u)[C], uint32_t x, uint32_t w)
+{
+    int32_t lev[C];
+    unsigned long long word[C], acc = 0;
+#pragma unroll
+    for (int q = 0; q < C; q++) {
+        lev[q] = u[q] != x ? __ldcg(D.dl + u[q]) : 0;
+        word[q] = u[q] != x ? __ldcg(D.deps + (size_t)u[q] * D.WW + w) : 0ull;
+    }
+#pragma unroll
+    for (int q = 0; q < C; q++)
+        if (lev[q] > 1 && 64u * w < (uint32_t)lev[q]) acc |= word[q];
+    return acc;
+}
+
+// Dependency bitmap (Section 4.2, mk_dl_bitmap) of variable x, assigned by
+// bucket nogood id, by a group of `lanes` lanes, this one the sub-th: each
+// takes every lanes-th word.  vars: the nogood's variables if it has at most eight literals and
+// they are known, else null.
+__device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t id, const uint4 *vars, uint32_t nw, uint32_t sub,
+                                            uint32_t lanes)
+{
+    const uint32_t L = ((id >> 27) & 15u) + 1u, n = D.bk_n[L];
+    if (vars && L <= 8u) {
+        const uint4 v = vars[0];
+        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+        if (L <= 4u) {
+            for (uint32_t w = sub; w < nw; w += lanes) D.deps[(size_t)x * D.WW + w] = deps_or<4>(D, u, x, w);
+        } else {
+            const uint4 t = vars[1];
+            const uint32_t u2[4] = {t.x, t.y, t.z, t.w};
+            for (uint32_t w = sub; w < nw; w += lanes) D.deps[(size_t)x * D.WW + w] = deps_or<4>(D, u, x, w) | deps_or<4>(D, u2, x, w);
         }
+        return;
+    }
+    const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
+    for (uint32_t w = sub; w < nw; w += lanes) {
+        unsigned long long acc = 0;
+        for (uint32_t q0 = 0; q0 < L; q0 += 5u) {
+            uint32_t u[5];
+#pragma unroll
+            for (uint32_t q = 0; q < 5u; q++) u[q] = q0 + q < L ? __ldg(base + (size_t)(q0 + q) * n) >> 1 : x;
+            acc |= deps_or<5>(D, u, x, w);
+        }
+        D.deps[(size_t)x * D.WW + w] = acc;
     }
 }
 
-// Frontier round: only the bucket nogoods that contain a variable of the
-// trail entries [fr0, fr1) (the previous round's assignments), or this
-// phase's decision variable X.dec_v when there is one, can have become unit
-// or violated since the last round; every other bucket nogood is as the
-// last sweep left it.  One warp per variable (round-robin over CTAs first),
-// one lane per nogood of its occurrence list, classified against the global
-// codes (this round's claims read as unassigned; the decision variable,
-// whose code the leader may still be writing, as true).
-__device__ __forceinline__ void frontier_round(const SweepCtx &X, uint32_t fr0, uint32_t fr1, unsigned long long &checks)
+// The bucket nogoods of the literals on the trail entries [fr0, fr1) (the
+// claims of the round before), by the whole grid: only these can have become
+// unit or violated.  A warp takes up to eight entries (fewer when there are
+// fewer than eight a warp) and its quads share out their lists; values are the
+// global codes, with this round's claims unseen.  The fresh bits of the entries
+// are cleared meanwhile.  For more claims than one CTA follows well and fewer
+// than make a sweep of the store worth its bytes (Dev::list_max): on the 400k
+// program a sweep takes 56 us, a round over 20k claims about 8 us.
+__device__ __forceinline__ void list_round(const SweepCtx &X, uint32_t fr0, uint32_t fr1, uint32_t &checks, uint32_t &visits)
 {
     const Dev &D = *X.D;
-    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t lane = threadIdx.x & 31u, sub = lane & 3u, quad = lane & 28u, n = fr1 - fr0;
     const uint32_t wpc = blockDim.x >> 5, slot = (X.gw % wpc) * (X.nw / wpc) + X.gw / wpc;
-    const bool dec = X.dec_v != 0xFFFFFFFFu;
-    const uint32_t count = dec ? 1u : fr1 - fr0;
-    for (uint32_t i = slot; i < count; i += X.nw) {
-        const uint32_t v = dec ? X.dec_v : __ldcg(D.trail + fr0 + i) & TRAIL_VAR;
-        if (v >= D.nv) continue;
-        const uint32_t o0 = __ldg(D.occ_off + 2u * v), o1 = __ldg(D.occ_off + 2u * v + 2u);
-        for (uint32_t ob = o0; ob < o1; ob += 32u) {
-            const uint32_t o = ob + lane;
-            const bool has = o < o1;
-            const uint32_t id = has ? __ldg(&D.occ[o].w[0]) : 0u;
-            const uint32_t L = has ? ((id >> 27) & 15u) + 1u : 0u, k = id & 0x7FFFFFFu;
-            const uint32_t *base = has ? D.lits + D.bk_base[L] + k : D.lits;
-            const uint32_t n = has ? D.bk_n[L] : 0u;
-            uint32_t lit[BUCKET_MAX];
-#pragma unroll
-            for (int q = 0; q < BUCKET_MAX; q++) lit[q] = (uint32_t)q < L ? __ldg(base + (size_t)q * n) : 0u;
-            bool sat = false;
-            uint32_t n_un = 0, ul = 0;
-#pragma unroll
-            for (int q = 0; q < BUCKET_MAX; q++) {
-                if ((uint32_t)q >= L) continue;
-                const uint32_t u = lit[q] >> 1;
-                const uint32_t val = u == X.dec_v ? V_T : global_val(D, u, X.fresh);
-                sat |= val == ((lit[q] & 1u) ? V_T : V_F);
-                if (val == 0u) { n_un++; ul = lit[q]; }
-            }
-            checks += L;
-            bool won = false;
-            uint32_t x = 0, valbit = 0;
-            if (has && !sat && n_un == 0u) {
-                report_conflict(X, id, L);
-            } else if (has && !sat && n_un == 1u) {
-                if (!X.do_claim) {
-                    atomicAdd(&X.acc->flag, 1u);
-                } else {
-                    x = ul >> 1;
-                    valbit = (ul & 1u) ? V_T : V_F;
-                    const int r = claim_var(D.asg, x, valbit, X.fresh);
-                    if (r == 2) report_conflict(X, id, L);
-                    else if (r == 0) { record_claim(X, x, valbit, id); won = true; }
-                }
-            }
-            if (X.cdl > 1u) {
-                unsigned m = __ballot_sync(FULL_MASK, won);
-                if (m) {
-                    while (m) {
-                        const int src = __ffs(m) - 1;
-                        m &= m - 1u;
-                        uint32_t var[BUCKET_MAX];
-#pragma unroll
-                        for (int q = 0; q < BUCKET_MAX; q++) var[q] = __shfl_sync(FULL_MASK, lit[q], src) >> 1;
-                        warp_deps_dyn(X, var, __shfl_sync(FULL_MASK, L, src), __shfl_sync(FULL_MASK, x, src));
-                    }
-                    __threadfence_block();
-                    __syncwarp();
-                }
-            }
-            if (won && X.use_view) {
-                __threadfence_block();
-                view_set(X.V, x, valbit);
+    const uint32_t each = min(8u, (n + X.nw - 1u) / X.nw), nw = X.cdl > 1u ? deps_words(D, X.cdl) : 0u;
+    const Codes<false> codes{D.asg};
+    for (uint32_t i0 = slot * each; i0 < n; i0 += X.nw * each) {
+        const uint32_t i = i0 + lane;
+        uint32_t y = 0, o0 = 0, c = 0;
+        if (lane < each && i < n) {
+            const uint32_t e = __ldcg(D.trail + fr0 + i), l = mk_lit(e & TRAIL_VAR, (e & TRAIL_F) != 0u);
+            if ((l >> 1) < D.nv) {
+                y = l >> 1;
+                o0 = __ldg(D.occ_off + l);
+                c = __ldg(D.occ_off + l + 1u) - o0;
             }
         }
+        warp_lists(o0, c, [&](uint32_t o, uint32_t li) {
+            const uint32_t yo = __shfl_sync(FULL_MASK, y, li);
+            const QuadCheck r = quad_check(D, codes, X.fresh, o);
+            const uint32_t x = r.ul >> 1, valbit = (r.ul & 1u) ? V_T : V_F;
+            uint32_t won = 0;
+            if (sub == 0u && o != 0xFFFFFFFFu) {
+                const uint32_t L = ((r.id >> 27) & 15u) + 1u;
+                checks += L;
+                visits++;
+                if (!r.sat && r.n_un < 2u) {
+                    const int k = r.n_un == 0u ? 2 : claim_var(D.asg, x, valbit, X.fresh);
+                    if (k == 2) report_conflict(X, r.id, L);
+                    else if (k == 0) { record_claim(X, x, valbit, r.id); won = 1u; }
+                }
+            }
+            if (!nw) return;
+            won = __shfl_sync(FULL_MASK, won, quad);
+            if (!__any_sync(FULL_MASK, won)) return;
+            // the claim's bitmap by its quad, from the words of the occurrence
+            uint32_t u[8];
+#pragma unroll
+            for (uint32_t q = 0; q < 8u; q++) u[q] = __shfl_sync(FULL_MASK, r.l[q & 1u], quad + (q >> 1));
+#pragma unroll
+            for (uint32_t q = 0; q < 8u; q++) u[q] = q == 0u ? yo : u[q] == PAD_LIT ? x : u[q] >> 1;
+            if (won) {
+                const uint4 v[2] = {make_uint4(u[0], u[1], u[2], u[3]), make_uint4(u[4], u[5], u[6], u[7])};
+                narrow_deps(D, x, r.id, r.len ? nullptr : v, nw, sub, 4u);
+            }
+            __syncwarp();
+        });
     }
 }
 
@@ -1177,7 +968,6 @@ __device__ __forceinline__ void unit_table(const Dev &D, uint32_t cta, bool list
     if (threadIdx.x != 0) return;
     s_unit = 0u;
     s_ncl = 0u;
-    s_nq = 0u;
     s_unit2[0] = 0u;
     s_unit2[1] = 0u;
     if (lists) return;
@@ -1195,12 +985,10 @@ __device__ __forceinline__ void unit_table(const Dev &D, uint32_t cta, bool list
 }
 
 // Propagate-and-check over this CTA's ranges of every bucket (full), or
-// over the frontier -- the nogoods of the previous round's assignments
-// (frontier = 1) or the dirty bucket units (frontier = 2), taken from the
-// CTA's queue (DQ = 1) -- then (grid-wide) the static long nogoods and the
-// learned nogoods.  DQ = 2: the latter alone (the bucket nogoods are followed
-// through the occurrence lists).
-template <int DQ>
+// over the lists of the trail entries [fr0, fr1) (list_round), then (grid-wide)
+// the static long nogoods and the learned nogoods.  ONLY_LONG: the latter
+// alone (one CTA follows the bucket nogoods in narrow rounds).
+template <bool ONLY_LONG>
 __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bool full = true,
                                       uint32_t fr0 = 0u, uint32_t fr1 = 0u, uint32_t pass = 0u)
 {
@@ -1234,23 +1022,6 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
     }
     const uint32_t *const ubase = s_ubase;     // set up once per launch (unit_table)
     uint32_t units = full ? ubase[BUCKET_MAX + 1] : 0u;
-    // frontier by units: the queue (or, if it overflowed, every unit of the
-    // CTA); the literals and nogoods of the units checked are counted here
-    bool queued = false, count_units = false;
-    if constexpr (DQ == 1) {
-        if (!full && D.frontier >= 2u) {
-            const uint32_t nq = s_nq;
-            queued = nq <= DQ_CAP;
-            units = queued ? nq : ubase[BUCKET_MAX + 1];
-            count_units = true;
-            X.chain = queued && D.frontier == 3u;
-        }
-    }
-    // frontier = 3: waves of the queue; wave w pops positions [lo, units)
-    // with its own counter, and the units claims of wave w queued form wave
-    // w + 1 (up to DQ_WAVES waves)
-    uint32_t wave = 0u, lo = 0u;
-    unsigned long long uvisits = 0;
     // Long and learned nogoods first (one warp each, round-robin over CTAs
     // first, then over the warps of a CTA); the warps that take one then
     // take fewer bucket units from the queue.
@@ -1259,41 +1030,14 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
     const uint32_t wpc = blockDim.x >> 5, slot = (X.gw % wpc) * (X.nw / wpc) + X.gw / wpc;
     for (uint32_t i = slot; i < nl; i += X.nw) {
         uint32_t id = i < D.n_long ? __ldg(D.long_ids + i) : __ldcg(D.learned_ids + (i - D.n_long));
-        classify_long<(DQ == 1)>(X, id, checks, D.nwatch ? D.nwatch + i : nullptr);
+        classify_long(X, id, checks, D.nwatch ? D.nwatch + i : nullptr);
     }
     const unsigned long long t1 = wtimer ? globaltimer_ns() : 0ull;
-    for (; DQ != 2;) {
+    while (!ONLY_LONG) {
         uint32_t u = 0;
-        {
-            if (lane == 0) {
-                if constexpr (DQ == 1) u = X.chain ? lo + atomicAdd(&s_wave[wave], 1u) : atomicAdd(uctr, 1u);
-                else u = atomicAdd(uctr, 1u);
-            }
-            u = __shfl_sync(FULL_MASK, u, 0);
-            if (u >= units) {
-                if constexpr (DQ == 1) {
-                    if (X.chain && wave + 1u < DQ_WAVES) {
-                        // every warp of the CTA arrives here once per wave;
-                        // the queue's length is read between two barriers, so
-                        // no warp pushes while it is read
-                        cta_sync();
-                        if (threadIdx.x == 0) s_ub[2] = min(s_nq, DQ_CAP);
-                        cta_sync();
-                        const uint32_t nq = s_ub[2];
-                        if (nq > units) {
-                            lo = units;
-                            units = nq;
-                            wave++;
-                            continue;
-                        }
-                    }
-                }
-                break;
-            }
-            if constexpr (DQ == 1) {
-                if (queued) u = s_dq[u];
-            }
-        }
+        if (lane == 0) u = atomicAdd(uctr, 1u);
+        u = __shfl_sync(FULL_MASK, u, 0);
+        if (u >= units) break;
         uint32_t L = 2;
 #pragma unroll
         for (uint32_t q = 3; q <= (uint32_t)BUCKET_MAX; q++)
@@ -1301,22 +1045,19 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
         const uint32_t first = ubase[L];
         const uint32_t b0 = s_krange[L][0], b1 = s_krange[L][1];
         const uint32_t k0 = b0 + (u - first) * unit_groups(L) * 32u;
-        if (D.view_mode == VIEW_BYTES) run_unit_view<true, (DQ == 1)>(X, L, k0, b1);
-        else if (D.view_mode == VIEW_PACKED) run_unit_view<false, (DQ == 1)>(X, L, k0, b1);
-        else run_unit<(DQ == 1)>(X, L, k0, b1);
-        if (count_units && lane == 0) {
-            const uint32_t n = min(b1 - k0, unit_groups(L) * 32u);
-            checks += (unsigned long long)L * n;
-            uvisits += n;
-        }
+        if (D.view_mode == VIEW_BYTES) run_unit_view<true>(X, L, k0, b1);
+        else if (D.view_mode == VIEW_PACKED) run_unit_view<false>(X, L, k0, b1);
+        else run_unit(X, L, k0, b1);
     }
-    if (DQ != 2 && !full && D.frontier == 1u && fr0 != fr1) {
-        unsigned long long fchecks = 0;           // per lane (classify_long's are per warp)
-        frontier_round(X, fr0, fr1, fchecks);
-        checks += __reduce_add_sync(FULL_MASK, (unsigned)fchecks);
+    uint32_t uvisits = 0;
+    if (!ONLY_LONG && fr0 < fr1) {
+        uint32_t c = 0, v = 0;
+        list_round(X, fr0, fr1, c, v);
+        checks += __reduce_add_sync(FULL_MASK, c);
+        uvisits = __reduce_add_sync(FULL_MASK, v);
     }
     if (lane == 0 && checks) atomicAdd(&X.acc->checks, checks);
-    if (lane == 0 && uvisits) atomicAdd(&X.acc->visits, uvisits);
+    if (lane == 0 && uvisits) atomicAdd(&X.acc->visits, (unsigned long long)uvisits);
     if (wtimer) {
         const unsigned long long t2 = globaltimer_ns();
         if (timer) {
@@ -1332,16 +1073,10 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
         cta_sync();
         const uint32_t n = min(s_ncl, CLAIM_BUF);
         if (threadIdx.x == 0) {
-            s_unit = 0u; s_nq = 0u;                  // every warp has left the unit queue
+            s_unit = 0u;                             // every warp has left the unit queue
             atomicMax(&X.acc->tlong, s_wmax[0]);
             atomicMax(&X.acc->tbuck, s_wmax[1]);
             s_wmax[0] = s_wmax[1] = 0ull;
-        }
-        if constexpr (DQ == 1) {
-            if (X.chain) {
-                for (uint32_t w = threadIdx.x; w < DQ_BITS / 32u; w += blockDim.x) s_dqbits[w] = 0u;
-                if (threadIdx.x < DQ_WAVES) s_wave[threadIdx.x] = 0u;
-            }
         }
         if (threadIdx.x < 32u) {
             uint32_t base = 0;
@@ -2078,56 +1813,6 @@ __device__ __forceinline__ void narrow_queue(Queue &Q, uint32_t buf, uint32_t sl
     }
 }
 
-// OR into acc of word w of the bitmaps of variables u[0 .. C) other than x.
-// The words are loaded beside the levels that say whether they count.
-template <int C>
-__device__ __forceinline__ unsigned long long deps_or(const Dev &D, const uint32_t (&u)[C], uint32_t x, uint32_t w)
-{
-    int32_t lev[C];
-    unsigned long long word[C], acc = 0;
-#pragma unroll
-    for (int q = 0; q < C; q++) {
-        lev[q] = u[q] != x ? __ldcg(D.dl + u[q]) : 0;
-        word[q] = u[q] != x ? __ldcg(D.deps + (size_t)u[q] * D.WW + w) : 0ull;
-    }
-#pragma unroll
-    for (int q = 0; q < C; q++)
-        if (lev[q] > 1 && 64u * w < (uint32_t)lev[q]) acc |= word[q];
-    return acc;
-}
-
-// Dependency bitmap (Section 4.2, mk_dl_bitmap) of variable x, assigned by
-// bucket nogood id, by the 8 lanes `sub` of a group: each takes every eighth
-// word.  vars: the nogood's variables if it has at most eight literals and
-// they are known, else null.
-__device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t id, const uint4 *vars, uint32_t nw, uint32_t sub)
-{
-    const uint32_t L = ((id >> 27) & 15u) + 1u, n = D.bk_n[L];
-    if (vars && L <= 8u) {
-        const uint4 v = vars[0];
-        const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-        if (L <= 4u) {
-            for (uint32_t w = sub; w < nw; w += 8u) D.deps[(size_t)x * D.WW + w] = deps_or<4>(D, u, x, w);
-        } else {
-            const uint4 t = vars[1];
-            const uint32_t u2[4] = {t.x, t.y, t.z, t.w};
-            for (uint32_t w = sub; w < nw; w += 8u) D.deps[(size_t)x * D.WW + w] = deps_or<4>(D, u, x, w) | deps_or<4>(D, u2, x, w);
-        }
-        return;
-    }
-    const uint32_t *base = D.lits + D.bk_base[L] + (id & 0x7FFFFFFu);
-    for (uint32_t w = sub; w < nw; w += 8u) {
-        unsigned long long acc = 0;
-        for (uint32_t q0 = 0; q0 < L; q0 += 5u) {
-            uint32_t u[5];
-#pragma unroll
-            for (uint32_t q = 0; q < 5u; q++) u[q] = q0 + q < L ? __ldg(base + (size_t)(q0 + q) * n) >> 1 : x;
-            acc |= deps_or<5>(D, u, x, w);
-        }
-        D.deps[(size_t)x * D.WW + w] = acc;
-    }
-}
-
 // What a round counts and where its claims go.
 struct NarrowRound {
     uint32_t cdl, fresh, buf, slot, out;      // buf, slot: of the next round's queue; out: trail index of its first claim
@@ -2203,10 +1888,10 @@ __device__ __forceinline__ void narrow_bitmaps(const Dev &D, const Queue &Q, uin
     for (uint32_t i = i0; i < n; i += step) {
         if (i < Queue::N) {
             const uint4 c = Q.e[buf][i];
-            narrow_deps(D, c.x & TRAIL_VAR, c.y, &Q.u[buf][i][0], nw, threadIdx.x & 7u);
+            narrow_deps(D, c.x & TRAIL_VAR, c.y, &Q.u[buf][i][0], nw, threadIdx.x & 7u, 8u);
         } else {
             const uint32_t x = __ldcg(D.trail + qs + i) & TRAIL_VAR;
-            narrow_deps(D, x, __ldcg(D.reason + x), nullptr, nw, threadIdx.x & 7u);
+            narrow_deps(D, x, __ldcg(D.reason + x), nullptr, nw, threadIdx.x & 7u, 8u);
         }
     }
 }
@@ -2219,8 +1904,8 @@ __device__ __forceinline__ void narrow_bitmaps(const Dev &D, const Queue &Q, uin
 // list for the literal that now holds -- only those nogoods can have become
 // unit or violated -- and claims become the next round's entries, at
 // tbase, tbase + 1, ... of the trail.  Ends when a round claims nothing, on a
-// conflict, or when a round claims more than D.narrow_max (a sweep by every CTA
-// is then the faster way).
+// conflict, or when a round claims more than D.narrow_max (every CTA following
+// a part is then the faster way).
 //
 // Why: a search round assigns a few dozen variables (62 on average in the
 // 100k-atom program), and a sweep round costs its chain of barriers and loads
@@ -2346,10 +2031,9 @@ __device__ __forceinline__ void injected_stall(const Dev &D)
 // Algorithm 1 on the device.  rank/size: thread index and thread count of
 // the solving group; cta: this CTA's part of the program's static partition;
 // cta0/leader: the CTA and thread that run conflict analysis and write the
-// next control block.  UNITS: compiled with the frontier by units (used by
-// programs with frontier = 2; the kernels without it keep the sweeps free of
-// the unit marks).
-template <bool BATCH, bool UNITS, bool LISTS>
+// next control block.  LISTS: bucket nogoods are followed through the
+// occurrence lists only, as in programs with D.lists (no sweep code, no view).
+template <bool BATCH, bool LISTS>
 __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const View &V, uint32_t rank,
                                             uint32_t size, bool cta0, bool leader, uint32_t cta)
 {
@@ -2381,15 +2065,6 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
     cta_sync();
     if (!lists) view_reload(D, V, 4u << (sC.round & 1u));
     unit_table(D, cta, lists);
-    if constexpr (UNITS && !BATCH) {
-        // frontier by units: the CTA's unit range, no unit queued yet
-        if (threadIdx.x == 0 && D.frontier >= 2u) {
-            s_ub[0] = __ldg(D.cta_ubase + cta);
-            s_ub[1] = __ldg(D.cta_ubase + cta + 1u);
-            for (uint32_t w = 0; w < DQ_BITS / 32u; w++) s_dqbits[w] = 0u;
-            for (uint32_t w = 0; w < DQ_WAVES; w++) s_wave[w] = 0u;
-        }
-    }
     cta_sync();
 
     for (uint32_t k = 0;; k++) {
@@ -2416,10 +2091,10 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
         // the propagate-and-check sweep of ROUND and APPLY runs after the
         // switch (one copy of its code)
         bool sw = false, sw_full = true, nar = false;
-        uint32_t sw_cdl = 0, sw_tbase = 0, sw_dec = 0xFFFFFFFFu, sw_fr0 = 0, sw_fr1 = 0;
+        uint32_t sw_cdl = 0, sw_tbase = 0, sw_fr0 = 0, sw_fr1 = 0;
         switch (C.op) {
         case OP_INIT: {
-            SweepCtx X{&D, V, fresh_cur, 1u, tend, acc, true, false, 0xFFFFFFFFu, cta, rank >> 5, size >> 5};
+            SweepCtx X{&D, V, fresh_cur, 1u, tend, acc, true, false, cta, rank >> 5, size >> 5};
             if (leader && D.heuristic == 5) reinterpret_cast<float *>(D.act)[D.J] = 1.0f;   // the first increment
             for (uint32_t i = gtid; i < D.n_units; i += nthreads) {
                 uint32_t id = D.units_base + i;
@@ -2526,10 +2201,9 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             }
             // without sweeps the caller's partial assignment is followed too
             const bool input = lists && D.mode == MODE_PROPAGATE && C.round == 1u;
-            const bool quiet = (A.nclaim == 0u || C.chased) && !input;   // no assignment is left to follow
+            const bool quiet = A.nclaim == 0u && !input;   // no assignment is left to follow
             if (quiet && C.clean) {
                 // fixpoint
-                if (leader) N.tb = tend;
                 if (D.mode == MODE_PROPAGATE) {
                     if (leader) { N.op = OP_DONE; N.status = 0; }
                     break;
@@ -2549,33 +2223,32 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 if (leader) atomicAdd(&D.stats->props, (unsigned long long)A.nclaim);
                 break;
             }
-            // frontier by units: this round's dirty units of the CTA
-            if constexpr (UNITS && !BATCH) {
-                if (D.frontier >= 2u) build_unit_queue(D, cta, D.dirty + (C.round & 1u) * D.dirty_words, 0xFFFFFFFFu);
-            }
+            // a full sweep, or the claims' lists, by the whole grid
+            sw_full = !lists && (C.full != 0u || (D.frontier == 0u && quiet) || (!quiet && A.nclaim > D.list_max));
             // make last round's claims visible: clear their fresh bit
-            // (grid-wide) and put them in this CTA's view
-            for (uint32_t i = (C.chased ? tend : C.tb) + gtid; i < tend; i += nthreads) {
+            // (grid-wide) and put them in this CTA's view, which only sweeps
+            // read
+            for (uint32_t i = (quiet ? tend : C.tb) + gtid; i < tend; i += nthreads) {
                 uint32_t v = __ldcg(D.trail + i) & TRAIL_VAR;
                 if (v >= D.nv) { atomicExch(&D.bar->err, 2u); continue; }   // corrupt trail: stop with an error
                 atomicAnd(D.asg + (v >> 3), ~(fresh_prev << ((v & 7u) * 4u)));
             }
-            if (lists) {
-                // no view
-            } else if (tend - C.tc > 4096u) {
-                view_reload(D, V, fresh_cur);
-            } else {
-                for (uint32_t i = C.tc + threadIdx.x; i < tend; i += blockDim.x) {
-                    const uint32_t e = __ldcg(D.trail + i);
-                    view_set(V, e & TRAIL_VAR, (e & TRAIL_F) ? V_F : V_T);
+            if (sw_full) {
+                if (tend - C.tc > 4096u) {
+                    view_reload(D, V, fresh_cur);
+                } else {
+                    for (uint32_t i = C.tc + threadIdx.x; i < tend; i += blockDim.x) {
+                        const uint32_t e = __ldcg(D.trail + i);
+                        view_set(V, e & TRAIL_VAR, (e & TRAIL_F) ? V_F : V_T);
+                    }
                 }
             }
             cta_sync();
             sw = true; sw_cdl = C.cdl; sw_tbase = tend;
-            sw_full = !lists && (C.full != 0u || D.frontier == 0u || (!UNITS && D.frontier >= 2u));
-            sw_fr0 = C.chased ? tend : C.tb; sw_fr1 = tend;
+            if (!sw_full && !quiet) { sw_fr0 = C.tb; sw_fr1 = tend; }
             if (leader) {
-                N.op = OP_ROUND; N.round = C.round + 1u; N.tc = tend; N.tb = tend; N.tcom = tend; N.clean = 1; N.full = 0; N.chased = 0;
+                N.op = OP_ROUND; N.round = C.round + 1u; N.tc = sw_full ? tend : C.tc; N.tb = tend; N.tcom = tend; N.full = 0;
+                N.clean = lists || D.frontier != 0u || sw_full;
                 atomicAdd(&D.stats->rounds, 1ull);
                 atomicAdd(&D.stats->props, (unsigned long long)A.nclaim);
                 if (sw_full) atomicAdd(&D.stats->checks, D.static_checks);
@@ -2588,7 +2261,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 // CompleteAssignment: falsify the unassigned atoms; their
                 // dependency bitmap is every decision level so far
                 kind = 2;
-                SweepCtx X{&D, V, fresh_cur, C.cdl, tend, acc, true, false, 0xFFFFFFFFu, cta, rank >> 5, size >> 5};
+                SweepCtx X{&D, V, fresh_cur, C.cdl, tend, acc, true, false, cta, rank >> 5, size >> 5};
                 const uint32_t nw = deps_words(D, C.cdl);
                 for (uint32_t p = gtid; p < D.na; p += nthreads) {
                     if ((nib(__ldcg(D.asg + (p >> 3)), p) & 3u) != 0u) continue;
@@ -2600,10 +2273,8 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                     }
                 }
                 if (leader) {
-                    // (frontier by units: completion claims mark no units, so
-                    // the next round sweeps everything)
-                    N.op = OP_ROUND; N.round = C.round + 1u; N.tb = tend; N.tcom = tend; N.clean = 0; N.chased = 0;
-                    N.full = D.frontier >= 2u ? 1u : 0u;
+                    N.op = OP_ROUND; N.round = C.round + 1u; N.tb = tend; N.tcom = tend; N.clean = 0;
+                    N.full = 0;
                     atomicAdd(&D.stats->completions, 1ull);
                 }
                 break;
@@ -2630,33 +2301,12 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 __threadfence();
                 atomicOr(D.asg + (bv >> 3), V_T << ((bv & 7u) * 4u));
             }
-            if (lists || D.narrow_max) {
-                // the decision's consequences by narrow rounds: the store is at
-                // a fixpoint, so only the decision's nogoods can change it
-                nar = true; sw_cdl = L; sw_fr0 = tend; sw_fr1 = sw_tbase = tend + 1u;
-                if (leader) {
-                    N.cdl = L;
-                    atomicAdd(&D.stats->decisions, 1ull);
-                    if ((unsigned long long)L > D.stats->max_level) D.stats->max_level = L;
-                }
-                break;
-            }
-            if (threadIdx.x == 0) view_set(V, bv, V_T);
-            if (UNITS && D.frontier >= 2u) {
-                if constexpr (UNITS && !BATCH) {
-                    build_unit_queue(D, cta, D.dirty + (C.round & 1u) * D.dirty_words, bv);
-                }
-            }
-            cta_sync();
-            sw = true; sw_cdl = L; sw_tbase = tend + 1u; sw_dec = bv;
-            sw_full = D.frontier == 0u || (!UNITS && D.frontier >= 2u);
+            // the decision's consequences by narrow rounds: the store is at a
+            // fixpoint, so only the decision's nogoods can change it
+            nar = true; sw_cdl = L; sw_fr0 = tend; sw_fr1 = sw_tbase = tend + 1u;
             if (leader) {
-                N.op = OP_ROUND; N.cdl = L; N.round = C.round + 1u; N.tc = tend + 1u; N.tb = tend + 1u;
-                N.tcom = tend + 1u; N.clean = 0; N.full = 0; N.chased = 0;
+                N.cdl = L;
                 atomicAdd(&D.stats->decisions, 1ull);
-                atomicAdd(&D.stats->rounds, 1ull);
-                if (sw_full) atomicAdd(&D.stats->checks, D.static_checks);
-                atomicAdd(&D.stats->visits, (sw_full ? D.static_nogoods : 0ull) + D.n_long + C.n_learned);
                 if ((unsigned long long)L > D.stats->max_level) D.stats->max_level = L;
             }
             break;
@@ -2674,7 +2324,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 for (uint32_t i = newend + threadIdx.x; i < tend; i += blockDim.x)
                     view_clear(V, __ldcg(D.trail + i) & TRAIL_VAR);
             if (leader) {
-                N.op = OP_ROUND; N.cdl = C.target; N.tc = min(C.tc, newend); N.tb = newend; N.tcom = newend; N.clean = 0; N.full = 1; N.chased = 0;
+                N.op = OP_ROUND; N.cdl = C.target; N.tc = min(C.tc, newend); N.tb = newend; N.tcom = newend; N.clean = 0; N.full = 1;
             }
             break;
         }
@@ -2856,18 +2506,18 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 ? narrow_rounds<true>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left)
                 : narrow_rounds<false>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left);
             if (leader) {
-                N.op = OP_ROUND; N.round = C.round + its; N.tb = sw_tbase; N.tcom = sw_tbase + n - left;
-                N.chased = left == 0u; N.full = left != 0u;
+                // the trail's last `left` claims are still to be followed
+                N.op = OP_ROUND; N.round = C.round + its; N.tb = N.tcom = sw_tbase + n - left; N.full = 0;
                 N.clean = (lists || D.frontier != 0u) && D.n_long + C.n_learned == 0u;
-                acc->nclaim = n;
+                acc->nclaim = left;
+                atomicAdd(&D.stats->props, (unsigned long long)(n - left));
                 atomicAdd(&D.stats->rounds, (unsigned long long)its);
             }
         }
         if (sw) {
             const unsigned long long ts = threadIdx.x == 0 ? globaltimer_ns() : 0ull;
-            SweepCtx X{&D, V, fresh_cur, sw_cdl, sw_tbase, acc, true, !lists, sw_dec, cta, rank >> 5, size >> 5};
-            if (UNITS && !lists && D.frontier >= 2u) X.dmark = D.dirty + ((C.round + 1u) & 1u) * D.dirty_words;
-            sweep<LISTS ? 2 : UNITS ? 1 : 0>(X, C.n_learned, sw_full, sw_fr0, sw_fr1);
+            SweepCtx X{&D, V, fresh_cur, sw_cdl, sw_tbase, acc, true, !lists, cta, rank >> 5, size >> 5};
+            sweep<LISTS>(X, C.n_learned, sw_full, sw_fr0, sw_fr1);
             if (threadIdx.x == 0) atomicMax(&acc->tsweep, globaltimer_ns() - ts);
         }
 

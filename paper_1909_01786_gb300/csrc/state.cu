@@ -42,8 +42,6 @@ __global__ void __launch_bounds__(256) reset_kernel(Dev D, bool codes, uint32_t 
     }
     for (uint32_t j = t; j < D.J + 2u; j += nt) D.act[j] = 0u;
     for (uint32_t j = t; j < D.J + 4u; j += nt) D.level_start[j] = 0u;
-    if (D.dirty)
-        for (uint32_t w = t; w < 2u * D.dirty_words; w += nt) D.dirty[w] = 0u;
     if (t == 0) first_control(D, n_input);
 }
 
@@ -228,7 +226,52 @@ __global__ void __launch_bounds__(256) occ_fill_kernel(Dev D, uint32_t n_lits, R
     }
 }
 
+// Where each program's models go in the packed words (-1: they do not fit,
+// or there are none), by one block: a scan over the programs in order.
+__global__ void __launch_bounds__(256) pack_places_kernel(const Dev *devs, uint32_t n, const long long *results, long long *places,
+                                                          long long packed)
+{
+    __shared__ long long s_w[256];
+    long long run = 0;
+    for (uint32_t i0 = 0; i0 < n; i0 += 256u) {
+        const uint32_t i = i0 + threadIdx.x;
+        const long long words = i < n ? min(results[4ull * i + 1], devs[i].models_cap) * (long long)((devs[i].na + 63u) / 64u) : 0;
+        s_w[threadIdx.x] = words;
+        __syncthreads();
+        for (uint32_t d = 1; d < 256u; d <<= 1) {
+            const long long x = threadIdx.x >= d ? s_w[threadIdx.x - d] : 0;
+            __syncthreads();
+            s_w[threadIdx.x] += x;
+            __syncthreads();
+        }
+        const long long end = run + s_w[threadIdx.x];
+        if (i < n) places[i] = words > 0 && end <= packed ? end - words : -1;
+        run += s_w[255];
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(128) pack_models_kernel(const Dev *devs, uint32_t n, const long long *results, const long long *places,
+                                                          unsigned long long *models)
+{
+    for (uint32_t i = blockIdx.x; i < n; i += gridDim.x) {
+        if (places[i] < 0) continue;
+        const long long words = min(results[4ull * i + 1], devs[i].models_cap) * (long long)((devs[i].na + 63u) / 64u);
+        for (long long w = threadIdx.x; w < words; w += blockDim.x) models[places[i] + w] = devs[i].models[w];
+    }
+}
+
 }  // namespace
+
+// After a batch: every program's models into one array, so that one copy
+// brings them to the host.
+cudaError_t launch_batch_pack(const Dev *devs, uint32_t n, const long long *results, long long *places,
+                              unsigned long long *models, int64_t packed, cudaStream_t st)
+{
+    pack_places_kernel<<<1, 256, 0, st>>>(devs, n, results, places, packed);
+    pack_models_kernel<<<(int)std::min<uint32_t>(n, 1216u), 128, 0, st>>>(devs, n, results, places, models);
+    return cudaGetLastError();
+}
 
 // Words of the rows of the bucket nogoods of more than eight literals.
 uint32_t row_words(const Dev &D)
@@ -264,7 +307,7 @@ cudaError_t launch_occurrences(const Dev &D, uint32_t n_lits, uint32_t *off, Occ
 
 cudaError_t launch_reset(const Dev &D, bool codes, cudaStream_t st)
 {
-    const uint32_t n = std::max(std::max(codes ? D.nv : 0u, D.J + 4u), 2u * (D.dirty ? D.dirty_words : 0u));
+    const uint32_t n = std::max(codes ? D.nv : 0u, D.J + 4u);
     reset_kernel<<<(int)std::min<uint32_t>((n + 255u) / 256u, 1216u), 256, 0, st>>>(D, codes, 0u);
     return cudaGetLastError();
 }
