@@ -80,9 +80,81 @@ __device__ __forceinline__ QuadCheck quad_check(const Dev &D, const C &codes, ui
     return r;
 }
 
+// The same by one lane, for rounds with many occurrences: a warp checks 32 at
+// a time with about the instructions of a quad's eight, but each lane reads
+// its literals one after another.
+struct LaneCheck {
+    uint32_t id, len, n_un, ul;
+    bool sat;
+    uint32_t l[7];      // of at most eight literals: the others (PAD_LIT: none)
+};
+
+template <class C>
+__device__ __forceinline__ void lane_classify(const C &codes, uint32_t fresh, uint32_t l, uint32_t word, LaneCheck &r)
+{
+    if (l == PAD_LIT) return;
+    const uint32_t c = word >> ((l >> 1 & 7u) * 4u);
+    if ((c & 3u) == 0u || (c & fresh)) { r.n_un++; r.ul = l; }
+    else r.sat |= (c & 3u) == ((l & 1u) ? V_T : V_F);
+}
+
+template <class C>
+__device__ __forceinline__ LaneCheck lane_check(const Dev &D, const C &codes, uint32_t fresh, uint32_t o)
+{
+    const uint4 *e = reinterpret_cast<const uint4 *>(D.occ + o);
+    const uint4 a = __ldg(e), b = __ldg(e + 1);
+    LaneCheck r{};
+    r.id = a.x;
+    if (a.y & END_BIT) {
+        r.len = a.y & 15u;
+        for (uint32_t q = 0; q < r.len && !r.sat && r.n_un < 2u; q++) {
+            const uint32_t l = __ldg(D.rows + a.z + q);
+            lane_classify(codes, fresh, l, codes.get(l >> 4), r);
+        }
+        return r;
+    }
+    const uint32_t l[7] = {a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+    uint32_t w[7];
+#pragma unroll
+    for (int q = 0; q < 7; q++) w[q] = l[q] != PAD_LIT ? codes.get(l[q] >> 4) : 0u;
+#pragma unroll
+    for (int q = 0; q < 7; q++) {
+        lane_classify(codes, fresh, l[q], w[q], r);
+        r.l[q] = l[q];
+    }
+    return r;
+}
+
+// Calls f(o, i) for every occurrence o of up to 32 lists, the lanes of the
+// warp taking one each at a time: lane i holds list i as [o0, o0 + c).
+// f(0xFFFFFFFF, i) on lanes with none left; all 32 lanes call it.
+template <class F>
+__device__ __forceinline__ void warp_lists_lanes(uint32_t o0, uint32_t c, F f)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t end = c;
+#pragma unroll
+    for (uint32_t d = 1; d < 32u; d <<= 1) {
+        const uint32_t x = __shfl_up_sync(0xFFFFFFFFu, end, d);
+        if (lane >= d) end += x;
+    }
+    const uint32_t total = __shfl_sync(0xFFFFFFFFu, end, 31);
+    const uint32_t base = o0 - (end - c);
+    for (uint32_t t0 = 0; t0 < total; t0 += 32u) {
+        const uint32_t t = t0 + lane;
+        uint32_t i = 0;
+#pragma unroll
+        for (uint32_t d = 16; d; d >>= 1)
+            if (__shfl_sync(0xFFFFFFFFu, end, i + d - 1u) <= t) i += d;
+        i = min(i, 31u);
+        const uint32_t b = __shfl_sync(0xFFFFFFFFu, base, i);
+        f(t < total ? b + t : 0xFFFFFFFFu, i);
+    }
+}
+
 // Calls f(o, i) for every occurrence o of up to eight lists, the quads of the
 // warp taking one each at a time: lanes i < 8 hold list i as [o0, o0 + c) (c = 0
-// on the others).  f(0xFFFFFFFF, 0) on quads with none left; all 32 lanes call
+// on the others).  f(0xFFFFFFFF, i) on quads with none left; all 32 lanes call
 // it.
 template <class F>
 __device__ __forceinline__ void warp_lists(uint32_t o0, uint32_t c, F f)

@@ -159,17 +159,17 @@ __device__ __forceinline__ void na_claim(uint32_t *asg, NaCtl *c, uint32_t l, ui
 }
 
 // Checks the bucket nogoods of the n literals at `from` (each holds since the
-// round before; no other nogood can have become unit or violated): warps w,
-// w + nw, ... take up to eight literals at a time (fewer when there are fewer
-// than eight a warp) and share out their lists (warp_lists, quad_check).  A literal's own fresh bit, of the other parity,
-// is cleared meanwhile.  SHARED: `from` is in shared memory.
+// round before; no other nogood can have become unit or violated).  With up to
+// eight literals a warp its quads share out their lists, for the shortest
+// chain; with more its lanes do, 32 literals at a time.  A literal's own fresh
+// bit, of the other parity, is cleared meanwhile.  SHARED: `from` is in shared
+// memory.
 template <bool SHARED>
 __device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c, const uint32_t *from, uint32_t n, uint32_t w,
                                           uint32_t nw, uint32_t fresh, uint32_t stale, const NaList &O)
 {
-    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t lane = threadIdx.x & 31u, each = min(32u, (n + nw - 1u) / nw);
     const Codes<false> codes{asg};
-    const uint32_t each = min(8u, (n + nw - 1u) / nw);
     for (uint32_t i0 = w * each; i0 < n; i0 += nw * each) {
         const uint32_t i = i0 + lane;
         uint32_t o0 = 0, count = 0;
@@ -179,14 +179,25 @@ __device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c,
             count = __ldg(D.occ_off + l + 1u) - o0;
             atomicAnd(asg + (y >> 3), ~(stale << ((y & 7u) * 4u)));
         }
-        warp_lists(o0, count, [&](uint32_t o, uint32_t) {
-            const QuadCheck r = quad_check(D, codes, fresh, o);
-            if ((lane & 3u) == 0u && !r.sat && r.n_un < 2u) {
-                if (r.n_un == 0u) na_conflict(c, O);
-                else na_claim(asg, c, r.ul, fresh, O);
-            }
-            __syncwarp();
-        });
+        if (each <= 8u) {
+            warp_lists(o0, count, [&](uint32_t o, uint32_t) {
+                const QuadCheck r = quad_check(D, codes, fresh, o);
+                if ((lane & 3u) == 0u && !r.sat && r.n_un < 2u) {
+                    if (r.n_un == 0u) na_conflict(c, O);
+                    else na_claim(asg, c, r.ul, fresh, O);
+                }
+                __syncwarp();
+            });
+        } else {
+            warp_lists_lanes(o0, count, [&](uint32_t o, uint32_t) {
+                if (o != 0xFFFFFFFFu) {
+                    const LaneCheck r = lane_check(D, codes, fresh, o);
+                    if (!r.sat && r.n_un == 0u) na_conflict(c, O);
+                    else if (!r.sat && r.n_un == 1u) na_claim(asg, c, r.ul, fresh, O);
+                }
+                __syncwarp();
+            });
+        }
     }
 }
 

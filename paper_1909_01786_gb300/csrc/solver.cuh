@@ -729,36 +729,19 @@ __device__ __forceinline__ void run_unit(const SweepCtx &X, uint32_t L, uint32_t
 // checked against the global codes, 128 at a time (four loads and their
 // gathers in flight before the first ballot).
 // Watched literals (Algorithm 2, which uses them for long learned nogoods
-// as well): *wslot holds two positions of the nogood.  If neither watched
+// as well): *wslot holds two positions of the nogood (wp).  If neither watched
 // literal holds -- one's complement is assigned, or both are unassigned --
-// the nogood is neither unit nor violated, and two checks settle it;
-// otherwise the scan runs and moves the watches to literals that do not
-// hold (the complement found, or the first unassigned ones).  Every such
-// nogood is checked every round by one warp, so the watches need no
-// per-variable lists and stay valid across backjumps.  Equal positions
-// (a nogood of one literal) always scan.
+// the nogood is neither unit nor violated, and two checks settle it (the
+// caller's); otherwise this scan runs and moves the watches to literals that do
+// not hold (the complement found, or the first unassigned ones).  Every such
+// nogood is checked every round, so the watches need no per-variable lists and
+// stay valid across backjumps.  Equal positions (a nogood of one literal)
+// always scan.
 __device__ __forceinline__ void classify_long(const SweepCtx &X, uint32_t id, unsigned long long &checks,
-                                              uint2 *wslot)
+                                              uint2 *wslot, uint2 wp)
 {
     const Dev &D = *X.D;
     const uint32_t lane = threadIdx.x & 31u;
-    uint2 wp = make_uint2(0u, 0u);
-    if (wslot) {
-        wp = __ldcg(wslot);
-        if (wp.x != wp.y) {
-            // lanes 0 and 1: the two watched literals
-            uint32_t val = 0u, l = 0u;
-            if (lane < 2u) {
-                l = lit_at(D, id + (lane ? wp.y : wp.x)) & ~END_BIT;
-                val = (l >> 1) < D.nv ? global_val(D, l >> 1, X.fresh) : 0u;
-            }
-            const bool opp = lane < 2u && val == ((l & 1u) ? V_T : V_F);
-            const bool un = lane < 2u && val == 0u;
-            const unsigned Bopp = __ballot_sync(FULL_MASK, opp), Bun = __ballot_sync(FULL_MASK, un);
-            checks += 2u;
-            if (Bopp || Bun == 3u) return;
-        }
-    }
     bool any_opp = false, done = false;
     uint32_t n_un = 0, ulit = 0, len = 0;
     uint32_t opos = 0, upos0 = 0, upos1 = 0;   // positions: a complement found, the first unassigned ones
@@ -904,19 +887,31 @@ __device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t i
 
 // The bucket nogoods of the literals on the trail entries [fr0, fr1) (the
 // claims of the round before), by the whole grid: only these can have become
-// unit or violated.  A warp takes up to eight entries (fewer when there are
-// fewer than eight a warp) and its quads share out their lists; values are the
-// global codes, with this round's claims unseen.  The fresh bits of the entries
-// are cleared meanwhile.  For more claims than one CTA follows well and fewer
-// than make a sweep of the store worth its bytes (Dev::list_max): on the 400k
-// program a sweep takes 56 us, a round over 20k claims about 8 us.
+// unit or violated.  With up to eight entries a warp its quads share out their
+// lists, for the shortest chain; with more its lanes do, 32 entries at a time.
+// Values are the global codes, with this round's claims unseen.  For more
+// claims than one CTA follows well and fewer than make a sweep of the store
+// worth its bytes (Dev::list_max): on the 400k program a sweep takes 56 us, a
+// round over 20k claims about 8 us.
 __device__ __forceinline__ void list_round(const SweepCtx &X, uint32_t fr0, uint32_t fr1, uint32_t &checks, uint32_t &visits)
 {
     const Dev &D = *X.D;
     const uint32_t lane = threadIdx.x & 31u, sub = lane & 3u, quad = lane & 28u, n = fr1 - fr0;
     const uint32_t wpc = blockDim.x >> 5, slot = (X.gw % wpc) * (X.nw / wpc) + X.gw / wpc;
-    const uint32_t each = min(8u, (n + X.nw - 1u) / X.nw), nw = X.cdl > 1u ? deps_words(D, X.cdl) : 0u;
+    const uint32_t each = min(32u, (n + X.nw - 1u) / X.nw), nw = X.cdl > 1u ? deps_words(D, X.cdl) : 0u;
     const Codes<false> codes{D.asg};
+    // claim of the unit literal, or conflict; whether this lane claimed
+    auto act = [&](uint32_t id, bool sat, uint32_t n_un, uint32_t ul) -> bool {
+        const uint32_t L = ((id >> 27) & 15u) + 1u;
+        checks += L;
+        visits++;
+        if (sat || n_un > 1u) return false;
+        const uint32_t x = ul >> 1, valbit = (ul & 1u) ? V_T : V_F;
+        const int k = n_un == 0u ? 2 : claim_var(D.asg, x, valbit, X.fresh);
+        if (k == 2) report_conflict(X, id, L);
+        else if (k == 0) record_claim(X, x, valbit, id);
+        return k == 0;
+    };
     for (uint32_t i0 = slot * each; i0 < n; i0 += X.nw * each) {
         const uint32_t i = i0 + lane;
         uint32_t y = 0, o0 = 0, c = 0;
@@ -928,21 +923,30 @@ __device__ __forceinline__ void list_round(const SweepCtx &X, uint32_t fr0, uint
                 c = __ldg(D.occ_off + l + 1u) - o0;
             }
         }
+        if (each > 8u) {
+            warp_lists_lanes(o0, c, [&](uint32_t o, uint32_t li) {
+                const uint32_t yo = __shfl_sync(FULL_MASK, y, li);
+                if (o != 0xFFFFFFFFu) {
+                    const LaneCheck r = lane_check(D, codes, X.fresh, o);
+                    if (act(r.id, r.sat, r.n_un, r.ul) && nw) {
+                        const uint32_t x = r.ul >> 1;
+                        uint32_t u[8];
+                        u[0] = yo;
+#pragma unroll
+                        for (uint32_t q = 0; q < 7u; q++) u[q + 1u] = r.l[q] == PAD_LIT ? x : r.l[q] >> 1;
+                        const uint4 v[2] = {make_uint4(u[0], u[1], u[2], u[3]), make_uint4(u[4], u[5], u[6], u[7])};
+                        narrow_deps(D, x, r.id, r.len ? nullptr : v, nw, 0u, 1u);
+                    }
+                }
+                __syncwarp();
+            });
+            continue;
+        }
         warp_lists(o0, c, [&](uint32_t o, uint32_t li) {
             const uint32_t yo = __shfl_sync(FULL_MASK, y, li);
             const QuadCheck r = quad_check(D, codes, X.fresh, o);
-            const uint32_t x = r.ul >> 1, valbit = (r.ul & 1u) ? V_T : V_F;
-            uint32_t won = 0;
-            if (sub == 0u && o != 0xFFFFFFFFu) {
-                const uint32_t L = ((r.id >> 27) & 15u) + 1u;
-                checks += L;
-                visits++;
-                if (!r.sat && r.n_un < 2u) {
-                    const int k = r.n_un == 0u ? 2 : claim_var(D.asg, x, valbit, X.fresh);
-                    if (k == 2) report_conflict(X, r.id, L);
-                    else if (k == 0) { record_claim(X, x, valbit, r.id); won = 1u; }
-                }
-            }
+            const uint32_t x = r.ul >> 1;
+            uint32_t won = sub == 0u && o != 0xFFFFFFFFu && act(r.id, r.sat, r.n_un, r.ul);
             if (!nw) return;
             won = __shfl_sync(FULL_MASK, won, quad);
             if (!__any_sync(FULL_MASK, won)) return;
@@ -1028,10 +1032,37 @@ __device__ __forceinline__ void sweep(const SweepCtx &X0, uint32_t n_learned, bo
     unsigned long long checks = 0;
     const uint32_t nl = D.n_long + n_learned;
     const uint32_t wpc = blockDim.x >> 5, slot = (X.gw % wpc) * (X.nw / wpc) + X.gw / wpc;
-    for (uint32_t i = slot; i < nl; i += X.nw) {
-        uint32_t id = i < D.n_long ? __ldg(D.long_ids + i) : __ldcg(D.learned_ids + (i - D.n_long));
-        classify_long(X, id, checks, D.nwatch ? D.nwatch + i : nullptr);
+    // a lane each for the two watched literals, which settle nearly all of
+    // them; the whole warp scans the rest (with a warp each, the three
+    // dependent loads of the watches were the cost of a round of a search with
+    // thousands of learned nogoods)
+    const uint32_t each = min(32u, (nl + X.nw - 1u) / X.nw);
+    uint32_t wchecks = 0;
+    for (uint32_t i0 = slot * each; i0 < nl; i0 += X.nw * each) {
+        const uint32_t i = i0 + lane;
+        uint32_t id = 0;
+        uint2 wp = make_uint2(0u, 0u);
+        bool scan = false;
+        if (lane < each && i < nl) {
+            id = i < D.n_long ? __ldg(D.long_ids + i) : __ldcg(D.learned_ids + (i - D.n_long));
+            if (D.nwatch) wp = __ldcg(D.nwatch + i);
+            scan = wp.x == wp.y;
+            if (!scan) {
+                const uint32_t l0 = lit_at(D, id + wp.x) & ~END_BIT, l1 = lit_at(D, id + wp.y) & ~END_BIT;
+                const uint32_t v0 = (l0 >> 1) < D.nv ? global_val(D, l0 >> 1, X.fresh) : 0u;
+                const uint32_t v1 = (l1 >> 1) < D.nv ? global_val(D, l1 >> 1, X.fresh) : 0u;
+                const bool opp = v0 == ((l0 & 1u) ? V_T : V_F) || v1 == ((l1 & 1u) ? V_T : V_F);
+                scan = !opp && (v0 != 0u || v1 != 0u);
+                wchecks += 2u;
+            }
+        }
+        for (unsigned m = __ballot_sync(FULL_MASK, scan); m; m &= m - 1u) {
+            const int src = __ffs(m) - 1;
+            classify_long(X, __shfl_sync(FULL_MASK, id, src), checks, D.nwatch ? D.nwatch + i0 + (uint32_t)src : nullptr,
+                          make_uint2(__shfl_sync(FULL_MASK, wp.x, src), __shfl_sync(FULL_MASK, wp.y, src)));
+        }
     }
+    if (nl) checks += __reduce_add_sync(FULL_MASK, wchecks);
     const unsigned long long t1 = wtimer ? globaltimer_ns() : 0ull;
     while (!ONLY_LONG) {
         uint32_t u = 0;
@@ -1819,65 +1850,95 @@ struct NarrowRound {
     uint32_t checks, visits;
 };
 
+// A claim made in a narrow round: its place in the queue (0xFFFFFFFF: none
+// made) and among the items, its occurrence list.
+struct NarrowClaim { uint32_t k, at, a0, a1; };
+
+// One lane's action on a checked nogood: claims its unit literal's complement,
+// or reports the conflict.  CACHED: the codes are the CTA's copy, and a claim
+// goes to global memory too, where nothing of the round waits for it.
+template <bool CACHED, class Queue>
+__device__ __forceinline__ NarrowClaim narrow_claim(const Dev &D, const Codes<CACHED> &codes, Acc *acc, Queue &Q, NarrowRound &R,
+                                                    uint32_t id, bool sat, uint32_t n_un, uint32_t ul)
+{
+    NarrowClaim C{0xFFFFFFFFu, 0u, 0u, 0u};
+    const uint32_t L = ((id >> 27) & 15u) + 1u;
+    R.checks += L;
+    R.visits++;
+    if (sat || n_un > 1u) return C;
+    bool clash = n_un == 0u;
+    if (!clash) {
+        const uint32_t x = ul >> 1, valbit = (ul & 1u) ? V_T : V_F;
+        // the claimed literal's list bounds load beside the claim
+        C.a0 = __ldg(D.occ_off + (ul ^ 1u));
+        C.a1 = __ldg(D.occ_off + (ul ^ 1u) + 1u);
+        const int c = claim_var(codes.w, x, valbit, R.fresh);
+        if (CACHED && c != 1) atomicOr(D.asg + (x >> 3), (valbit | R.fresh) << ((x & 7u) * 4u));
+        if (c == 0) {
+            C.k = atomicAdd(&Q.n[R.slot], 1u);
+            C.at = atomicAdd(&Q.m[R.slot], C.a1 - C.a0);
+            D.dl[x] = (int32_t)R.cdl;
+            D.reason[x] = id;
+            const uint32_t pos = R.out + C.k;
+            if (pos < D.nv) {
+                D.trail[pos] = x | (valbit == V_F ? TRAIL_F : 0u);
+                if (D.tpos) D.tpos[x] = pos;
+            }
+        }
+        clash = c == 2;
+    }
+    if (clash) {
+        const unsigned long long key = ((unsigned long long)L << 32) | id;
+        atomicMin(&acc->ckey, key);
+        atomicMin(&acc->cslot[id % 3u], key);
+        Q.conf[R.slot] = 1u;
+    }
+    return C;
+}
+
 // Checks occurrence o (0xFFFFFFFF: none) of a literal of variable y by a quad
-// of lanes; its first lane claims the unit literal's complement, or reports
-// the conflict, and all four write the claim's queue entry.  CACHED: the codes
-// are the CTA's copy, and a claim goes to global memory too, where nothing of
-// the round waits for it.  All 32 lanes call it.
+// of lanes; the first acts on it, and all four write a claim's queue entry.
+// All 32 lanes call it.
 template <bool CACHED, class Queue>
 __device__ __forceinline__ void narrow_check(const Dev &D, const Codes<CACHED> &codes, Acc *acc, Queue &Q, NarrowRound &R, uint32_t o,
                                              uint32_t y)
 {
     const uint32_t sub = threadIdx.x & 3u, quad = threadIdx.x & 28u;
     const QuadCheck r = quad_check(D, codes, R.fresh, o);
-    const uint32_t x = r.ul >> 1, valbit = (r.ul & 1u) ? V_T : V_F;
-    uint32_t k = 0xFFFFFFFFu, at = 0u, a0 = 0u, a1 = 0u;
-    if (sub == 0u && o != 0xFFFFFFFFu) {
-        const uint32_t L = ((r.id >> 27) & 15u) + 1u;
-        R.checks += L;
-        R.visits++;
-        if (!r.sat && r.n_un < 2u) {
-            bool clash = r.n_un == 0u;
-            if (!clash) {
-                // the claimed literal's list bounds load beside the claim
-                a0 = __ldg(D.occ_off + (r.ul ^ 1u));
-                a1 = __ldg(D.occ_off + (r.ul ^ 1u) + 1u);
-                const int c = claim_var(codes.w, x, valbit, R.fresh);
-                if (CACHED && c != 1) atomicOr(D.asg + (x >> 3), (valbit | R.fresh) << ((x & 7u) * 4u));
-                if (c == 0) {
-                    k = atomicAdd(&Q.n[R.slot], 1u);
-                    at = atomicAdd(&Q.m[R.slot], a1 - a0);
-                    D.dl[x] = (int32_t)R.cdl;
-                    D.reason[x] = r.id;
-                    const uint32_t pos = R.out + k;
-                    if (pos < D.nv) {
-                        D.trail[pos] = x | (valbit == V_F ? TRAIL_F : 0u);
-                        if (D.tpos) D.tpos[x] = pos;
-                    }
-                }
-                clash = c == 2;
-            }
-            if (clash) {
-                const unsigned long long key = ((unsigned long long)L << 32) | r.id;
-                atomicMin(&acc->ckey, key);
-                atomicMin(&acc->cslot[r.id % 3u], key);
-                Q.conf[R.slot] = 1u;
-            }
-        }
-    }
-    k = __shfl_sync(FULL_MASK, k, quad);
+    NarrowClaim C{0xFFFFFFFFu, 0u, 0u, 0u};
+    if (sub == 0u && o != 0xFFFFFFFFu) C = narrow_claim(D, codes, acc, Q, R, r.id, r.sat, r.n_un, r.ul);
+    const uint32_t k = __shfl_sync(FULL_MASK, C.k, quad);
     if (!__any_sync(FULL_MASK, k != 0xFFFFFFFFu)) return;
-    at = __shfl_sync(FULL_MASK, at, quad);
-    a0 = __shfl_sync(FULL_MASK, a0, quad);
-    a1 = __shfl_sync(FULL_MASK, a1, quad);
+    const uint32_t at = __shfl_sync(FULL_MASK, C.at, quad), a0 = __shfl_sync(FULL_MASK, C.a0, quad), a1 = __shfl_sync(FULL_MASK, C.a1, quad);
     if (k != 0xFFFFFFFFu) {
-        narrow_queue(Q, R.buf, R.slot, k, at, x | (valbit == V_F ? TRAIL_F : 0u), r.id, a0, a1, sub, 4u);
+        const uint32_t x = r.ul >> 1;
+        narrow_queue(Q, R.buf, R.slot, k, at, x | ((r.ul & 1u) ? 0u : TRAIL_F), r.id, a0, a1, sub, 4u);
         // the reason's variables for the bitmap, two per lane of the quad
         if (k < Queue::N && !r.len)
             reinterpret_cast<uint2 *>(&Q.u[R.buf][k][0])[sub] =
                 make_uint2(sub == 0u ? y : r.l[0] == PAD_LIT ? x : r.l[0] >> 1, r.l[1] == PAD_LIT ? x : r.l[1] >> 1);
     }
     __syncwarp();
+}
+
+// The same by one lane.
+template <bool CACHED, class Queue>
+__device__ __forceinline__ void narrow_check_lane(const Dev &D, const Codes<CACHED> &codes, Acc *acc, Queue &Q, NarrowRound &R,
+                                                  uint32_t o, uint32_t y)
+{
+    const LaneCheck r = lane_check(D, codes, R.fresh, o);
+    const NarrowClaim C = narrow_claim(D, codes, acc, Q, R, r.id, r.sat, r.n_un, r.ul);
+    if (C.k == 0xFFFFFFFFu) return;
+    const uint32_t x = r.ul >> 1;
+    narrow_queue(Q, R.buf, R.slot, C.k, C.at, x | ((r.ul & 1u) ? 0u : TRAIL_F), r.id, C.a0, C.a1, 0u, 1u);
+    if (C.k < Queue::N && !r.len) {
+        uint32_t u[8];
+        u[0] = y;
+#pragma unroll
+        for (uint32_t q = 0; q < 7u; q++) u[q + 1u] = r.l[q] == PAD_LIT ? x : r.l[q] >> 1;
+        Q.u[R.buf][C.k][0] = make_uint4(u[0], u[1], u[2], u[3]);
+        Q.u[R.buf][C.k][1] = make_uint4(u[4], u[5], u[6], u[7]);
+    }
 }
 
 // Bitmaps of entries [i0, i0 + step, ...) of the n in queue buf (trail from qs).
@@ -1959,11 +2020,12 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache,
                 const uint2 t = i < items ? Q.item[cur][i] : make_uint2(0xFFFFFFFFu, 0u);
                 narrow_check(D, codes, acc, Q, R, t.x, t.y);
             }
-            // lists past the items, and entries past the queue
-            for (uint32_t i0 = warp * 8u; rest && i0 < qn; i0 += wa * 8u) {
+            // lists past the items, and entries past the queue: many, so a lane
+            // each
+            for (uint32_t i0 = warp * 32u; rest && i0 < qn; i0 += wa * 32u) {
                 const uint32_t i = i0 + lane;
                 uint32_t y = 0, o = 0, o1 = 0;
-                if (lane < 8u && i < qn) {
+                if (i < qn) {
                     if (i < N) {
                         const uint4 c = Q.e[cur][i];
                         y = c.x & TRAIL_VAR; o = c.z; o1 = c.w;
@@ -1974,8 +2036,10 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache,
                         else { o = __ldg(D.occ_off + l); o1 = __ldg(D.occ_off + l + 1u); }
                     }
                 }
-                warp_lists(o, o1 - o, [&](uint32_t oc, uint32_t li) {
-                    narrow_check(D, codes, acc, Q, R, oc, __shfl_sync(FULL_MASK, y, li));
+                warp_lists_lanes(o, o1 - o, [&](uint32_t oc, uint32_t li) {
+                    const uint32_t yo = __shfl_sync(FULL_MASK, y, li);
+                    if (oc != 0xFFFFFFFFu) narrow_check_lane(D, codes, acc, Q, R, oc, yo);
+                    __syncwarp();
                 });
             }
         }
