@@ -170,7 +170,7 @@ def _traffic(kernel_src_sha, checks_per_launch, atoms, rules):
 
 def _src_sha():
     h = hashlib.sha256()
-    for f in ("solver.cuh", "kernels.cuh", "solve.cu", "sweep.cu", "device.cuh", "store.cpp", "store.h", "api.cpp"):
+    for f in ("solver.cuh", "follow.cuh", "kernels.cuh", "solve.cu", "sweep.cu", "device.cuh", "store.cpp", "store.h", "api.cpp"):
         h.update(open(os.path.join(ROOT, "paper_1909_01786_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 

@@ -96,19 +96,17 @@ extern "C" {
 #define ASP_LEARN_RES 1
 
 /* Propagation rounds (Section 4.1; Algorithm 2 checks only the nogoods of
- * the literals assigned last).  FULL: every round sweeps every nogood.
- * NOGOODS: a round checks the nogoods holding a variable assigned in the
- * previous round, one lane per nogood from per-variable occurrence lists.
- * UNITS: a round sweeps the units of the static partition (32-nogood groups
- * of one bucket, as full sweeps take them) that hold a variable assigned in
- * the previous round; a claim marks them in a dirty bitmap for the next
- * round (single-program solving; a batch sweeps everything). */
+ * the literals assigned last).  A round follows the claims of the round before
+ * through occurrence lists by literal: one CTA while they are few, the whole
+ * grid when they are more; where that would cost more than reading the store
+ * (the first round, after backjumps, very many claims) it sweeps every nogood.
+ * FULL: a sweep of every nogood also confirms each fixpoint.  NOGOODS, UNITS
+ * and UNITS_CHAINED: none does (the three are the same; they name schedules
+ * that differed by what a round checked).  Programs solved by one CTA, and
+ * batches, never sweep. */
 #define ASP_FRONTIER_FULL 0
 #define ASP_FRONTIER_NOGOODS 1
 #define ASP_FRONTIER_UNITS 2
-/* UNITS_CHAINED: as UNITS, and inside a round a claim also queues its CTA's
- * own units that hold the claimed variable, which later waves of the same
- * sweep check (up to three more waves; single-program solving). */
 #define ASP_FRONTIER_UNITS_CHAINED 3
 
 /* Backjump target of fwd-learning, with h the highest level in the
@@ -148,9 +146,8 @@ typedef struct {
     /* ASP_VIEW_*: the widest view allowed (a wider one than fits in shared
        memory falls back to the next narrower); 0 = ASP_VIEW_AUTO */
     int32_t view_mode;
-    /* ASP_FRONTIER_*: which static nogoods a propagation round checks
-       (Algorithm 2's frontier idea; the long and learned nogoods are checked
-       every round, and rounds after backjumps sweep everything) */
+    /* ASP_FRONTIER_*: whether sweeps of every nogood confirm the fixpoints
+       (the long and learned nogoods are checked before each in any case) */
     int32_t frontier;
     /* ASP_LEARN_*: conflict analysis */
     int32_t learning;
@@ -197,8 +194,8 @@ typedef struct {
                                                    counts every analysed one */
     int64_t nogood_visits;                      /* nogoods classified by the sweeps (the long
                                                    and learned ones every sweep, the bucket
-                                                   ones in full sweeps; frontier rounds'
-                                                   nogoods are not counted) */
+                                                   ones in full sweeps or as their
+                                                   occurrence lists are followed) */
     int64_t ns_slowest_long, ns_slowest_buckets; /* sums over sweeps of the slowest warp's time
                                                    (any CTA) on long and learned nogoods, and
                                                    on bucket units */
@@ -253,14 +250,14 @@ typedef struct asp_batch asp_batch;
  * propagation schedule, and captures the launch (queue reset + batch
  * kernel) in a CUDA graph.  Configurations: 0 = 256 threads per CTA, 3 CTAs
  * per SM; 1 = 128 threads, 6 per SM (twice the programs in flight, smaller
- * shared-memory views).  With an explicit configuration each program keeps
- * its own frontier option.  config = ASP_BATCH_AUTOTUNE tries every schedule
- * -- each configuration with full sweeps and, where the programs are small
- * enough to have the lists (about 20k atoms at 4 rules per atom), with the
- * frontier by units -- once on a sample of up to 256 programs spread over
- * the queue (each with at most 8 conflicts and 0.5 s of device time), and
- * keeps the one with the lowest device time per program (the trial solves
- * change nothing but the programs' last results).  models_cap may be NULL
+ * shared memory).  With an explicit configuration claims are followed through
+ * the occurrence lists.  config = ASP_BATCH_AUTOTUNE tries every schedule --
+ * each configuration with sweeps (and lists for few claims) and with lists
+ * only -- once on a sample of up to 256 programs spread over the queue (each
+ * with at most 8 conflicts and 0.5 s of device time), and keeps the one with
+ * the lowest device time per program (the trial solves change nothing but the
+ * programs' last results).  In batches of no more programs than SMs it runs
+ * configuration 0 with lists only as 768 threads per CTA.  models_cap may be NULL
  * (no models kept).  The programs must stay loaded until asp_batch_free.
  * Errors: ASP_E_ARG, ASP_E_OOM, ASP_E_CUDA. */
 int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each, const int64_t *models_cap,
@@ -272,11 +269,11 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
 int asp_batch_run(asp_batch *b, int32_t *statuses, int64_t *n_models, uint64_t *const *models);
 
 /* The configuration in use (0 or 1), its threads per CTA, the grid, the
- * propagation schedule (ASP_FRONTIER_UNITS for programs with unit lists, or
- * ASP_FRONTIER_FULL), and trial_ns (host double[4]): the autotuner's device
- * time per program of configurations 0 and 1 with full sweeps, then 0 and 1
- * with the unit frontier (ns; 0 if not tried, < 0 if it could not run); any
- * output may be NULL. */
+ * propagation schedule (ASP_FRONTIER_UNITS: occurrence lists only;
+ * ASP_FRONTIER_FULL: with sweeps), and trial_ns (host double[4]): the
+ * autotuner's device time per program of configurations 0 and 1 with sweeps,
+ * then 0 and 1 with lists only (ns; 0 if not tried, < 0 if it could not run);
+ * any output may be NULL. */
 int asp_batch_info(const asp_batch *b, int32_t *config, int32_t *block_threads, int32_t *grid,
                    int32_t *frontier, double *trial_ns);
 
@@ -450,8 +447,8 @@ int asp_mlp_score(const float *weights, const float *features, int64_t n, float 
  * asp_debug_propagate (unit propagation of a root-level partial assignment
  * to fixpoint over the program's nogoods) but keeps all of its working
  * memory in one static device array inside the library: at most 2^20
- * solver variables (512 KB of 4-bit codes plus 256 B of counters), held by
- * every GPU that loads the library until the process exits.  It calls no
+ * solver variables (512 KB of 4-bit codes, 4 MB of assigned literals and
+ * 256 B of counters), held by every GPU that loads the library until the process exits.  It calls no
  * cudaMalloc, cudaFree or other allocating routine.
  *   p          a program loaded earlier with asp_load_ground (read only)
  *   d_partial  device int8[n_vars]: 1 true, -1 false, 0 unassigned

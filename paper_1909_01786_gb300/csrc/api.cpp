@@ -658,6 +658,13 @@ int asp_load_ground(int32_t n_atoms, int32_t n_rules, const int32_t *head,
     if (rc == ASP_OK) rc = plan_batch(p, H, 0);
     if (rc == ASP_OK) rc = plan_batch(p, H, 1);
     if (rc == ASP_OK) {
+        // a cleared state, so that a sweep or the statistics before the first
+        // solve read no left-over memory (a sweep timed on left-over codes took
+        // 250 us instead of 30 on the 400k-atom program)
+        cudaError_t e = launch_reset(D, true, p->stream);
+        if (e != cudaSuccess) rc = cuda_fail(e, "clear state");
+    }
+    if (rc == ASP_OK) {
         cudaError_t e = p->stream ? cudaStreamSynchronize(p->stream) : cudaDeviceSynchronize();
         if (e != cudaSuccess) rc = cuda_fail(e, "load");
     }

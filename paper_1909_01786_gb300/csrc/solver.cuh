@@ -9,6 +9,12 @@
 // next phase into the other half of a double buffer, so all CTAs read a
 // stable copy while it is being updated.
 //
+// Propagation.  Claims are followed through occurrence lists by literal: one
+// CTA while they are few (narrow_rounds), the grid when they are more
+// (list_round).  Sweeps of the whole store run initial propagation, the round
+// after a backjump, rounds with very many claims, and the confirmation of a
+// full-sweep program's fixpoint.  One-CTA programs never sweep.
+//
 // Sweep design.  The static nogoods sit in one bucket per exact length
 // (Section 4: one kernel per length class), stored structure-of-arrays, and
 // are cut into contiguous ranges, one per CTA, along groups of nogoods (an
@@ -19,8 +25,9 @@
 // claimed variable's dependency bitmap at once, from its reason, and is then
 // published in the CTA's own view, so chains of implications inside a CTA
 // can resolve within one sweep; other CTAs see the claim after the next
-// barrier.  Long and learned nogoods are classified by one warp each (ballot
-// and popc over lanes), against the global codes.
+// barrier.  Long and learned nogoods are settled by a lane each through their
+// watched literals, or scanned by one warp (ballot and popc over lanes),
+// against the global codes.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -1975,8 +1982,9 @@ __device__ __forceinline__ void narrow_bitmaps(const Dev &D, const Queue &Q, uin
 // 0.6 us) and the instructions around it.  A claim puts its list's positions
 // into the next round's items, so a quad of lanes checks one nogood whatever
 // the lists' lengths (a program whose codes fit keeps a copy of them in shared
-// memory, which halves the chain); two thirds of the warps check while the others compute the bitmaps of the round's entries (nothing in the
-// round reads those), from the variables that the claim left in shared memory.
+// memory, which halves the chain); two thirds of the warps check while the
+// others compute the bitmaps of the round's entries (nothing in the round reads
+// those), from the variables that the claim left in shared memory.
 // The fresh bits alternate by round exactly as in sweeps: an entry's bit is
 // cleared while its round runs, when only the other parity's bit hides a
 // variable.  Returns the number of rounds; *n_claims is the number of claims,
