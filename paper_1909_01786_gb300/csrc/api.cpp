@@ -219,16 +219,23 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     const int max_grid = p->n_sms * per_sm;
     uint64_t total = 0;
     for (uint64_t x : H.group_lits) total += x;
-    // every SM for any real store; one CTA, which needs no grid barrier, for
-    // small programs
+    // every SM for any real store; one CTA, which needs no grid barrier and no
+    // sweep, for small programs.  Until the first conflict, one CTA against the
+    // grid: 300 atoms (24k literals) 245 and 294 us, 800 (63k) 439 and 460, 2000
+    // (158k) 1077 and 1106, 5000 (396k) 2973 and 2670; long searches also check
+    // their learned nogoods with that many fewer warps, hence the low line
     int64_t want = total <= 65536u ? 1 : (int64_t)(total / 2048) + 1;
     int g = (int)std::max<int64_t>(1, std::min<int64_t>(want, max_grid));
     if (p->opt.grid_ctas > 0) g = std::min(p->opt.grid_ctas, max_grid);
     p->grid = g;
     D.G = (uint32_t)g;
-    // claims of a round that one CTA follows in the time of a round of the
+    // Claims of a round that one CTA follows in the time of a round of the
     // grid (about 6 us), and that the grid follows in the time of a sweep (a
-    // claim checks about three nogoods of 32 bytes each, at random)
+    // claim checks about three nogoods of 32 bytes each, at random).  Until the
+    // first conflict / to the closure, with narrow_max 64, 256, 1024: 20k atoms
+    // 5.72, 5.19, 5.19 ms; 100k 48.5, 43.9, 44.1; closure of 50k atoms 1.30,
+    // 1.21, 1.49; of 400k 3.01, 2.98, 3.39.  With list_max the literals / 32,
+    // 128, 512: closure of 400k atoms 2.96, 2.98, 3.11.
     D.narrow_max = 256u;
     D.list_max = (uint32_t)(total / 128u);
     D.lists = g == 1;

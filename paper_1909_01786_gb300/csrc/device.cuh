@@ -123,7 +123,7 @@ struct DevStats {
 struct Barrier { unsigned long long count; unsigned int err, stall; };
 
 // An entry of the occurrence lists (see Dev::occ)
-struct __align__(32) Occurrence { uint32_t w[8]; };
+struct __align__(16) Occurrence { uint32_t w[8]; };
 
 struct Dev {
     uint32_t na, J, nv, asg_words;
