@@ -71,8 +71,8 @@ def _args():
     ap.add_argument("--batch-ms", type=int, default=2000,
                     help="device time budget per program of the batched leg (the oracle gets the same in CPU time)")
     ap.add_argument("--batch-frontier", type=int, default=2,
-                    help="propagation rounds of the one-at-a-time comparison and of an explicitly configured "
-                         "batch (0 full sweeps, 2 the unit frontier); the autotuned batch chooses its own")
+                    help="frontier option of the batched and one-at-a-time programs (0: sweeps confirm the "
+                         "fixpoints of one-at-a-time solves; 2: they do not)")
     ap.add_argument("--batch-rules-per-atom", type=int, default=2,
                     help="rules per atom of the batched workload (2: the family decides within the budget)")
     ap.add_argument("--sweep-only", type=int, default=0,
@@ -430,9 +430,10 @@ def _learning(a, aspgpu, prog):
 
 def _frontiers(a, aspgpu, prog):
     """The same search (same program, budget and heuristic) under each
-    propagation-round mode: full sweeps, the nogood frontier (occurrence
-    lists), and the unit frontier (dirty bucket units).  Device time, rates,
-    rounds per decision, and literals and nogoods checked per round."""
+    frontier option: with sweeps that confirm the fixpoints ("full") and
+    without (the other modes, which are the same), and on fewer CTAs.  Device
+    time, rates, rounds per decision, and literals and nogoods checked per
+    round."""
     out = {}
     for name, fr, grid in (("full", aspgpu.FRONTIER_FULL, 0), ("nogoods", aspgpu.FRONTIER_NOGOODS, 0),
                            ("units", aspgpu.FRONTIER_UNITS, 0), ("units_chained", aspgpu.FRONTIER_UNITS_CHAINED, 0),
