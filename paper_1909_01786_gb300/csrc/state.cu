@@ -200,30 +200,58 @@ __global__ void __launch_bounds__(256) occ_offsets_kernel(const uint32_t *count,
 // eight literals.
 struct RowBase { uint32_t at[BUCKET_MAX + 1]; };
 
+// The entry of literal word i, and its word of the rows.
+__device__ __forceinline__ void occ_fill(const Dev &D, uint32_t i, const RowBase &R, const uint32_t *off, uint32_t *count,
+                                         Occurrence *occ, uint32_t *rows)
+{
+    uint32_t L = 2;
+    for (uint32_t q = 3; q <= (uint32_t)BUCKET_MAX; q++)
+        if (i >= D.bk_base[q]) L = q;
+    const uint32_t n = D.bk_n[L], r = i - D.bk_base[L], q = r / n, k = r % n;
+    const uint32_t *base = D.lits + D.bk_base[L] + k;
+    const uint32_t l = __ldg(D.lits + i);
+    uint32_t w[8] = {bucket_nogood_id(L, k), PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT};
+    if (L <= 8u) {
+#pragma unroll
+        for (uint32_t j = 1; j < 8u; j++)
+            if (j < L) w[j] = __ldg(base + (size_t)(q + j < L ? q + j : q + j - L) * n);
+    } else {
+        w[1] = END_BIT | L;
+        w[2] = R.at[L] + k * L;
+        rows[w[2] + q] = l;
+    }
+    uint4 *e = reinterpret_cast<uint4 *>(occ + (__ldcg(off + l) + atomicSub(count + l, 1u) - 1u));
+    e[0] = make_uint4(w[0], w[1], w[2], w[3]);
+    e[1] = make_uint4(w[4], w[5], w[6], w[7]);
+}
+
 __global__ void __launch_bounds__(256) occ_fill_kernel(Dev D, uint32_t n_lits, RowBase R, const uint32_t *off, uint32_t *count,
                                                        Occurrence *occ, uint32_t *rows)
 {
-    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_lits; i += gridDim.x * blockDim.x) {
-        uint32_t L = 2;
-        for (uint32_t q = 3; q <= (uint32_t)BUCKET_MAX; q++)
-            if (i >= D.bk_base[q]) L = q;
-        const uint32_t n = D.bk_n[L], r = i - D.bk_base[L], q = r / n, k = r % n;
-        const uint32_t *base = D.lits + D.bk_base[L] + k;
-        const uint32_t l = __ldg(D.lits + i);
-        uint32_t w[8] = {bucket_nogood_id(L, k), PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT, PAD_LIT};
-        if (L <= 8u) {
-#pragma unroll
-            for (uint32_t j = 1; j < 8u; j++)
-                if (j < L) w[j] = __ldg(base + (size_t)(q + j < L ? q + j : q + j - L) * n);
-        } else {
-            w[1] = END_BIT | L;
-            w[2] = R.at[L] + k * L;
-            rows[w[2] + q] = l;
-        }
-        uint4 *e = reinterpret_cast<uint4 *>(occ + (off[l] + atomicSub(count + l, 1u) - 1u));
-        e[0] = make_uint4(w[0], w[1], w[2], w[3]);
-        e[1] = make_uint4(w[4], w[5], w[6], w[7]);
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n_lits; i += gridDim.x * blockDim.x) occ_fill(D, i, R, off, count, occ, rows);
+}
+
+// The whole construction by one block, for small programs: one launch instead
+// of six (loading a 20-atom program took 12 % longer with those).
+__global__ void __launch_bounds__(256) occ_small_kernel(Dev D, uint32_t n_lits, RowBase R, uint32_t *off, uint32_t *count,
+                                                        Occurrence *occ, uint32_t *rows)
+{
+    const uint32_t n = 2u * D.nv;
+    for (uint32_t i = threadIdx.x; i < n; i += 256u) count[i] = 0u;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < n_lits; i += 256u) atomicAdd(count + __ldg(D.lits + i), 1u);
+    __syncthreads();
+    uint32_t run = 0;
+    for (uint32_t i0 = 0; i0 < n; i0 += 256u) {
+        const uint32_t i = i0 + threadIdx.x, x = i < n ? __ldcg(count + i) : 0u;
+        uint32_t total;
+        const uint32_t at = run + block_scan(x, &total);
+        if (i < n) off[i] = at;
+        run += total;
     }
+    if (threadIdx.x == 0) off[n] = run;
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < n_lits; i += 256u) occ_fill(D, i, R, off, count, occ, rows);
 }
 
 // Where each program's models go in the packed words (-1: they do not fit,
@@ -294,6 +322,10 @@ cudaError_t launch_occurrences(const Dev &D, uint32_t n_lits, uint32_t *off, Occ
         w += L * D.bk_n[L];
     }
     const uint32_t n = 2u * D.nv, blocks = (n + OCC_BLOCK - 1u) / OCC_BLOCK;
+    if (n_lits <= 8192u) {
+        occ_small_kernel<<<1, 256, 0, st>>>(D, n_lits, R, off, count, occ, rows);
+        return cudaGetLastError();
+    }
     const int grid = (int)std::max<uint32_t>(1u, std::min<uint32_t>((n_lits + 255u) / 256u, 4864u));
     cudaError_t e = cudaMemsetAsync(count, 0, (size_t)n * 4, st);
     if (e != cudaSuccess) return e;
