@@ -1964,6 +1964,15 @@ __device__ __forceinline__ void narrow_bitmaps(const Dev &D, const Queue &Q, uin
     }
 }
 
+// Rounds of one narrow phase.  The search's time budget is looked at between
+// phases, and the grid's other CTAs wait for the end of this one at a barrier
+// that gives up (20 s): a chain a_i :- a_(i-1) claims one variable a round for
+// three rounds an atom, so a phase that ran to the fixpoint overran a budget of
+// 200 ms by 350 ms on a chain of 100k atoms, and from about 2M atoms on it
+// would have outlasted the barrier.  1024 rounds are about 2.5 ms; the phase
+// that follows costs a few us.
+constexpr uint32_t NARROW_ROUNDS = 1024u;
+
 // Propagation by one CTA, following the claims instead of sweeping the store
 // (Algorithm 2's Last/Next): the trail entries [first, tend) are the
 // assignments whose nogoods have not been checked yet (claims of the phase
@@ -1972,8 +1981,8 @@ __device__ __forceinline__ void narrow_bitmaps(const Dev &D, const Queue &Q, uin
 // list for the literal that now holds -- only those nogoods can have become
 // unit or violated -- and claims become the next round's entries, at
 // tbase, tbase + 1, ... of the trail.  Ends when a round claims nothing, on a
-// conflict, or when a round claims more than D.narrow_max (every CTA following
-// a part is then the faster way).
+// conflict, after NARROW_ROUNDS rounds, or when a round claims more than
+// D.narrow_max (every CTA following a part is then the faster way).
 //
 // Why: a search round assigns a few dozen variables (62 on average in the
 // 100k-atom program), and a sweep round costs its chain of barriers and loads
@@ -2065,7 +2074,7 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache,
             narrow_bitmaps(D, Q, cur, qs, qn, (split ? warp - wa : warp) * 4u + (lane >> 3), (split ? nwarp - wa : nwarp) * 4u, nw);
         cta_sync();
         const uint32_t n_new = Q.n[R.slot];
-        done = n_new == 0u || Q.conf[R.slot] || n_new > D.narrow_max || R.out + n_new > D.nv;
+        done = n_new == 0u || Q.conf[R.slot] || n_new > D.narrow_max || R.out + n_new > D.nv || it + 1u >= NARROW_ROUNDS;
         qs = R.out;
         qn = n_new;
         R.out += n_new;
@@ -2564,8 +2573,8 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             break;
         }
         if (nar && cta0) {
-            // few claims (or the decision): CTA 0 follows them to the end, the
-            // others wait at the barrier; their views catch up with the trail
+            // few claims (or the decision): CTA 0 follows them, the others wait
+            // at the barrier; their views catch up with the trail
             // at the next sweep.  A full-sweep program confirms the fixpoint
             // with a sweep; so does a program with long or learned nogoods,
             // which no list holds
