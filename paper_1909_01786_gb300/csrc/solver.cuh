@@ -1343,6 +1343,12 @@ __device__ __forceinline__ bool least_model_pass(const Dev &D, uint32_t gtid, ui
     return more;
 }
 
+// Passes that one CTA makes in a phase (a grid makes one): the time budget is
+// looked at between phases, and on a chain the least model takes a pass per
+// atom (100k atoms: 8.7 s, all past the budget when they were one phase).  64
+// passes of the 300k-rule program of that chain are about 6 ms.
+constexpr uint32_t STAB_PASSES = 64u;
+
 // The smallest true atom outside the least model, into acc->minU.
 __device__ __forceinline__ void unfounded_min(const Dev &D, Acc *acc, uint32_t gtid, uint32_t nthreads)
 {
@@ -2414,23 +2420,30 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             const uint32_t words = (D.na + 31u) >> 5;
             for (uint32_t w = gtid; w < words; w += nthreads) D.lm[w] = 0u;
             if (leader) { N.op = OP_STAB_ITER; N.stab_first = 1; N.tb = tend; }
+            if (!BATCH && gridDim.x > 1u) break;
+            // one CTA goes on in this phase
+        }
+        [[fallthrough]];
+        case OP_STAB_ITER: {
+            kind = 3;
             if (BATCH || gridDim.x == 1u) {
-                // one CTA: every pass in this phase
+                // one CTA: several passes in a phase
                 __shared__ uint32_t s_more;
-                do {
+                uint32_t more = 1u;
+                for (uint32_t i = 0; more && i < STAB_PASSES; i++) {
                     cta_sync();
                     if (threadIdx.x == 0) s_more = 0u;
                     cta_sync();
                     if (least_model_pass(D, gtid, nthreads)) s_more = 1u;
                     cta_sync();
-                } while (s_more);
-                unfounded_min(D, acc, gtid, nthreads);
-                if (leader) N.op = OP_STAB_RESULT;
+                    more = s_more;
+                }
+                if (!more) {
+                    unfounded_min(D, acc, gtid, nthreads);
+                    if (leader) N.op = OP_STAB_RESULT;
+                }
+                break;
             }
-            break;
-        }
-        case OP_STAB_ITER: {
-            kind = 3;
             if (!C.stab_first && A.flag == 0u) {
                 // least model reached: look for true atoms outside it
                 unfounded_min(D, acc, gtid, nthreads);

@@ -36,6 +36,17 @@ def test_time_budget_holds_on_a_chain(gpu, grid):
     assert 95e6 < s["ns_total"] < 150e6, s["ns_total"]
 
 
+def test_time_budget_holds_in_the_stability_step(gpu):
+    """One CTA: the assignment is total after about 600 ms, and the least model
+    of the chain then takes seconds, a pass per atom; the search stops within
+    a phase of passes of its budget."""
+    P = gpu.Program(_chain(100_000), grid_ctas=1, time_budget_ms=1_500)
+    status, _, n = P.solve(1, cap=1)
+    s = P.stats()
+    assert status == gpu.UNKNOWN and n == 0 and s["ns_stability"] > 0
+    assert 1495e6 < s["ns_total"] < 1600e6, s["ns_total"]
+
+
 @pytest.mark.parametrize("atom", [0, 1])
 def test_barrier_limit_does_not_bound_a_chain(gpu, atom):
     """A limit of 100 ms against a chain of about 500 ms.  Atom 0 true makes
