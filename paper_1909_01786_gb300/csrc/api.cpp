@@ -204,6 +204,10 @@ static int choose_view(asp_prog *p, const HostStore &H, Dev &D, const std::vecto
     return ASP_OK;
 }
 
+// One CTA: lists from here on are shared out to its warps (a program of 64k
+// literals has few)
+constexpr uint32_t ONE_CTA_LONG_LIST = 256u;
+
 // Grid size, the static partition of the buckets over the CTAs along groups
 // (an atom with its rules; a constraint), each CTA's slice of auxiliary
 // variables kept in shared memory, and the shared-memory layout.
@@ -240,6 +244,10 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     D.list_max = (uint32_t)(total / 128u);
     D.lists = g == 1;
     if (D.lists) D.narrow_max = 0xFFFFFFFFu;
+    // A warp walks 32 occurrences in about 2 us and a sweep reads a warp's share
+    // of the store, four literals in the time of one of them, after a few us of
+    // its own: up to this length the list is the faster one
+    D.long_list = g == 1 ? ONE_CTA_LONG_LIST : 128u + (uint32_t)(total / (4u * (uint64_t)g * ((uint32_t)p->block / 32u)));
     // groups [glo[i], glo[i+1]) for CTA i, balanced by literal count
     const uint32_t ng = (uint32_t)H.n_groups;
     std::vector<uint32_t> glo(g + 1, ng);
@@ -309,6 +317,7 @@ static int plan_batch(asp_prog *p, const HostStore &H, int config)
     D1.lists = D1.code_cache = 0u;
     D1.narrow_max = (uint32_t)std::min<uint64_t>(64u + p->D.static_checks / 1024u, 1u << 20);
     D1.list_max = D1.narrow_max;
+    D1.long_list = ONE_CTA_LONG_LIST;
     int rc = choose_view(p, H, D1, boff, alo, an, base, BATCH_SMEM_BUDGET[config]);
     if (rc != ASP_OK) return rc;
     D1.cta_boff = upload(p, boff, rc);

@@ -71,7 +71,8 @@ struct Ctl {              // double-buffered control block (phase parity)
     int32_t status, err;
     int32_t conflict;
     uint32_t full;              // the next round sweeps every nogood
-    uint32_t pad, tcom;                     // trail entries whose assignments are committed (tc: those in the views)
+    uint32_t wide;              // the next round's claims go to the grid however few they are
+    uint32_t tcom;              // trail entries whose assignments are committed (tc: those in the views)
 };
 
 struct Acc {              // per-phase accumulators, indexed by phase % 4
@@ -80,7 +81,7 @@ struct Acc {              // per-phase accumulators, indexed by phase % 4
                                  // conflicts per round)
     unsigned long long dkey;    // max over candidate rules of (score << 32 | ~j)
     uint32_t nclaim;            // variables claimed in the phase
-    uint32_t flag;              // something changed (least-model iteration)
+    uint32_t flag;              // something changed (least-model iteration); lists were passed over (list round)
     uint32_t minU;              // smallest unfounded true atom
     uint32_t nlits;             // literals appended to the loop nogood
     unsigned long long checks;  // literals classified outside full sweeps of the buckets
@@ -127,7 +128,8 @@ struct __align__(16) Occurrence { uint32_t w[8]; };
 
 struct Dev {
     uint32_t na, J, nv, asg_words;
-    uint32_t n_long, n_units, units_base, pad1;
+    uint32_t n_long, n_units, units_base;
+    uint32_t long_list;         // occurrences that one warp should not walk alone (see occ)
     // bucket L (2..15): literal q of nogood k at lits[bk_base[L] + q*bk_n[L] + k]
     uint32_t bk_base[16], bk_n[16];
     uint32_t lits_static, lits_cap, learned_ng_cap, pad0;
@@ -186,7 +188,9 @@ struct Dev {
     // literals, id, END_BIT | length and the place of its literals in rows.
     // A phase with at most narrow_max claims to follow is run by one CTA
     // through them (narrow_rounds), one with at most list_max by the grid
-    // (list_round), one with more is a sweep.
+    // (list_round), one with more is a sweep.  Lists of more than long_list
+    // occurrences in the hands of one warp: a grid sweeps the store instead, one
+    // CTA shares them out to its warps.
     // lists: one CTA solves the program, and its bucket nogoods are checked
     // through the lists only: no sweep, no view
     // code_cache: narrow rounds work on a copy of the codes in shared memory

@@ -892,6 +892,38 @@ __device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t i
     }
 }
 
+// One lane's action on a checked nogood of a list round: claim of its unit
+// literal, or conflict; whether it claimed.
+__device__ __forceinline__ bool list_act(const SweepCtx &X, uint32_t id, bool sat, uint32_t n_un, uint32_t ul, uint32_t &checks,
+                                         uint32_t &visits)
+{
+    const uint32_t L = ((id >> 27) & 15u) + 1u;
+    checks += L;
+    visits++;
+    if (sat || n_un > 1u) return false;
+    const uint32_t x = ul >> 1, valbit = (ul & 1u) ? V_T : V_F;
+    const int k = n_un == 0u ? 2 : claim_var(X.D->asg, x, valbit, X.fresh);
+    if (k == 2) report_conflict(X, id, L);
+    else if (k == 0) record_claim(X, x, valbit, id);
+    return k == 0;
+}
+
+// Occurrence o of a literal of variable y by one lane: check, claim and, above
+// the root level (nw > 0), the claim's bitmap.
+__device__ __forceinline__ void list_check_lane(const SweepCtx &X, uint32_t o, uint32_t y, uint32_t nw, uint32_t &checks, uint32_t &visits)
+{
+    const Codes<false> codes{X.D->asg};
+    const LaneCheck r = lane_check(*X.D, codes, X.fresh, o);
+    if (!list_act(X, r.id, r.sat, r.n_un, r.ul, checks, visits) || !nw) return;
+    const uint32_t x = r.ul >> 1;
+    uint32_t u[8];
+    u[0] = y;
+#pragma unroll
+    for (uint32_t q = 0; q < 7u; q++) u[q + 1u] = r.l[q] == PAD_LIT ? x : r.l[q] >> 1;
+    const uint4 v[2] = {make_uint4(u[0], u[1], u[2], u[3]), make_uint4(u[4], u[5], u[6], u[7])};
+    narrow_deps(*X.D, x, r.id, r.len ? nullptr : v, nw, 0u, 1u);
+}
+
 // The bucket nogoods of the literals on the trail entries [fr0, fr1) (the
 // claims of the round before), by the whole grid: only these can have become
 // unit or violated.  With up to eight entries a warp its quads share out their
@@ -899,7 +931,10 @@ __device__ __forceinline__ void narrow_deps(const Dev &D, uint32_t x, uint32_t i
 // Values are the global codes, with this round's claims unseen.  For more
 // claims than one CTA follows well and fewer than make a sweep of the store
 // worth its bytes (Dev::list_max): on the 400k program a sweep takes 56 us, a
-// round over 20k claims about 8 us.
+// round over 20k claims about 8 us.  A warp whose lists hold more than
+// Dev::long_list occurrences passes them over and sets the phase's flag: the
+// next round is then a sweep (an atom in half of the positive bodies of 320k
+// rules kept one warp busy for 9 ms).
 __device__ __forceinline__ void list_round(const SweepCtx &X, uint32_t fr0, uint32_t fr1, uint32_t &checks, uint32_t &visits)
 {
     const Dev &D = *X.D;
@@ -907,18 +942,6 @@ __device__ __forceinline__ void list_round(const SweepCtx &X, uint32_t fr0, uint
     const uint32_t wpc = blockDim.x >> 5, slot = (X.gw % wpc) * (X.nw / wpc) + X.gw / wpc;
     const uint32_t each = min(32u, (n + X.nw - 1u) / X.nw), nw = X.cdl > 1u ? deps_words(D, X.cdl) : 0u;
     const Codes<false> codes{D.asg};
-    // claim of the unit literal, or conflict; whether this lane claimed
-    auto act = [&](uint32_t id, bool sat, uint32_t n_un, uint32_t ul) -> bool {
-        const uint32_t L = ((id >> 27) & 15u) + 1u;
-        checks += L;
-        visits++;
-        if (sat || n_un > 1u) return false;
-        const uint32_t x = ul >> 1, valbit = (ul & 1u) ? V_T : V_F;
-        const int k = n_un == 0u ? 2 : claim_var(D.asg, x, valbit, X.fresh);
-        if (k == 2) report_conflict(X, id, L);
-        else if (k == 0) record_claim(X, x, valbit, id);
-        return k == 0;
-    };
     for (uint32_t i0 = slot * each; i0 < n; i0 += X.nw * each) {
         const uint32_t i = i0 + lane;
         uint32_t y = 0, o0 = 0, c = 0;
@@ -930,21 +953,14 @@ __device__ __forceinline__ void list_round(const SweepCtx &X, uint32_t fr0, uint
                 c = __ldg(D.occ_off + l + 1u) - o0;
             }
         }
+        if (__reduce_add_sync(FULL_MASK, c) > D.long_list) {
+            if (lane == 0) atomicOr(&X.acc->flag, 1u);
+            continue;
+        }
         if (each > 8u) {
             warp_lists_lanes(o0, c, [&](uint32_t o, uint32_t li) {
                 const uint32_t yo = __shfl_sync(FULL_MASK, y, li);
-                if (o != 0xFFFFFFFFu) {
-                    const LaneCheck r = lane_check(D, codes, X.fresh, o);
-                    if (act(r.id, r.sat, r.n_un, r.ul) && nw) {
-                        const uint32_t x = r.ul >> 1;
-                        uint32_t u[8];
-                        u[0] = yo;
-#pragma unroll
-                        for (uint32_t q = 0; q < 7u; q++) u[q + 1u] = r.l[q] == PAD_LIT ? x : r.l[q] >> 1;
-                        const uint4 v[2] = {make_uint4(u[0], u[1], u[2], u[3]), make_uint4(u[4], u[5], u[6], u[7])};
-                        narrow_deps(D, x, r.id, r.len ? nullptr : v, nw, 0u, 1u);
-                    }
-                }
+                if (o != 0xFFFFFFFFu) list_check_lane(X, o, yo, nw, checks, visits);
                 __syncwarp();
             });
             continue;
@@ -953,7 +969,7 @@ __device__ __forceinline__ void list_round(const SweepCtx &X, uint32_t fr0, uint
             const uint32_t yo = __shfl_sync(FULL_MASK, y, li);
             const QuadCheck r = quad_check(D, codes, X.fresh, o);
             const uint32_t x = r.ul >> 1;
-            uint32_t won = sub == 0u && o != 0xFFFFFFFFu && act(r.id, r.sat, r.n_un, r.ul);
+            uint32_t won = sub == 0u && o != 0xFFFFFFFFu && list_act(X, r.id, r.sat, r.n_un, r.ul, checks, visits);
             if (!nw) return;
             won = __shfl_sync(FULL_MASK, won, quad);
             if (!__any_sync(FULL_MASK, won)) return;
@@ -1825,6 +1841,15 @@ __device__ __forceinline__ bool group_sync(const Dev &D, uint32_t gen)
 
 // ------------------------------------------------------------ narrow rounds
 
+// Long lists of a round that its warps put off; with more of them (64k literals
+// hold at most 250) the others go to a warp each.
+constexpr uint32_t LONG_LISTS = 16u;
+
+// What a round leaves to the next one: claims, items drawn, whether some lists
+// are not among the items, whether there was a conflict, lists in lng (found;
+// LONG_LISTS of them are kept).  Read at once, after the round's barrier.
+struct __align__(16) NarrowCount { uint32_t n, m; uint16_t rest, conf; uint32_t nlong; };
+
 // Claims of the previous and of the current narrow round, cached in shared
 // memory (the trail holds all of them): e = trail entry, reason, and its
 // literal's occurrence list [z, w) unless the list is among the round's items;
@@ -1835,8 +1860,8 @@ struct NarrowQueue {
     static constexpr uint32_t N = ENTRIES, M = ITEMS;
     uint4 e[2][N], u[2][N][2];
     uint2 item[2][M];             // position in D.occ, variable it is the list of
-    // of round i, at (i + 1) % 3: claims, items, conflict, lists not among the items
-    uint32_t n[3], m[3], conf[3], rest[3];
+    uint4 lng[LONG_LISTS];        // lists of more than Dev::long_list outside the items: [x, y) of variable z
+    NarrowCount count[3];         // of round i, at (i + 1) % 3
 };
 
 // Entry k of a round's queue (k and at: its place among the items, drawn by
@@ -1853,7 +1878,7 @@ __device__ __forceinline__ void narrow_queue(Queue &Q, uint32_t buf, uint32_t sl
         for (uint32_t j = at + sub; j < Queue::M && j - at < c; j += lanes) Q.item[buf][j] = make_uint2(0xFFFFFFFFu, 0u);   // drawn, not used
     if (sub == 0u) {
         if (k < Queue::N) Q.e[buf][k] = make_uint4(entry, id, o0, fits ? o0 : o1);
-        if (!fits) Q.rest[slot] = 1u;
+        if (!fits) Q.count[slot].rest = 1u;
     }
 }
 
@@ -1888,8 +1913,8 @@ __device__ __forceinline__ NarrowClaim narrow_claim(const Dev &D, const Codes<CA
         const int c = claim_var(codes.w, x, valbit, R.fresh);
         if (CACHED && c != 1) atomicOr(D.asg + (x >> 3), (valbit | R.fresh) << ((x & 7u) * 4u));
         if (c == 0) {
-            C.k = atomicAdd(&Q.n[R.slot], 1u);
-            C.at = atomicAdd(&Q.m[R.slot], C.a1 - C.a0);
+            C.k = atomicAdd(&Q.count[R.slot].n, 1u);
+            C.at = atomicAdd(&Q.count[R.slot].m, C.a1 - C.a0);
             D.dl[x] = (int32_t)R.cdl;
             D.reason[x] = id;
             const uint32_t pos = R.out + C.k;
@@ -1904,7 +1929,7 @@ __device__ __forceinline__ NarrowClaim narrow_claim(const Dev &D, const Codes<CA
         const unsigned long long key = ((unsigned long long)L << 32) | id;
         atomicMin(&acc->ckey, key);
         atomicMin(&acc->cslot[id % 3u], key);
-        Q.conf[R.slot] = 1u;
+        Q.count[R.slot].conf = 1u;
     }
     return C;
 }
@@ -1979,6 +2004,11 @@ __device__ __forceinline__ void narrow_bitmaps(const Dev &D, const Queue &Q, uin
 // that follows costs a few us.
 constexpr uint32_t NARROW_ROUNDS = 1024u;
 
+// Occurrences of a round that one CTA of a grid follows (about 15 us), and why
+// it ends its phase: the next round has more of them, or (LEAVE_LONG + their
+// number) long lists were put off.
+constexpr uint32_t NARROW_OCC = 2048u, LEAVE_WIDE = 1u, LEAVE_LONG = 2u;
+
 // Propagation by one CTA, following the claims instead of sweeping the store
 // (Algorithm 2's Last/Next): the trail entries [first, tend) are the
 // assignments whose nogoods have not been checked yet (claims of the phase
@@ -1988,7 +2018,12 @@ constexpr uint32_t NARROW_ROUNDS = 1024u;
 // unit or violated -- and claims become the next round's entries, at
 // tbase, tbase + 1, ... of the trail.  Ends when a round claims nothing, on a
 // conflict, after NARROW_ROUNDS rounds, or when a round claims more than
-// D.narrow_max (every CTA following a part is then the faster way).
+// D.narrow_max (every CTA following a part is then the faster way).  A list of
+// more than D.long_list occurrences that is not among the items is not walked by
+// its warp: it ends the phase (*leave = LEAVE_LONG + such lists), after which all
+// of one CTA's warps walk it (long_lists) or a grid sweeps the store.  In a grid
+// a phase also ends, at once if need be, when a round's lists hold more than
+// NARROW_OCC (LEAVE_WIDE).
 //
 // Why: a search round assigns a few dozen variables (62 on average in the
 // 100k-atom program), and a sweep round costs its chain of barriers and loads
@@ -2006,7 +2041,8 @@ constexpr uint32_t NARROW_ROUNDS = 1024u;
 // *n_left that of the last ones, still to be checked.
 template <bool CACHED, class Queue>
 __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache, Queue &Q, Acc *acc, uint32_t cdl, uint32_t round,
-                                                  uint32_t first, uint32_t tend, uint32_t tbase, uint32_t *n_claims, uint32_t *n_left)
+                                                  uint32_t first, uint32_t tend, uint32_t tbase, uint32_t *n_claims, uint32_t *n_left,
+                                                  uint32_t *leave)
 {
     constexpr uint32_t N = Queue::N, M = Queue::M;
     const uint32_t tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5, nwarp = blockDim.x >> 5;
@@ -2016,27 +2052,29 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache,
     // when there is one warp, and all check at the root level
     const bool split = nw && nwarp > 1u;
     const uint32_t wa = split ? max(1u, nwarp * 2u / 3u) : nwarp;
-    if (tid < 3u) Q.n[tid] = Q.m[tid] = Q.conf[tid] = Q.rest[tid] = 0u;
+    if (tid < 3u) Q.count[tid] = NarrowCount{};
     if (CACHED)
         for (uint32_t w = tid; w < D.asg_words; w += blockDim.x) cache[w] = __ldcg(D.asg + w);
     cta_sync();
-    if (tid == 0 && tend - first > N) Q.rest[0] = 1u;
+    if (tid == 0 && tend - first > N) Q.count[0].rest = 1u;
     for (uint32_t i = tid; i < min(tend - first, N); i += blockDim.x) {
         const uint32_t e = __ldcg(D.trail + first + i), l = mk_lit(e & TRAIL_VAR, (e & TRAIL_F) != 0u);
         if ((l >> 1) >= D.nv) { atomicExch(&D.bar->err, 2u); Q.e[0][i] = make_uint4(0u, 0u, 0u, 0u); continue; }   // corrupt trail
         const uint32_t a0 = __ldg(D.occ_off + l), a1 = __ldg(D.occ_off + l + 1u);
-        narrow_queue(Q, 0u, 0u, i, atomicAdd(&Q.m[0], a1 - a0), e, 0u, a0, a1, 0u, 1u);
+        narrow_queue(Q, 0u, 0u, i, atomicAdd(&Q.count[0].m, a1 - a0), e, 0u, a0, a1, 0u, 1u);
     }
     cta_sync();
+    const uint32_t occ_max = D.G > 1u ? NARROW_OCC : 0xFFFFFFFFu;
     uint32_t qs = first, qn = tend - first, it = 0;
+    NarrowCount count = Q.count[0];
     NarrowRound R{cdl, 0u, 0u, 0u, tbase, 0u, 0u};
-    for (bool done = false; !done;) {
-        const uint32_t cur = it & 1u, stale = 4u << ((round + 1u) & 1u), items = min(Q.m[it % 3u], M), rest = Q.rest[it % 3u];
+    for (bool done = count.m > occ_max; !done;) {
+        const uint32_t cur = it & 1u, stale = 4u << ((round + 1u) & 1u), items = min(count.m, M), rest = count.rest;
         R.fresh = 4u << (round & 1u);
         R.buf = cur ^ 1u;
         R.slot = (it + 1u) % 3u;
         // cleared for the next round's claims; last read two barriers ago
-        if (tid == 0) Q.n[(it + 2u) % 3u] = Q.m[(it + 2u) % 3u] = Q.conf[(it + 2u) % 3u] = Q.rest[(it + 2u) % 3u] = 0u;
+        if (tid == 0) Q.count[(it + 2u) % 3u] = NarrowCount{};
         if (warp < wa) {
             for (uint32_t i0 = warp * 8u; i0 < items; i0 += wa * 8u) {
                 const uint32_t i = i0 + (lane >> 2);
@@ -2059,6 +2097,10 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache,
                         else { o = __ldg(D.occ_off + l); o1 = __ldg(D.occ_off + l + 1u); }
                     }
                 }
+                if (o1 - o > D.long_list) {
+                    const uint32_t k = atomicAdd(&Q.count[R.slot].nlong, 1u);
+                    if (k < LONG_LISTS) { Q.lng[k] = make_uint4(o, o1, y, 0u); o1 = o; }
+                }
                 warp_lists_lanes(o, o1 - o, [&](uint32_t oc, uint32_t li) {
                     const uint32_t yo = __shfl_sync(FULL_MASK, y, li);
                     if (oc != 0xFFFFFFFFu) narrow_check_lane(D, codes, acc, Q, R, oc, yo);
@@ -2079,16 +2121,18 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache,
         if (nw && it > 0u && (!split || warp >= wa))
             narrow_bitmaps(D, Q, cur, qs, qn, (split ? warp - wa : warp) * 4u + (lane >> 3), (split ? nwarp - wa : nwarp) * 4u, nw);
         cta_sync();
-        const uint32_t n_new = Q.n[R.slot];
-        done = n_new == 0u || Q.conf[R.slot] || n_new > D.narrow_max || R.out + n_new > D.nv || it + 1u >= NARROW_ROUNDS;
+        count = Q.count[R.slot];
+        const uint32_t n_new = count.n;
+        done = n_new - 1u >= D.narrow_max || (count.conf | count.nlong) || R.out + n_new > D.nv || count.m > occ_max || it + 1u >= NARROW_ROUNDS;
         qs = R.out;
         qn = n_new;
         R.out += n_new;
         round++;
         it++;
     }
+    *leave = count.nlong ? LEAVE_LONG + min(count.nlong, LONG_LISTS) : count.m > occ_max ? LEAVE_WIDE : 0u;
     // the last claims' bitmaps, by every warp
-    if (nw) narrow_bitmaps(D, Q, it & 1u, qs, qn, warp * 4u + (lane >> 3), nwarp * 4u, nw);
+    if (nw && it) narrow_bitmaps(D, Q, it & 1u, qs, qn, warp * 4u + (lane >> 3), nwarp * 4u, nw);
     cta_sync();
     const uint32_t c32 = __reduce_add_sync(FULL_MASK, R.checks), v32 = __reduce_add_sync(FULL_MASK, R.visits);
     if (lane == 0 && v32) {
@@ -2098,6 +2142,28 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache,
     *n_claims = R.out - tbase;
     *n_left = qn;
     return it;
+}
+
+// The lists that one CTA's narrow rounds put off, by all of its warps, as the
+// tail of the last round (X.fresh is that round's, so its claims stay unseen).
+// Apart from the rounds, whose every instruction counts: shared out there, the
+// lists cost 2 to 7 % of searches that have none.  A list of 1500 occurrences
+// kept its warp busy for 0.1 ms.
+__device__ __forceinline__ void long_lists(const SweepCtx &X, const uint4 *lists, uint32_t n)
+{
+    const uint32_t nw = X.cdl > 1u ? deps_words(*X.D, X.cdl) : 0u;
+    uint32_t checks = 0, visits = 0;
+    for (uint32_t i = 0; i < n; i++) {
+        const uint4 t = lists[i];
+        for (uint32_t o = t.x + threadIdx.x; o < t.y; o += blockDim.x) list_check_lane(X, o, t.z, nw, checks, visits);
+    }
+    __syncwarp();
+    checks = __reduce_add_sync(FULL_MASK, checks);
+    visits = __reduce_add_sync(FULL_MASK, visits);
+    if ((threadIdx.x & 31u) == 0u && visits) {
+        atomicAdd(&X.acc->checks, (unsigned long long)checks);
+        atomicAdd(&X.acc->visits, (unsigned long long)visits);
+    }
 }
 
 // Test-only failure injection: CTA D.stall_cta (thread 0) waits on a flag
@@ -2289,7 +2355,8 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             // without sweeps the caller's partial assignment is followed too
             const bool input = lists && D.mode == MODE_PROPAGATE && C.round == 1u;
             const bool quiet = A.nclaim == 0u && !input;   // no assignment is left to follow
-            if (quiet && C.clean) {
+            const bool owed = A.flag != 0u;                // lists passed over in the last round
+            if (quiet && C.clean && !owed) {
                 // fixpoint
                 if (D.mode == MODE_PROPAGATE) {
                     if (leader) { N.op = OP_DONE; N.status = 0; }
@@ -2305,13 +2372,13 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
                 if (leader) N.op = OP_APPLY;
                 break;
             }
-            if (!quiet && (lists || (!C.full && A.nclaim <= D.narrow_max))) {
+            if (!quiet && (lists || (!C.full && !C.wide && !owed && A.nclaim <= D.narrow_max))) {
                 nar = true; sw_cdl = C.cdl; sw_fr0 = input ? 0u : C.tb; sw_fr1 = sw_tbase = tend;
                 if (leader) atomicAdd(&D.stats->props, (unsigned long long)A.nclaim);
                 break;
             }
             // a full sweep, or the claims' lists, by the whole grid
-            sw_full = !lists && (C.full != 0u || (D.frontier == 0u && quiet) || (!quiet && A.nclaim > D.list_max));
+            sw_full = !lists && (C.full != 0u || owed || (D.frontier == 0u && quiet) || (!quiet && A.nclaim > D.list_max));
             // make last round's claims visible: clear their fresh bit
             // (grid-wide) and put them in this CTA's view, which only sweeps
             // read
@@ -2334,7 +2401,7 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             sw = true; sw_cdl = C.cdl; sw_tbase = tend;
             if (!sw_full && !quiet) { sw_fr0 = C.tb; sw_fr1 = tend; }
             if (leader) {
-                N.op = OP_ROUND; N.round = C.round + 1u; N.tc = sw_full ? tend : C.tc; N.tb = tend; N.tcom = tend; N.full = 0;
+                N.op = OP_ROUND; N.round = C.round + 1u; N.tc = sw_full ? tend : C.tc; N.tb = tend; N.tcom = tend; N.full = 0; N.wide = 0;
                 N.clean = lists || D.frontier != 0u || sw_full;
                 atomicAdd(&D.stats->rounds, 1ull);
                 atomicAdd(&D.stats->props, (unsigned long long)A.nclaim);
@@ -2595,16 +2662,24 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             constexpr uint32_t QN = !BATCH ? 192u : LISTS ? 96u : 24u;
             __shared__ NarrowQueue<QN, 4u * QN> Q;
             cta_sync();
-            uint32_t n = 0, left = 0;
+            uint32_t n = 0, left = 0, leave = 0;
             const uint32_t its = D.code_cache
-                ? narrow_rounds<true>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left)
-                : narrow_rounds<false>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left);
+                ? narrow_rounds<true>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left, &leave)
+                : narrow_rounds<false>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left, &leave);
+            if (leave > LEAVE_LONG && D.G == 1u) {
+                SweepCtx X{&D, V, 4u << ((C.round + its - 1u) & 1u), sw_cdl, sw_tbase + n, acc, true, false, cta, rank >> 5, size >> 5};
+                long_lists(X, Q.lng, leave - LEAVE_LONG);
+                cta_sync();
+                leave = 0u;
+            }
             if (leader) {
-                // the trail's last `left` claims are still to be followed
-                N.op = OP_ROUND; N.round = C.round + its; N.tb = N.tcom = sw_tbase + n - left; N.full = 0;
-                N.clean = (lists || D.frontier != 0u) && D.n_long + C.n_learned == 0u;
-                acc->nclaim = left;
-                atomicAdd(&D.stats->props, (unsigned long long)(n - left));
+                // the trail's last `left` claims, and those of the long lists
+                // after them, are still to be followed
+                N.op = OP_ROUND; N.round = C.round + its; N.tb = N.tcom = sw_tbase + n - left;
+                N.full = leave > LEAVE_LONG; N.wide = leave == LEAVE_WIDE;
+                N.clean = (lists || D.frontier != 0u) && D.n_long + C.n_learned == 0u && leave <= LEAVE_LONG;
+                atomicAdd(&acc->nclaim, left);
+                atomicAdd(&D.stats->props, (unsigned long long)((long long)n - (long long)left));
                 atomicAdd(&D.stats->rounds, (unsigned long long)its);
             }
         }
