@@ -42,12 +42,15 @@ namespace {
 struct NaCtl {                 // first words of the scratch array
     unsigned int count, err, conflict;
     // of the grid's rounds, by their number modulo 3 (a round clears the next
-    // one's, whose last readers are two barriers back): literals listed, conflict
-    unsigned int nclaim[3], conf[3];
+    // one's, whose last readers are two barriers back): literals listed, why to
+    // stop following them (NA_CONFLICT, NA_LONG)
+    unsigned int nclaim[3], stop[3];
     // CTA 0's narrow rounds: number of the next round, literals it left to
-    // follow, conflict; and the counter of literals past its shared lists
-    unsigned int next, left, nconf, nover;
+    // follow, why it stopped; and the counter of literals past its shared lists
+    unsigned int next, left, nstop, nover;
 };
+// a nogood is violated; lists too long for a warp were passed over
+constexpr unsigned int NA_CONFLICT = 1u, NA_LONG = 2u;
 
 constexpr uint32_t NA_THREADS = 768, NA_LIST = 1024;
 // claims that CTA 0 follows alone: a round of the grid costs its barrier and
@@ -118,7 +121,7 @@ struct NaList {
     unsigned int *n;           // counter of the round
     uint32_t *s_lit;           // [NA_LIST]
     unsigned int *s_n;
-    unsigned int *conf;        // the round's conflict flag
+    unsigned int *stop;        // the round's reasons to stop
 };
 
 __device__ __forceinline__ void na_push(const NaList &O, uint32_t l)
@@ -146,7 +149,7 @@ __device__ __forceinline__ void na_flush(const NaList &O)
 __device__ __forceinline__ void na_conflict(NaCtl *c, const NaList &O)
 {
     atomicExch(&c->conflict, 1u);
-    atomicExch(O.conf, 1u);
+    atomicOr(O.stop, NA_CONFLICT);
 }
 
 // claim the complement of literal l; conflict flag on a clash
@@ -163,10 +166,12 @@ __device__ __forceinline__ void na_claim(uint32_t *asg, NaCtl *c, uint32_t l, ui
 // eight literals a warp its quads share out their lists, for the shortest
 // chain; with more its lanes do, 32 literals at a time.  A literal's own fresh
 // bit, of the other parity, is cleared meanwhile.  SHARED: `from` is in shared
-// memory.
+// memory.  A warp whose lists hold more than `longest` occurrences passes them
+// over and stops the rounds for a sweep of the store (a literal of 160k nogoods
+// kept one warp busy for 10 ms).
 template <bool SHARED>
 __device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c, const uint32_t *from, uint32_t n, uint32_t w,
-                                          uint32_t nw, uint32_t fresh, uint32_t stale, const NaList &O)
+                                          uint32_t nw, uint32_t fresh, uint32_t stale, uint32_t longest, const NaList &O)
 {
     const uint32_t lane = threadIdx.x & 31u, each = min(32u, (n + nw - 1u) / nw);
     const Codes<false> codes{asg};
@@ -178,6 +183,10 @@ __device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c,
             o0 = __ldg(D.occ_off + l);
             count = __ldg(D.occ_off + l + 1u) - o0;
             atomicAnd(asg + (y >> 3), ~(stale << ((y & 7u) * 4u)));
+        }
+        if (__reduce_add_sync(0xFFFFFFFFu, count) > longest) {
+            if (lane == 0) atomicOr(O.stop, NA_LONG);
+            continue;
         }
         if (each <= 8u) {
             warp_lists(o0, count, [&](uint32_t o, uint32_t) {
@@ -201,18 +210,52 @@ __device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c,
     }
 }
 
+// Checks every bucket nogood of the store, a lane each, and clears the fresh
+// bits of the n literals at `from`.
+__device__ __forceinline__ void na_sweep(const Dev &D, uint32_t *asg, NaCtl *c, const uint32_t *from, uint32_t n, uint32_t gt,
+                                         uint32_t nth, uint32_t fresh, uint32_t stale, const NaList &O)
+{
+    for (uint32_t i = gt; i < n; i += nth) {
+        const uint32_t y = __ldcg(from + i) >> 1;
+        atomicAnd(asg + (y >> 3), ~(stale << ((y & 7u) * 4u)));
+    }
+    for (uint32_t L = 2; L <= (uint32_t)BUCKET_MAX; L++) {
+        const uint32_t *base = D.lits + D.bk_base[L];
+        const uint32_t m = D.bk_n[L];
+        for (uint32_t k = gt; k < m; k += nth) {
+            bool sat = false;
+            uint32_t n_un = 0, ul = 0;
+            for (uint32_t q0 = 0; q0 < L && !sat && n_un < 2u; q0 += 4u) {
+                uint32_t l[4], v[4];
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; q++) l[q] = q0 + q < L ? __ldg(base + (size_t)(q0 + q) * m + k) : PAD_LIT;
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; q++) v[q] = l[q] != PAD_LIT ? na_val(asg, l[q] >> 1, fresh) : 3u;
+#pragma unroll
+                for (uint32_t q = 0; q < 4u; q++) {
+                    if (v[q] == 0u) { n_un++; ul = l[q]; }
+                    sat |= v[q] == ((l[q] & 1u) ? V_T : V_F);
+                }
+            }
+            if (!sat && n_un == 0u) na_conflict(c, O);
+            else if (!sat && n_un == 1u) na_claim(asg, c, ul, fresh, O);
+        }
+    }
+}
+
 // The fixpoint by following assignments: a round checks the nogoods of the
 // literals listed by the round before (first the caller's assignment), found
 // through the occurrence lists, instead of every nogood of the store; with at
 // most NA_NARROW of them CTA 0 goes on alone, with CTA barriers.  Nogoods in
 // no list (more than BUCKET_MAX literals) are checked in the grid's rounds,
-// and the last round is one.  A round is bound by its chain of dependent loads
-// (list, list bounds, nogood id, literals, codes, claim) and its barrier.
+// and the last round is one.  After lists too long for a warp the grid's next
+// round is a sweep of the store.  A round is bound by its chain of dependent
+// loads (list, list bounds, occurrence, codes, claim) and its barrier.
 __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D, const int8_t *partial, int8_t *closure,
                                                                           int32_t *conflict_out, uint32_t *scratch)
 {
     __shared__ uint32_t s_lit[2][NA_LIST];
-    __shared__ unsigned int s_n[3], s_conf;
+    __shared__ unsigned int s_n[3], s_stop;
     NaCtl *c = reinterpret_cast<NaCtl *>(scratch);
     uint32_t *asg = scratch + NOALLOC_CTL_WORDS, *list = asg + NOALLOC_CODES;
     const uint32_t nth = gridDim.x * blockDim.x, gt = blockIdx.x * blockDim.x + threadIdx.x;
@@ -221,9 +264,9 @@ __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D,
     // spread over the SMs
     const uint32_t gw = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     const uint32_t words = (D.nv + 7u) >> 3;
-    if (threadIdx.x == 0) s_n[0] = s_n[1] = s_n[2] = s_conf = 0u;
+    if (threadIdx.x == 0) s_n[0] = s_n[1] = s_n[2] = s_stop = 0u;
     na_cta_sync();
-    NaList O{list, 0u, &c->nclaim[2], s_lit[0], &s_n[0], &c->conf[2]};
+    NaList O{list, 0u, &c->nclaim[2], s_lit[0], &s_n[0], &c->stop[2]};
     // the caller's partial assignment, committed (no fresh bits); round -1
     const bool aligned = ((reinterpret_cast<uintptr_t>(partial) | reinterpret_cast<uintptr_t>(closure)) & 7u) == 0u;
     for (uint32_t w = gt; w < words; w += nth) {
@@ -246,12 +289,17 @@ __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D,
     uint32_t gen = 0, from = 0, to = 0;       // literals [from, to) are to be followed
     bool ok = na_sync(c, gen++);
     if (ok) to = __ldcg(&c->nclaim[2]);
+    // what a warp walks in the time of a sweep: a sweep reads a warp's share of
+    // the store four literals in the time of one occurrence, after a barrier
+    const uint32_t longest = 128u + (uint32_t)(D.static_checks / (4u * nw));
     // r: rounds so far (its parity names the fresh bit), k: the grid's rounds;
     // the first also applies the unit nogoods
-    for (uint32_t r = 0, k = 0; ok; k++) {
+    uint32_t r = 0, k = 0, stop = 0;
+follow:
+    for (; ok; k++) {
         const uint32_t fresh = 4u << (r & 1u), stale = 4u << ((r + 1u) & 1u), slot = k % 3u;
-        if (gt == 0) c->nclaim[(k + 1u) % 3u] = c->conf[(k + 1u) % 3u] = 0u;
-        O = NaList{list, to, &c->nclaim[slot], s_lit[0], &s_n[0], &c->conf[slot]};
+        if (gt == 0) c->nclaim[(k + 1u) % 3u] = c->stop[(k + 1u) % 3u] = 0u;
+        O = NaList{list, to, &c->nclaim[slot], s_lit[0], &s_n[0], &c->stop[slot]};
         if (k == 0)
             for (uint32_t i = gt; i < D.n_units; i += nth) {
                 const uint32_t l = __ldg(D.lits + D.units_base + i) & ~END_BIT;
@@ -259,7 +307,7 @@ __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D,
                 if (v == 0u) na_claim(asg, c, l, fresh, O);
                 else if (v == ((l & 1u) ? V_F : V_T)) na_conflict(c, O);
             }
-        na_follow<false>(D, asg, c, list + from, to - from, gw, nw, fresh, stale, O);
+        na_follow<false>(D, asg, c, list + from, to - from, gw, nw, fresh, stale, longest, O);
         // long nogoods: one warp per nogood, lanes over literals
         for (uint32_t i = gw; i < D.n_long; i += nw) {
             __syncwarp();
@@ -290,46 +338,69 @@ __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D,
         if (!(ok = na_sync(c, gen++))) break;
         // every thread sees the same counters after the barrier
         const uint32_t n = __ldcg(&c->nclaim[slot]);
-        if (__ldcg(&c->conf[slot]) || n == 0u) break;
+        stop = __ldcg(&c->stop[slot]);
         from = to;
         to += n;
         r++;
+        if (stop || n == 0u) break;
         if (n > NA_NARROW) continue;
         if (blockIdx.x == 0) {
             // narrow rounds: a round's literals stay in shared memory, two
-            // lists in turn; if the last one lists too many they go to the
-            // list after `to`, for the grid
+            // lists in turn; if the last one lists too many, or lists were
+            // passed over, they go to the list after `to`, for the grid
             for (uint32_t i = threadIdx.x; i < n; i += blockDim.x) s_lit[0][i] = __ldcg(list + from + i);
             if (threadIdx.x == 0) c->nover = 0u;
             uint32_t m = n, i = 0;
             O.base = to;
             O.n = &c->nover;
-            O.conf = &s_conf;
+            O.stop = &s_stop;
             do {
                 na_cta_sync();
                 if (threadIdx.x == 0) s_n[(i + 2u) % 3u] = 0u;     // the next round's counter
                 O.s_lit = s_lit[(i + 1u) & 1u];
                 O.s_n = &s_n[(i + 1u) % 3u];
                 na_follow<true>(D, asg, c, s_lit[i & 1u], m, threadIdx.x >> 5, blockDim.x >> 5, 4u << ((r + i) & 1u),
-                                4u << ((r + i + 1u) & 1u), O);
+                                4u << ((r + i + 1u) & 1u), longest, O);
                 na_cta_sync();
                 m = *O.s_n;
                 i++;
-            } while (m != 0u && m <= NA_NARROW && !s_conf);
-            if (m > NA_NARROW) na_flush(O);
+            } while (m != 0u && m <= NA_NARROW && !s_stop);
+            const bool over = m > NA_NARROW || (m != 0u && s_stop);
+            if (over) na_flush(O);
             na_cta_sync();
             if (threadIdx.x == 0) {
-                s_n[0] = s_n[1] = s_n[2] = 0u;
                 c->next = r + i;
-                c->left = m > NA_NARROW ? m : 0u;
-                c->nconf = s_conf;
+                c->left = over ? m : 0u;
+                c->nstop = s_stop;
+                s_n[0] = s_n[1] = s_n[2] = s_stop = 0u;
             }
         }
         if (!(ok = na_sync(c, gen++))) break;
         r = __ldcg(&c->next);
         from = to;
         to += __ldcg(&c->left);
-        if (__ldcg(&c->nconf) || (from == to && D.n_long == 0u)) break;
+        stop = __ldcg(&c->nstop);
+        if (stop || (from == to && D.n_long == 0u)) break;
+    }
+    if (ok && stop == NA_LONG) {
+        // a round of the whole store.  Apart from the others: as a case among
+        // them, with a test in each, it took 6 % of an 80k-atom program's
+        // propagation, which has no such list
+        k++;
+        const uint32_t slot = k % 3u;
+        if (gt == 0) c->nclaim[(k + 1u) % 3u] = c->stop[(k + 1u) % 3u] = 0u;
+        O = NaList{list, to, &c->nclaim[slot], s_lit[0], &s_n[0], &c->stop[slot]};
+        na_sweep(D, asg, c, list + from, to - from, gt, nth, 4u << (r & 1u), 4u << ((r + 1u) & 1u), O);
+        na_flush(O);
+        if ((ok = na_sync(c, gen++))) {
+            const uint32_t n = __ldcg(&c->nclaim[slot]);
+            stop = __ldcg(&c->stop[slot]);
+            from = to;
+            to += n;
+            r++;
+            k++;
+            if (!stop) goto follow;
+        }
     }
     if (!ok && !gt) *conflict_out = -1;
     if (!ok) return;

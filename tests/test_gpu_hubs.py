@@ -96,3 +96,22 @@ def test_a_hub_costs_a_sweep_not_a_walk(env):
         assert not P.propagate(partial)[0]
         times.append(P.stats()["ns_total"])
     assert min(times) < 1.5e6, times
+
+
+def test_a_hub_costs_a_sweep_without_allocation(env):
+    """The same through asp_propagate_noalloc."""
+    torch, gpu = env
+    P = gpu.Program(_hubs(1, 80_000, 40_000, 160_000, 1))
+    d = torch.zeros(P.n_vars, dtype=torch.int8, device="cuda")
+    d[0] = 1
+    out, conflict = torch.empty_like(d), torch.zeros(1, dtype=torch.int32, device="cuda")
+    times = []
+    for _ in range(4):
+        start, end = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        start.record()
+        assert P.propagate_noalloc(d.data_ptr(), out.data_ptr(), conflict.data_ptr()) == 0
+        end.record()
+        torch.cuda.synchronize()
+        assert conflict.item() == 0
+        times.append(start.elapsed_time(end))
+    assert min(times) < 2.0, times
