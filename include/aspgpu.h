@@ -103,7 +103,8 @@ extern "C" {
  * FULL: a sweep of every nogood also confirms each fixpoint.  NOGOODS, UNITS
  * and UNITS_CHAINED: none does (the three are the same; they name schedules
  * that differed by what a round checked).  Programs solved by one CTA, and
- * batches, never sweep. */
+ * batches solved with lists only, never sweep; programs whose lists did not fit
+ * in memory always do. */
 #define ASP_FRONTIER_FULL 0
 #define ASP_FRONTIER_NOGOODS 1
 #define ASP_FRONTIER_UNITS 2
@@ -176,7 +177,8 @@ typedef struct {
     int64_t n_vars, n_atoms, n_rules_with_head;
     int64_t n_nogoods, n_literals;       /* static completion + constraint nogoods */
     int64_t n_unit_nogoods, n_long_nogoods;
-    int64_t store_bytes;                 /* device bytes of the static nogood store */
+    int64_t store_bytes;                 /* device bytes of the static nogood store (without
+                                            its occurrence lists) */
     int64_t rounds;                      /* propagate-and-check sweeps (Section 4.1) */
     int64_t literal_checks;              /* literals read and classified by the sweeps */
     int64_t propagations, conflicts, decisions, completions;
@@ -205,8 +207,10 @@ typedef struct {
 void asp_default_options(asp_options *opt);
 
 /* Build the completion nogoods of a ground normal program (Section 2) and
- * upload them.  Input arrays belong to the caller and are only read during
- * the call.  opt may be NULL.  On success *out owns device memory until
+ * upload them, with occurrence lists for propagation (32 bytes per literal of
+ * the static nogoods of 2 to 15 literals; a program whose lists cannot be
+ * allocated is propagated by sweeps of the store, more slowly).  Input arrays
+ * belong to the caller and are only read during the call.  opt may be NULL.  On success *out owns device memory until
  * asp_free.  Errors: ASP_E_ARG, ASP_E_RANGE, ASP_E_OOM, ASP_E_CUDA,
  * ASP_E_NODEVICE. */
 int asp_load_ground(int32_t n_atoms, int32_t n_rules, const int32_t *head,

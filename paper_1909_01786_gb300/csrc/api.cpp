@@ -105,6 +105,15 @@ static void *dalloc(asp_prog *p, size_t bytes)
     return ptr;
 }
 
+// Gives the last allocation back, if ptr is it.
+static void dfree_last(asp_prog *p, void *ptr)
+{
+    if (!ptr || p->bufs.empty() || p->bufs.back().p != ptr) return;
+    if (p->opt.dev_free) p->opt.dev_free(ptr, p->bufs.back().bytes, p->opt.alloc_ctx);
+    else cudaFree(ptr);
+    p->bufs.pop_back();
+}
+
 static void release_all(asp_prog *p)
 {
     if (p->stream) cudaStreamSynchronize(p->stream);
@@ -657,22 +666,31 @@ int asp_load_ground(int32_t n_atoms, int32_t n_rules, const int32_t *head,
             if (e != cudaSuccess) rc = cuda_fail(e, "clear stamps");
         }
     }
-    if (rc == ASP_OK && D.nv > 0) {
-        // occurrence lists by literal, built on the device; the bitmaps and
-        // the trail, not in use yet, hold its counters
-        uint32_t *off = (uint32_t *)alloc(((size_t)2 * D.nv + 1) * 4), *rows = (uint32_t *)alloc((size_t)row_words(D) * 4);
-        Occurrence *occ = (Occurrence *)alloc((size_t)bucket_lits * sizeof(Occurrence));
-        if (rc == ASP_OK) {
-            D.occ_off = off;
-            D.occ = occ;
-            D.rows = rows;
-            cudaError_t e = launch_occurrences(D, (uint32_t)bucket_lits, off, occ, rows, (uint32_t *)D.deps, D.trail, p->stream);
-            if (e != cudaSuccess) rc = cuda_fail(e, "occurrence lists");
-        }
-    }
     if (rc == ASP_OK) rc = plan_grid(p, H);
     if (rc == ASP_OK) rc = plan_batch(p, H, 0);
     if (rc == ASP_OK) rc = plan_batch(p, H, 1);
+    if (rc == ASP_OK && D.nv > 0) {
+        // occurrence lists by literal, after everything that a search cannot do
+        // without: they take eight times the store's memory, and a program
+        // without them is propagated by sweeps.  Built on the device; the
+        // bitmaps and the trail, not in use yet, hold its counters
+        uint32_t *off = (uint32_t *)dalloc(p, ((size_t)2 * D.nv + 1) * 4);
+        uint32_t *rows = off ? (uint32_t *)dalloc(p, (size_t)row_words(D) * 4) : nullptr;
+        Occurrence *occ = rows ? (Occurrence *)dalloc(p, (size_t)bucket_lits * sizeof(Occurrence)) : nullptr;
+        if (occ) {
+            cudaError_t e = launch_occurrences(D, (uint32_t)bucket_lits, off, occ, rows, (uint32_t *)D.deps, D.trail, p->stream);
+            if (e != cudaSuccess) rc = cuda_fail(e, "occurrence lists");
+        } else {
+            dfree_last(p, rows);
+            dfree_last(p, off);
+        }
+        for (Dev *d : {&p->D, &p->D1[0], &p->D1[1]}) {
+            d->occ_off = occ ? off : nullptr;
+            d->occ = occ;
+            d->rows = rows;
+            if (!occ) d->narrow_max = d->list_max = d->lists = 0u;
+        }
+    }
     if (rc == ASP_OK) {
         // a cleared state, so that a sweep or the statistics before the first
         // solve read no left-over memory (a sweep timed on left-over codes took
@@ -1067,8 +1085,11 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
     b->max_models_each = max_models_each;
     b->caps.resize(n);
     for (int32_t i = 0; i < n; i++) b->caps[i] = models_cap ? models_cap[i] : 0;
-    // an explicit configuration follows the occurrence lists; the autotuner
-    // tries the sweeps too
+    // an explicit configuration follows the occurrence lists, unless some program
+    // has none; the autotuner tries the sweeps too
+    bool have_lists = true;
+    for (int32_t i = 0; i < n; i++) have_lists = have_lists && progs[i]->D.narrow_max != 0u;
+    b->lists = have_lists;
     auto bail = [&](int rc) { asp_batch_free(b); return rc; };
     // model buffers of every program
     for (int32_t i = 0; i < n; i++) {
@@ -1118,7 +1139,7 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
         double best = -1.0;
         bool best_lists = true;
         b->wide = n <= progs[0]->n_sms;
-        for (int u = 0; u < 2; u++) {
+        for (int u = 0; u < (have_lists ? 2 : 1); u++) {
             b->lists = u == 1;
             for (int c = 0; c < 2; c++) {
                 const double t = batch_trial(b, c, sample);

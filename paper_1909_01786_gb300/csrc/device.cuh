@@ -194,6 +194,8 @@ struct Dev {
     // lists: one CTA solves the program, and its bucket nogoods are checked
     // through the lists only: no sweep, no view
     // code_cache: narrow rounds work on a copy of the codes in shared memory
+    // A program whose lists did not fit has narrow_max = 0 and occ_off = null:
+    // every round is a sweep.
     uint32_t narrow_max, list_max, lists, code_cache;
     // frontier propagation (Algorithm 2's idea; any value but 0): once the
     // claims of a round are followed through the lists the static buckets are

@@ -243,6 +243,49 @@ __device__ __forceinline__ void na_sweep(const Dev &D, uint32_t *asg, NaCtl *c, 
     }
 }
 
+// The unit nogoods.
+__device__ __forceinline__ void na_units(const Dev &D, uint32_t *asg, NaCtl *c, uint32_t gt, uint32_t nth, uint32_t fresh,
+                                         const NaList &O)
+{
+    for (uint32_t i = gt; i < D.n_units; i += nth) {
+        const uint32_t l = __ldg(D.lits + D.units_base + i) & ~END_BIT;
+        const uint32_t v = na_val(asg, l >> 1, fresh);
+        if (v == 0u) na_claim(asg, c, l, fresh, O);
+        else if (v == ((l & 1u) ? V_F : V_T)) na_conflict(c, O);
+    }
+}
+
+// Long nogoods: one warp per nogood, lanes over literals.
+__device__ __forceinline__ void na_long(const Dev &D, uint32_t *asg, NaCtl *c, uint32_t gw, uint32_t nw, uint32_t fresh, const NaList &O)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    for (uint32_t i = gw; i < D.n_long; i += nw) {
+        __syncwarp();
+        const uint32_t id = __ldg(D.long_ids + i);
+        bool sat = false;
+        uint32_t n_un = 0, ul = 0;
+        for (uint32_t off = id;; off += 32u) {
+            const uint32_t w = __ldg(D.lits + off + lane);
+            const unsigned Bend = __ballot_sync(0xFFFFFFFFu, (w & END_BIT) != 0u);
+            const unsigned valid = Bend ? ((2u << (__ffs(Bend) - 1)) - 1u) : 0xFFFFFFFFu;
+            const uint32_t l = w & ~END_BIT;
+            const bool mine = (valid >> lane) & 1u;
+            const uint32_t v = mine ? na_val(asg, l >> 1, fresh) : 0u;
+            const unsigned Bopp = __ballot_sync(0xFFFFFFFFu, mine && v == ((l & 1u) ? V_T : V_F));
+            const unsigned Bun = __ballot_sync(0xFFFFFFFFu, mine && v == 0u);
+            const uint32_t first = __shfl_sync(0xFFFFFFFFu, l, Bun ? __ffs(Bun) - 1 : 0);
+            if (Bun && n_un == 0) ul = first;
+            n_un += (uint32_t)__popc(Bun);
+            if (Bopp) { sat = true; break; }
+            if (Bend || n_un > 1u) break;
+        }
+        if (lane == 0 && !sat) {
+            if (n_un == 0u) na_conflict(c, O);
+            else if (n_un == 1u) na_claim(asg, c, ul, fresh, O);
+        }
+    }
+}
+
 // The fixpoint by following assignments: a round checks the nogoods of the
 // literals listed by the round before (first the caller's assignment), found
 // through the occurrence lists, instead of every nogood of the store; with at
@@ -295,45 +338,32 @@ __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D,
     // r: rounds so far (its parity names the fresh bit), k: the grid's rounds;
     // the first also applies the unit nogoods
     uint32_t r = 0, k = 0, stop = 0;
+    if (D.narrow_max == 0u) {
+        // no lists: every round reads the whole store
+        for (; ok; k++, r++) {
+            const uint32_t fresh = 4u << (r & 1u), slot = k % 3u;
+            if (gt == 0) c->nclaim[(k + 1u) % 3u] = c->stop[(k + 1u) % 3u] = 0u;
+            O = NaList{list, to, &c->nclaim[slot], s_lit[0], &s_n[0], &c->stop[slot]};
+            if (k == 0) na_units(D, asg, c, gt, nth, fresh, O);
+            na_sweep(D, asg, c, list + from, to - from, gt, nth, fresh, 4u << ((r + 1u) & 1u), O);
+            na_long(D, asg, c, gw, nw, fresh, O);
+            na_flush(O);
+            if (!(ok = na_sync(c, gen++))) break;
+            const uint32_t n = __ldcg(&c->nclaim[slot]);
+            if (__ldcg(&c->stop[slot]) || n == 0u) break;
+            from = to;
+            to += n;
+        }
+        goto done;
+    }
 follow:
     for (; ok; k++) {
         const uint32_t fresh = 4u << (r & 1u), stale = 4u << ((r + 1u) & 1u), slot = k % 3u;
         if (gt == 0) c->nclaim[(k + 1u) % 3u] = c->stop[(k + 1u) % 3u] = 0u;
         O = NaList{list, to, &c->nclaim[slot], s_lit[0], &s_n[0], &c->stop[slot]};
-        if (k == 0)
-            for (uint32_t i = gt; i < D.n_units; i += nth) {
-                const uint32_t l = __ldg(D.lits + D.units_base + i) & ~END_BIT;
-                const uint32_t v = na_val(asg, l >> 1, fresh);
-                if (v == 0u) na_claim(asg, c, l, fresh, O);
-                else if (v == ((l & 1u) ? V_F : V_T)) na_conflict(c, O);
-            }
+        if (k == 0) na_units(D, asg, c, gt, nth, fresh, O);
         na_follow<false>(D, asg, c, list + from, to - from, gw, nw, fresh, stale, longest, O);
-        // long nogoods: one warp per nogood, lanes over literals
-        for (uint32_t i = gw; i < D.n_long; i += nw) {
-            __syncwarp();
-            const uint32_t id = __ldg(D.long_ids + i);
-            bool sat = false;
-            uint32_t n_un = 0, ul = 0;
-            for (uint32_t off = id;; off += 32u) {
-                const uint32_t w = __ldg(D.lits + off + lane);
-                const unsigned Bend = __ballot_sync(0xFFFFFFFFu, (w & END_BIT) != 0u);
-                const unsigned valid = Bend ? ((2u << (__ffs(Bend) - 1)) - 1u) : 0xFFFFFFFFu;
-                const uint32_t l = w & ~END_BIT;
-                const bool mine = (valid >> lane) & 1u;
-                const uint32_t v = mine ? na_val(asg, l >> 1, fresh) : 0u;
-                const unsigned Bopp = __ballot_sync(0xFFFFFFFFu, mine && v == ((l & 1u) ? V_T : V_F));
-                const unsigned Bun = __ballot_sync(0xFFFFFFFFu, mine && v == 0u);
-                const uint32_t first = __shfl_sync(0xFFFFFFFFu, l, Bun ? __ffs(Bun) - 1 : 0);
-                if (Bun && n_un == 0) ul = first;
-                n_un += (uint32_t)__popc(Bun);
-                if (Bopp) { sat = true; break; }
-                if (Bend || n_un > 1u) break;
-            }
-            if (lane == 0 && !sat) {
-                if (n_un == 0u) na_conflict(c, O);
-                else if (n_un == 1u) na_claim(asg, c, ul, fresh, O);
-            }
-        }
+        na_long(D, asg, c, gw, nw, fresh, O);
         na_flush(O);
         if (!(ok = na_sync(c, gen++))) break;
         // every thread sees the same counters after the barrier
@@ -402,6 +432,7 @@ follow:
             if (!stop) goto follow;
         }
     }
+done:
     if (!ok && !gt) *conflict_out = -1;
     if (!ok) return;
     for (uint32_t w = gt; w < words; w += nth) {

@@ -2663,10 +2663,13 @@ __device__ __forceinline__ void solver_loop(const Dev &D, const Smem &S, const V
             __shared__ NarrowQueue<QN, 4u * QN> Q;
             cta_sync();
             uint32_t n = 0, left = 0, leave = 0;
-            const uint32_t its = D.code_cache
+            // without lists (only decisions come here then) it is left to a sweep
+            uint32_t its = 0;
+            if (D.narrow_max == 0u) { left = sw_fr1 - sw_fr0; leave = LEAVE_LONG + 1u; }
+            else its = D.code_cache
                 ? narrow_rounds<true>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left, &leave)
                 : narrow_rounds<false>(D, S.codes, Q, acc, sw_cdl, C.round, sw_fr0, sw_fr1, sw_tbase, &n, &left, &leave);
-            if (leave > LEAVE_LONG && D.G == 1u) {
+            if (leave > LEAVE_LONG && D.G == 1u && its) {
                 SweepCtx X{&D, V, 4u << ((C.round + its - 1u) & 1u), sw_cdl, sw_tbase + n, acc, true, false, cta, rank >> 5, size >> 5};
                 long_lists(X, Q.lng, leave - LEAVE_LONG);
                 cta_sync();

@@ -1,0 +1,125 @@
+"""Programs and batches where device memory is short (needs a GB300): a program
+whose occurrence lists cannot be allocated is propagated by sweeps."""
+import numpy as np
+import pytest
+
+import oracle
+from synth.programs import coloring_program, program_seed, random_program, tiny_program
+
+from test_gpu_fwd_learning import _check_at_conflict, _completion
+from test_gpu_lists import _noalloc, _perm
+
+pytestmark = pytest.mark.gpu
+
+ASP_E_OOM = -3
+
+
+@pytest.fixture(scope="module")
+def env():
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_1909_01786_gb300 import aspgpu
+    aspgpu.lib()
+    return torch, aspgpu
+
+
+def _schedule(gpu, programs):
+    plan = gpu.BatchPlan(programs, config=0)
+    out = plan.info()["frontier"]
+    plan.close()
+    return out
+
+
+def _without_lists(gpu, prog, which=0, **options):
+    """The program loaded while one of the allocations fails that a load
+    survives (the first such, or the `which`-th after it)."""
+    L = gpu.lib()
+    try:
+        for nth in range(1, 64):
+            assert L.asp_debug_fail_alloc(nth) == 0
+            try:
+                P = gpu.Program(prog, **options)
+            except gpu.AspError as e:
+                assert e.code == ASP_E_OOM
+                continue
+            break
+        if which:
+            assert L.asp_debug_fail_alloc(nth + which) == 0
+            P = gpu.Program(prog, **options)
+    finally:
+        L.asp_debug_fail_alloc(0)
+    return P
+
+
+@pytest.mark.parametrize("which", [0, 1, 2])
+def test_any_of_the_lists_allocations_may_fail(env, which):
+    _, gpu = env
+    prog = random_program(60, 120, program_seed(1301, 0))
+    assert _schedule(gpu, [gpu.Program(prog)]) == "units"
+    P = _without_lists(gpu, prog, which)
+    assert _schedule(gpu, [P]) == "full"
+    assert _schedule(gpu, [gpu.Program(prog), P]) == "full"
+
+
+# one CTA (with nogoods of more than 15 literals), a grid
+@pytest.mark.parametrize("atoms,rules", [(40, 70), (100, 2000), (5000, 20000)])
+@pytest.mark.parametrize("frontier", [0, 2])
+def test_closures_without_lists(env, atoms, rules, frontier):
+    torch, gpu = env
+    prog = random_program(atoms, rules, program_seed(1302, atoms))
+    P = _without_lists(gpu, prog, frontier=frontier)
+    perm = _perm(prog)
+    rng = np.random.default_rng(atoms)
+    agreed = 0
+    for k in (0, 1, 2, 3, 5, atoms // 4):
+        partial = np.zeros(P.n_vars, np.int8)
+        pick = rng.choice(atoms, size=k, replace=False)
+        partial[pick] = rng.choice([-1, 1], size=k)
+        opart = np.zeros(P.n_vars, np.int8)
+        opart[perm] = partial
+        want_conflict, want, _, _ = oracle.up_closure(prog, opart)
+        conflict, got = P.propagate(partial)
+        nconflict, ngot = _noalloc(torch, P, partial, k % 8)
+        assert conflict == nconflict == bool(want_conflict)
+        if not want_conflict:
+            agreed += 1
+            assert (got == want[perm]).all() and (ngot == want[perm]).all()
+    assert agreed
+
+
+@pytest.mark.parametrize("options", [dict(), dict(frontier=2), dict(learning=1, frontier=2), dict(grid_ctas=5), dict(grid_ctas=5, learning=1)])
+def test_answer_sets_without_lists(env, options):
+    _, gpu = env
+    for prog in [tiny_program(i) for i in (3, 77, 151, 402)] + [coloring_program(20, 4.0, seed_index=1)]:
+        _, want, n = gpu.Program(prog).solve(0, cap=1 << 12)
+        assert all(oracle.is_answer_set(prog, m) for m in want[:50])
+        status, models, k = _without_lists(gpu, prog, **options).solve(0, cap=1 << 12)
+        assert k == n and status == (gpu.SAT if n else gpu.UNSAT)
+        assert {bytes(m) for m in models} == {bytes(m) for m in want}
+
+
+@pytest.mark.parametrize("grid", [1, 0])
+@pytest.mark.parametrize("k", [1, 9])
+def test_learning_without_lists(env, grid, k):
+    _, gpu = env
+    prog = random_program(2000, 5000, program_seed(705, 2))
+    P = _without_lists(gpu, prog, grid_ctas=grid, conflict_budget=k)
+    status, _, _ = P.solve(1, cap=1)
+    assert status == gpu.UNKNOWN and P.stats()["conflicts"] == k
+    compared, reasons = _check_at_conflict(gpu, P, prog, _completion(prog), 0)
+    assert compared > 0 and reasons > 0
+
+
+@pytest.mark.parametrize("config", [-1, 0, 1])
+def test_batches_with_some_lists_missing(env, config):
+    _, gpu = env
+    progs = [tiny_program(i) for i in range(12)] + [random_program(200, 400, program_seed(1303, i)) for i in range(4)]
+    P = [gpu.Program(p) if i % 2 else _without_lists(gpu, p) for i, p in enumerate(progs)]
+    plan = gpu.BatchPlan(P, max_models_each=0, cap_each=1 << 12, config=config)
+    assert plan.info()["frontier"] == "full"
+    st, nm, models = plan.run()
+    for i, p in enumerate(progs):
+        s, want, n = gpu.Program(p).solve(0, cap=1 << 12)
+        assert (st[i], nm[i]) == (s, n) and n <= 1 << 12
+        assert {bytes(m) for m in models[i]} == {bytes(m) for m in want}
