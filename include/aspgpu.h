@@ -135,7 +135,7 @@ typedef struct {
     int32_t grid_ctas;        /* CTAs of the persistent solver grid; 0 = one per SM */
     int32_t block_threads;    /* threads per CTA (multiple of 32, <= 768); 0 = 768 */
     void *cuda_stream;        /* cudaStream_t for all work of this program; NULL = default */
-    /* device memory hooks (16-byte aligned memory); both NULL = cudaMalloc/cudaFree */
+    /* device memory hooks (memory aligned to 8 bytes); both NULL = cudaMalloc/cudaFree */
     void *(*dev_alloc)(size_t bytes, void *ctx);
     void (*dev_free)(void *ptr, size_t bytes, void *ctx);
     void *alloc_ctx;

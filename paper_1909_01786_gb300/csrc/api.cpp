@@ -676,7 +676,9 @@ int asp_load_ground(int32_t n_atoms, int32_t n_rules, const int32_t *head,
         // bitmaps and the trail, not in use yet, hold its counters
         uint32_t *off = (uint32_t *)dalloc(p, ((size_t)2 * D.nv + 1) * 4);
         uint32_t *rows = off ? (uint32_t *)dalloc(p, (size_t)row_words(D) * 4) : nullptr;
-        Occurrence *occ = rows ? (Occurrence *)dalloc(p, (size_t)bucket_lits * sizeof(Occurrence)) : nullptr;
+        // entries start on a 16-byte boundary, whatever the caller's allocator gives
+        uint8_t *raw = rows ? (uint8_t *)dalloc(p, (size_t)bucket_lits * sizeof(Occurrence) + 16) : nullptr;
+        Occurrence *occ = raw ? (Occurrence *)(((uintptr_t)raw + 15u) & ~(uintptr_t)15u) : nullptr;
         if (occ) {
             cudaError_t e = launch_occurrences(D, (uint32_t)bucket_lits, off, occ, rows, (uint32_t *)D.deps, D.trail, p->stream);
             if (e != cudaSuccess) rc = cuda_fail(e, "occurrence lists");

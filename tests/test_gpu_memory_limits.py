@@ -1,5 +1,6 @@
-"""Programs and batches where device memory is short (needs a GB300): a program
-whose occurrence lists cannot be allocated is propagated by sweeps."""
+"""The caller's device memory (needs a GB300): a program whose occurrence lists
+cannot be allocated is propagated by sweeps; memory need be aligned to 8 bytes
+only."""
 import numpy as np
 import pytest
 
@@ -123,3 +124,45 @@ def test_batches_with_some_lists_missing(env, config):
         s, want, n = gpu.Program(p).solve(0, cap=1 << 12)
         assert (st[i], nm[i]) == (s, n) and n <= 1 << 12
         assert {bytes(m) for m in models[i]} == {bytes(m) for m in want}
+
+
+def _allocator(gpu, monkeypatch, allow=lambda n: True, shift=0):
+    """Program loads take their memory `shift` bytes past what PyTorch gives,
+    where allow(bytes) says so, else none."""
+    class Hooks(gpu._TorchAllocator):
+        def __init__(self, torch, device, stream):
+            def alloc(n, ctx):
+                if not allow(n):
+                    return None
+                return torch.cuda.caching_allocator_alloc(int(n) + shift, device=device, stream=stream) + shift
+
+            def free(p, n, ctx):
+                torch.cuda.caching_allocator_delete(p - shift)
+
+            self.c_alloc, self.c_free = gpu._ALLOC(alloc), gpu._FREE(free)
+
+    monkeypatch.setattr(gpu, "_TorchAllocator", Hooks)
+
+
+@pytest.mark.parametrize("atoms,rules", [(40, 70), (100, 2000), (5000, 20000)])
+def test_memory_aligned_to_eight_bytes(env, monkeypatch, atoms, rules):
+    torch, gpu = env
+    prog = random_program(atoms, rules, program_seed(1304, atoms))
+    Q = gpu.Program(prog, conflict_budget=20)
+    _allocator(gpu, monkeypatch, shift=8)
+    P = gpu.Program(prog, conflict_budget=20)
+    partial = np.zeros(P.n_vars, np.int8)
+    partial[:2] = -1
+    want_conflict, want = Q.propagate(partial)
+    conflict, got = P.propagate(partial)
+    nconflict, ngot = _noalloc(torch, P, partial, 0)
+    assert conflict == nconflict == want_conflict
+    if not conflict:
+        assert (got == want).all() and (ngot == want).all()
+    status, models, _ = P.solve(1, cap=1)
+    plan = gpu.BatchPlan([P], config=0)
+    st, nm, rows = plan.run()
+    for s, ms in ((status, models), (st[0], rows[0])):
+        assert s in (gpu.SAT, gpu.UNSAT, gpu.UNKNOWN)
+        assert all(oracle.is_answer_set(prog, m) for m in ms)
+    assert Q.solve(1, cap=1)[0] in (status, gpu.UNKNOWN) or status == gpu.UNKNOWN
