@@ -74,9 +74,6 @@ struct asp_prog {
     unsigned long long *d_models = nullptr;
     int64_t d_models_rows = 0;
     Acc *d_sweep_acc = nullptr;
-    // asp_debug_propagate, allocated by its first call: the input's and the
-    // closure's bytes (8 x asg_words), then the counts of launch_input
-    int8_t *d_io = nullptr;
 };
 
 namespace aspgpu {
@@ -845,18 +842,18 @@ int asp_debug_propagate(asp_prog *p, const int8_t *partial, int8_t *closure, int
     g_err.clear();
     if (!p || !partial || !closure) return fail(ASP_E_ARG, "bad argument");
     const Dev &D = p->D;
+    // the input's and the closure's bytes (8 x asg_words), then the counts of
+    // launch_input, lie in the dependency bitmaps (8 bytes a variable at least),
+    // which nothing reads at the root level
+    int8_t *const d_io = reinterpret_cast<int8_t *>(D.deps);
     const size_t io = (size_t)D.asg_words * 8;
-    if (!p->d_io) {
-        p->d_io = (int8_t *)dalloc(p, io + 4 * (size_t)input_blocks(D));
-        if (!p->d_io) return fail(ASP_E_OOM, "device allocation failed (partial assignment)");
-    }
     // codes, levels, reasons and trail are made on the device from one byte a
     // variable (for 5.2M variables, 16 ms of host loops and 47 MB of copies
     // were two thirds of the call)
     cudaStream_t st = p->stream;
     set_launch(p, MODE_PROPAGATE, 0, 0, nullptr, p->d_result);
-    cudaError_t e = cudaMemcpyAsync(p->d_io, partial, D.nv, cudaMemcpyHostToDevice, st);
-    if (e == cudaSuccess) e = launch_input(D, p->d_io, reinterpret_cast<uint32_t *>(p->d_io + io), st);
+    cudaError_t e = cudaMemcpyAsync(d_io, partial, D.nv, cudaMemcpyHostToDevice, st);
+    if (e == cudaSuccess) e = launch_input(D, d_io, reinterpret_cast<uint32_t *>(d_io + io), st);
     if (e != cudaSuccess) return cuda_fail(e, "upload partial");
     long long res[4] = {0, 0, 0, 0};
     if (p->empty_nogood) {
@@ -865,8 +862,8 @@ int asp_debug_propagate(asp_prog *p, const int8_t *partial, int8_t *closure, int
         e = launch_solve(p->D, p->grid, p->block, p->smem, st);
         if (e != cudaSuccess) return cuda_fail(e, "launch");
     }
-    e = launch_closure(D, p->d_io, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(closure, p->d_io, D.nv, cudaMemcpyDeviceToHost, st);
+    e = launch_closure(D, d_io, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(closure, d_io, D.nv, cudaMemcpyDeviceToHost, st);
     if (e != cudaSuccess) return cuda_fail(e, "download closure");
     if (!p->empty_nogood) {
         const int rc = finish(p, res);

@@ -1,11 +1,11 @@
 """The caller's device memory (needs a GB300): a program whose occurrence lists
 cannot be allocated is propagated by sweeps; memory need be aligned to 8 bytes
-only."""
+only; propagation allocates nothing."""
 import numpy as np
 import pytest
 
 import oracle
-from synth.programs import coloring_program, program_seed, random_program, tiny_program
+from synth.programs import coloring_program, from_rules, program_seed, random_program, tiny_program
 
 from test_gpu_fwd_learning import _check_at_conflict, _completion
 from test_gpu_lists import _noalloc, _perm
@@ -166,3 +166,24 @@ def test_memory_aligned_to_eight_bytes(env, monkeypatch, atoms, rules):
         assert s in (gpu.SAT, gpu.UNSAT, gpu.UNKNOWN)
         assert all(oracle.is_answer_set(prog, m) for m in ms)
     assert Q.solve(1, cap=1)[0] in (status, gpu.UNKNOWN) or status == gpu.UNKNOWN
+
+
+@pytest.mark.parametrize("prog", [from_rules(1, []), from_rules(1, [(0, [], [])]), from_rules(2, [(0, [], [1]), (1, [], [0])]),
+                                  random_program(40, 70, program_seed(1305, 0)), random_program(5000, 20000, program_seed(1305, 1))],
+                         ids=lambda prog: f"{prog.n_atoms}-{prog.n_rules}")
+def test_propagation_allocates_nothing(env, monkeypatch, prog):
+    _, gpu = env
+    left = [True]
+    _allocator(gpu, monkeypatch, allow=lambda n: left[0])
+    P = gpu.Program(prog)
+    left[0] = False
+    partial = np.zeros(P.n_vars, np.int8)
+    partial[0] = -1
+    opart = np.zeros(P.n_vars, np.int8)
+    opart[_perm(prog)] = partial
+    want_conflict, want, _, _ = oracle.up_closure(prog, opart)
+    for _ in range(2):
+        conflict, got = P.propagate(partial)
+        assert conflict == bool(want_conflict)
+        if not conflict:
+            assert (got == want[_perm(prog)]).all()
