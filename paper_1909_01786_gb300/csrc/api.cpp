@@ -1112,12 +1112,16 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
     }
     asp_prog *p0 = progs[0];
     // room for every program's models, up to 64 MB (what does not fit is copied
-    // program by program)
+    // program by program, as is everything where that room cannot be had)
     for (int32_t i = 0; i < n; i++) b->packed += std::min<int64_t>(b->caps[i] * (((int64_t)progs[i]->D.na + 63) / 64), 1ll << 40);
     b->packed = std::min<int64_t>(b->packed, 8ll << 20);
-    b->scratch_bytes = b->bytes();
-    if (p0->opt.dev_alloc) b->scratch = p0->opt.dev_alloc(b->scratch_bytes, p0->opt.alloc_ctx);
-    else if (cudaMalloc(&b->scratch, b->scratch_bytes) != cudaSuccess) { cudaGetLastError(); b->scratch = nullptr; }
+    for (;;) {
+        b->scratch_bytes = b->bytes();
+        if (p0->opt.dev_alloc) b->scratch = p0->opt.dev_alloc(b->scratch_bytes, p0->opt.alloc_ctx);
+        else if (cudaMalloc(&b->scratch, b->scratch_bytes) != cudaSuccess) { cudaGetLastError(); b->scratch = nullptr; }
+        if (b->scratch || b->packed == 0) break;
+        b->packed = 0;
+    }
     if (!b->scratch) return bail(fail(ASP_E_OOM, "device allocation failed (batch descriptors)"));
     // queue order: largest store first
     std::vector<uint32_t> order(n);

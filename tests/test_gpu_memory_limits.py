@@ -1,6 +1,7 @@
 """The caller's device memory (needs a GB300): a program whose occurrence lists
 cannot be allocated is propagated by sweeps; memory need be aligned to 8 bytes
-only; propagation allocates nothing."""
+only; propagation allocates nothing; a batch without room for every model copies
+them program by program."""
 import numpy as np
 import pytest
 
@@ -187,3 +188,29 @@ def test_propagation_allocates_nothing(env, monkeypatch, prog):
         assert conflict == bool(want_conflict)
         if not conflict:
             assert (got == want[_perm(prog)]).all()
+
+
+def _batch_in_little_memory(gpu, monkeypatch, progs, cap):
+    """The batch's plan where no block of 100 kB or more can be had."""
+    small = [False]
+    _allocator(gpu, monkeypatch, allow=lambda n: n < 100_000 or not small[0])
+    P = [gpu.Program(p) for p in progs]
+    small[0] = True
+    return P, gpu.BatchPlan(P, max_models_each=0, cap_each=cap, config=0)
+
+
+def _check_batch(gpu, progs, plan, cap):
+    st, nm, models = plan.run()
+    for i, p in enumerate(progs):
+        s, want, n = gpu.Program(p, torch_memory=False).solve(0, cap=cap)
+        assert (st[i], nm[i]) == (s, n) and n <= cap
+        assert {bytes(m) for m in models[i]} == {bytes(m) for m in want}
+
+
+def test_batch_without_room_for_its_models(env, monkeypatch):
+    """Room for 12 x 2048 rows would be 197 kB."""
+    _, gpu = env
+    progs = [tiny_program(i) for i in (3, 77, 151, 402, 555, 918)] + [tiny_program(i) for i in range(5, 11)]
+    _, plan = _batch_in_little_memory(gpu, monkeypatch, progs, 2048)
+    for _ in range(2):
+        _check_batch(gpu, progs, plan, 2048)
