@@ -340,6 +340,8 @@ static int plan_batch(asp_prog *p, const HostStore &H, int config)
 // + batch kernel) captured in a CUDA graph.
 struct asp_batch {
     std::vector<asp_prog *> progs;
+    std::vector<unsigned long long *> rows;   // the model buffers that the launch writes (a program's
+                                              // own later solve may take a larger one)
     std::vector<int64_t> caps;
     int64_t max_models_each = 0;
     int config = 0, kernel = 0, grid = 0;   // kernel: configuration of the instantiation in use
@@ -392,7 +394,7 @@ std::vector<Dev> batch_descriptors(const asp_batch *b, int config, bool trial = 
         d.mode = MODE_SOLVE;
         d.max_models = b->max_models_each;
         d.models_cap = b->caps[i];
-        d.models = p->d_models;
+        d.models = b->rows[i];
         d.result = b->results() + 4 * i;
         d.conflict_budget = p->opt.conflict_budget;
         d.time_budget_ns = p->opt.time_budget_ms > 0 ? p->opt.time_budget_ms * 1000000ll : 0;
@@ -1101,6 +1103,7 @@ int asp_batch_create(int32_t n, asp_prog *const *progs, int64_t max_models_each,
             p->d_models = (unsigned long long *)q;
             p->d_models_rows = rows;
         }
+        b->rows.push_back(p->d_models);
     }
     // a stream that can be captured (the legacy default stream cannot)
     b->stream = progs[0]->stream;
@@ -1208,7 +1211,7 @@ int asp_batch_run(asp_batch *b, int32_t *statuses, int64_t *n_models, uint64_t *
         if (place[i] >= 0) {
             std::memcpy(models[i], rows.data() + place[i], (size_t)words * 8);
         } else {
-            e = cudaMemcpy(models[i], b->progs[i]->d_models, (size_t)words * 8, cudaMemcpyDeviceToHost);
+            e = cudaMemcpy(models[i], b->rows[i], (size_t)words * 8, cudaMemcpyDeviceToHost);
             if (e != cudaSuccess) return cuda_fail(e, "batch models");
         }
     }

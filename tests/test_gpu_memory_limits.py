@@ -199,6 +199,11 @@ def _batch_in_little_memory(gpu, monkeypatch, progs, cap):
     return P, gpu.BatchPlan(P, max_models_each=0, cap_each=cap, config=0)
 
 
+def _choices(k):
+    """2^k answer sets"""
+    return from_rules(2 * k, [(a, [], [a ^ 1]) for a in range(2 * k)])
+
+
 def _check_batch(gpu, progs, plan, cap):
     st, nm, models = plan.run()
     for i, p in enumerate(progs):
@@ -214,3 +219,14 @@ def test_batch_without_room_for_its_models(env, monkeypatch):
     _, plan = _batch_in_little_memory(gpu, monkeypatch, progs, 2048)
     for _ in range(2):
         _check_batch(gpu, progs, plan, 2048)
+
+
+def test_batch_rows_after_a_larger_solve(env, monkeypatch):
+    """A solve with a larger cap takes another model buffer; the batch's rows
+    stay where its launch writes them."""
+    _, gpu = env
+    progs = [_choices(k) for k in range(12)]
+    P, plan = _batch_in_little_memory(gpu, monkeypatch, progs, 2048)
+    for p in P:
+        p.solve(1, cap=4096)
+    _check_batch(gpu, progs, plan, 2048)
