@@ -9,6 +9,7 @@ import oracle
 from synth.programs import from_rules
 
 from test_gpu_fwd_learning import _check_at_conflict, _completion
+from test_gpu_learning import _check_conflict
 from test_gpu_lists import _noalloc, _perm
 
 pytestmark = pytest.mark.gpu
@@ -73,15 +74,39 @@ def test_closures_with_hubs_equal_the_oracle(env, hubs, each, pool, filler, grid
 @pytest.mark.parametrize("hubs,each,pool,filler,grid", [(1, 1500, 500, 300, 0), (17, 260, 800, 0, 0), (1, 3000, 4000, 9000, 0),
                                                         (300, 60, 6000, 6000, 0), (300, 100, 3000, 3000, 2)])
 @pytest.mark.parametrize("k", [1, 5])
-def test_learning_with_hubs(env, hubs, each, pool, filler, grid, k):
+@pytest.mark.parametrize("learning", [0, 1])
+def test_learning_with_hubs(env, hubs, each, pool, filler, grid, k, learning):
     _, gpu = env
     prog = _hubs(hubs, each, pool, filler, k)
-    P = gpu.Program(prog, grid_ctas=grid, conflict_budget=k)
+    P = gpu.Program(prog, grid_ctas=grid, conflict_budget=k, learning=learning)
     status, _, _ = P.solve(1, cap=1)
     if status != gpu.UNKNOWN or P.stats()["conflicts"] != k:
         pytest.skip("search ended before the k-th conflict")
+    if learning:
+        _check_conflict(gpu, P)
+        return
     compared, reasons = _check_at_conflict(gpu, P, prog, _completion(prog), 0)
     assert compared > 0 and reasons > 0
+
+
+@pytest.mark.parametrize("learning", [0, 1])
+@pytest.mark.parametrize("k", [1, 4, 12])
+def test_list_rounds_by_lanes_above_the_root(env, learning, k):
+    """Deciding atom 0 claims the 300 hubs' bodies at once, more than one CTA
+    follows alone and few enough for lists; two CTAs of one warp each follow them
+    a lane per occurrence, and the lanes write the claims' bitmaps."""
+    _, gpu = env
+    prog = _hubs(300, 40, 1500, 1500, k)
+    P = gpu.Program(prog, grid_ctas=2, block_threads=32, conflict_budget=k, learning=learning)
+    status, _, _ = P.solve(1, cap=1)
+    s = P.stats()
+    if status != gpu.UNKNOWN or s["conflicts"] != k:
+        pytest.skip("search ended before the k-th conflict")
+    if learning:
+        _check_conflict(gpu, P)
+    else:
+        compared, reasons = _check_at_conflict(gpu, P, prog, _completion(prog), 0)
+        assert compared > 300 and reasons > 300
 
 
 def test_a_hub_costs_a_sweep_not_a_walk(env):
