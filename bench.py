@@ -700,6 +700,8 @@ def _summary(out):
         return round(d, 4) if isinstance(d, float) else d
     return {
         "checks_per_s": g(out, "value"), "frac_hbm": g(out, "roofline", "frac"),
+        # the search's own speed: checks/s falls when rounds need fewer checks
+        "ms_per_step": g(out, "ms_per_step"), "conflicts_per_s": g(out, "search", "conflicts_per_s"),
         "decisions_per_s": g(out, "search", "decisions_per_s"),
         "propagations_per_s": g(out, "search", "propagations_per_s"),
         "work_vs_oracle": out.get("work_vs_oracle"),

@@ -405,7 +405,8 @@ int asp_debug_barrier(asp_prog *p, int32_t stall_cta, int32_t wait_limit_ms);
 
 /* Test-only failure injection on the host: the nth device allocation the
  * library makes from now on (any program, any thread) fails as if the
- * allocator had no memory, so the call that needed it returns ASP_E_OOM.
+ * allocator had no memory, so the call that needed it returns ASP_E_OOM
+ * (a load goes on without its occurrence lists).
  * nth = 0 switches it off.  Errors: ASP_E_ARG. */
 int asp_debug_fail_alloc(int64_t nth);
 

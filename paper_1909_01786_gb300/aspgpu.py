@@ -193,7 +193,7 @@ class Program:
             opt.mlp_weights = w.ctypes.data
         opt.trace_capacity = int(trace_capacity)
         opt.view_mode = int(view_mode)
-        opt.frontier = int(frontier)         # False/True = full / nogood frontier; FRONTIER_UNITS
+        opt.frontier = int(frontier)         # FRONTIER_*: 0 = sweeps confirm the fixpoints
         opt.learning = int(learning)
         opt.backjump = int(backjump)
         opt.restart_conflicts = int(restart_conflicts)

@@ -13,7 +13,8 @@
 // CTA while they are few (narrow_rounds), the grid when they are more
 // (list_round).  Sweeps of the whole store run initial propagation, the round
 // after a backjump, rounds with very many claims, and the confirmation of a
-// full-sweep program's fixpoint.  One-CTA programs never sweep.
+// full-sweep program's fixpoint, and lists too long for a warp.  One-CTA programs
+// never sweep; programs whose lists did not fit in memory always do.
 //
 // Sweep design.  The static nogoods sit in one bucket per exact length
 // (Section 4: one kernel per length class), stored structure-of-arrays, and
@@ -741,8 +742,9 @@ __device__ __forceinline__ void run_unit(const SweepCtx &X, uint32_t L, uint32_t
 // the nogood is neither unit nor violated, and two checks settle it (the
 // caller's); otherwise this scan runs and moves the watches to literals that do
 // not hold (the complement found, or the first unassigned ones).  Every such
-// nogood is checked every round, so the watches need no per-variable lists and
-// stay valid across backjumps.  Equal positions (a nogood of one literal)
+// nogood is checked in list rounds and sweeps, and before each fixpoint (narrow
+// rounds check none), whatever was assigned, so the watches need no per-variable
+// lists and stay valid across backjumps.  Equal positions (a nogood of one literal)
 // always scan.
 __device__ __forceinline__ void classify_long(const SweepCtx &X, uint32_t id, unsigned long long &checks,
                                               uint2 *wslot, uint2 wp)
