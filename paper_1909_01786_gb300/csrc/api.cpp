@@ -210,8 +210,9 @@ static int choose_view(asp_prog *p, const HostStore &H, Dev &D, const std::vecto
     return ASP_OK;
 }
 
-// One CTA: lists from here on are shared out to its warps (a program of 64k
-// literals has few)
+// One CTA: longer lists are shared out to its warps.  Closure of 37k literals with
+// one list of 200, 400 and 800 occurrences, walked by a warp and shared out: 127
+// and 127 us, 116 and 116, 187 and 166
 constexpr uint32_t ONE_CTA_LONG_LIST = 256u;
 
 // Grid size, the static partition of the buckets over the CTAs along groups
@@ -250,10 +251,11 @@ static int plan_grid(asp_prog *p, const HostStore &H)
     D.list_max = (uint32_t)(total / 128u);
     D.lists = g == 1;
     if (D.lists) D.narrow_max = 0xFFFFFFFFu;
-    // A warp walks 32 occurrences in about 2 us and a sweep reads a warp's share
-    // of the store, four literals in the time of one of them, after a few us of
-    // its own: up to this length the list is the faster one
-    D.long_list = g == 1 ? ONE_CTA_LONG_LIST : 128u + (uint32_t)(total / (4u * (uint64_t)g * ((uint32_t)p->block / 32u)));
+    // What a warp walks in the time of a sweep, about 0.15 us an occurrence.
+    // Closure with one list of n occurrences, walked and with a sweep instead:
+    // 335k literals, n = 200 100 and 99 us, 800 125 and 108; 5.9M literals, 400 88
+    // and 87, 800 139 and 115; 21.9M literals, 400 157 and 158, 800 229 and 199
+    D.long_list = g == 1 ? ONE_CTA_LONG_LIST : 128u + (uint32_t)(total / (16u * (uint64_t)g * ((uint32_t)p->block / 32u)));
     // groups [glo[i], glo[i+1]) for CTA i, balanced by literal count
     const uint32_t ng = (uint32_t)H.n_groups;
     std::vector<uint32_t> glo(g + 1, ng);

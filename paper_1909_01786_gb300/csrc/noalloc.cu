@@ -167,8 +167,8 @@ __device__ __forceinline__ void na_claim(uint32_t *asg, NaCtl *c, uint32_t l, ui
 // chain; with more its lanes do, 32 literals at a time.  A literal's own fresh
 // bit, of the other parity, is cleared meanwhile.  SHARED: `from` is in shared
 // memory.  A warp whose lists hold more than `longest` occurrences passes them
-// over and stops the rounds for a sweep of the store (a literal of 160k nogoods
-// kept one warp busy for 10 ms).
+// over and stops the rounds for a sweep of the store (a literal of 130k nogoods
+// kept one warp busy for 26 ms).
 template <bool SHARED>
 __device__ __forceinline__ void na_follow(const Dev &D, uint32_t *asg, NaCtl *c, const uint32_t *from, uint32_t n, uint32_t w,
                                           uint32_t nw, uint32_t fresh, uint32_t stale, uint32_t longest, const NaList &O)
@@ -332,9 +332,11 @@ __global__ void __launch_bounds__(NA_THREADS, 1) noalloc_propagate_kernel(Dev D,
     uint32_t gen = 0, from = 0, to = 0;       // literals [from, to) are to be followed
     bool ok = na_sync(c, gen++);
     if (ok) to = __ldcg(&c->nclaim[2]);
-    // what a warp walks in the time of a sweep: a sweep reads a warp's share of
-    // the store four literals in the time of one occurrence, after a barrier
-    const uint32_t longest = 128u + (uint32_t)(D.static_checks / (4u * nw));
+    // what a warp walks in the time of a sweep.  A call with one list of n
+    // occurrences, walked and with a sweep instead: 335k literals, n = 100 74 and 66
+    // us, 200 114 and 109, 400 136 and 86; 5.9M literals, 200 92 and 89, 400 118
+    // and 84
+    const uint32_t longest = 128u + (uint32_t)(D.static_checks / (16u * nw));
     // r: rounds so far (its parity names the fresh bit), k: the grid's rounds;
     // the first also applies the unit nogoods
     uint32_t r = 0, k = 0, stop = 0;

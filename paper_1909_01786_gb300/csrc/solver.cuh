@@ -2006,9 +2006,12 @@ __device__ __forceinline__ void narrow_bitmaps(const Dev &D, const Queue &Q, uin
 // that follows costs a few us.
 constexpr uint32_t NARROW_ROUNDS = 1024u;
 
-// Occurrences of a round that one CTA of a grid follows (about 15 us), and why
-// it ends its phase: the next round has more of them, or (LEAVE_LONG + their
-// number) long lists were put off.
+// Occurrences of a round that one CTA of a grid follows, and why it ends its
+// phase: the next round has more of them, or (LEAVE_LONG + their number) long
+// lists were put off.  Closures with 960, 1920, 3840 and 7680 occurrences in one
+// round, by one CTA and by the grid: 122 and 130, 147 and 146, 167 and 155, 253
+// and 166 us (1.1M literals); 206 and 197, 244 and 198, 316 and 199, 388 and 215
+// (22M).  A round of narrow_max claims has about 1000.
 constexpr uint32_t NARROW_OCC = 2048u, LEAVE_WIDE = 1u, LEAVE_LONG = 2u;
 
 // Propagation by one CTA, following the claims instead of sweeping the store
@@ -2149,8 +2152,8 @@ __device__ __forceinline__ uint32_t narrow_rounds(const Dev &D, uint32_t *cache,
 // The lists that one CTA's narrow rounds put off, by all of its warps, as the
 // tail of the last round (X.fresh is that round's, so its claims stay unseen).
 // Apart from the rounds, whose every instruction counts: shared out there, the
-// lists cost 2 to 7 % of searches that have none.  A list of 1500 occurrences
-// kept its warp busy for 0.1 ms.
+// lists cost 2 to 7 % of searches that have none.  A closure with a list of 800
+// occurrences takes 166 us, and took 187 with one warp on it.
 __device__ __forceinline__ void long_lists(const SweepCtx &X, const uint4 *lists, uint32_t n)
 {
     const uint32_t nw = X.cdl > 1u ? deps_words(*X.D, X.cdl) : 0u;

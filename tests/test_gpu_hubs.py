@@ -41,7 +41,7 @@ def _hubs(hubs, each, pool, filler, seed):
 # the whole GPU).  A hub's list has a nogood more than its rules.
 CASES = [(1, 254, 300, 600, 0), (1, 255, 300, 600, 0), (1, 256, 300, 600, 0), (1, 1500, 500, 300, 0), (3, 500, 500, 200, 0),
          (16, 260, 800, 0, 0), (17, 260, 800, 0, 0), (40, 257, 900, 0, 1),
-         (1, 140, 4000, 9000, 0), (1, 3000, 4000, 9000, 0), (60, 100, 4000, 9000, 0), (300, 60, 6000, 6000, 0), (300, 200, 6000, 1000, 0),
+         (1, 125, 4000, 9000, 0), (1, 140, 4000, 9000, 0), (1, 3000, 4000, 9000, 0), (60, 100, 4000, 9000, 0), (300, 60, 6000, 6000, 0), (300, 200, 6000, 1000, 0),
          (20, 300, 3000, 3000, 2), (300, 100, 3000, 3000, 2)]
 
 
