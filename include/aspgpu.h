@@ -255,7 +255,8 @@ typedef struct asp_batch asp_batch;
  * kernel) in a CUDA graph.  Configurations: 0 = 256 threads per CTA, 3 CTAs
  * per SM; 1 = 128 threads, 6 per SM (twice the programs in flight, smaller
  * shared memory).  With an explicit configuration claims are followed through
- * the occurrence lists.  config = ASP_BATCH_AUTOTUNE tries every schedule --
+ * the occurrence lists, unless some program has none (see asp_load_ground): then
+ * the batch sweeps.  config = ASP_BATCH_AUTOTUNE tries every schedule --
  * each configuration with sweeps (and lists for few claims) and with lists
  * only -- once on a sample of up to 256 programs spread over the queue (each
  * with at most 8 conflicts and 0.5 s of device time), and keeps the one with
